@@ -359,7 +359,7 @@ __device__ __forceinline__ void batch_filter(const BatchArgs<R>& a, const BatchI
         if (full || base + 4 * q + e < n) {
           R ex;
           const R dl = v[e] - m;
-          wq = quant_exp<R>(dl, k, &ex);
+          wq = quant_exp(dl, k, &ex);
           epart = epart + ex;
           if (ess) sq = add128(sq, mul64(wq, wq));
         }
@@ -772,13 +772,13 @@ __device__ __forceinline__ void batch_filter(const BatchArgs<R>& a, const BatchI
       const R xa = cur.x, sa = cur.s2, ta = cur.t2;
       // V and mu share one correctly rounded reciprocal of s
       const R s = sa + ta;
-      const R ri = (R)1 / s;
+      const R ri = div_rn((R)1, s);
       const R p = sa * ta;
       const R V = p * ri;
       const R n2 = yr * ta;
       const R nn = fmaR(xa, sa, n2);
       const R mu = nn * ri;
-      const R sv = sqrt(V);
+      const R sv = sqrt_rn(V);
       R Z;
       theta_draws<R>(seed, fid, t, (uint32_t)j, &Z, &Zs, &Us, &Zt, &Ut);
       const R xj = fmaR(sv, Z, mu);
@@ -977,7 +977,7 @@ __device__ __forceinline__ void batch_estimate_weighted(const BatchArgs<R>& a,
       const uint64_t i = base + e;
       if (i < n) {
         R wr;
-        (void)quant_exp<R>(a.lam[off + i], k, &wr);
+        (void)quant_exp(a.lam[off + i], k, &wr);
         const double wd = (double)wr;
         const double dx = (double)(st.x[off + i] - c0), ds = (double)(st.s2[off + i] - c1),
                      dt = (double)(st.t2[off + i] - c2);

@@ -208,12 +208,12 @@ template <> struct SuffOps<float> {
 };
 template <> struct SuffOps<double> {
   static __device__ __forceinline__ double from_prior(double b) { return b; }
+  // b + r^2 / 2: the halving is exact, so it shares the addition's rounding
   static __device__ __forceinline__ double add_half_square(double b, double r, bool*) {
     const double r2 = r * r;
-    const double h = 0.5 * r2;
-    return b + h;
+    return __fma_rn(r2, 0.5, b);
   }
-  static __device__ __forceinline__ double ig(double b, double G) { return b / G; }
+  static __device__ __forceinline__ double ig(double b, double G) { return div_rn(b, G); }
 };
 
 // Constants of Marsaglia-Tsang for shape a, in binary64: d = a - 1/3,
@@ -293,10 +293,42 @@ __device__ __forceinline__ R log_pred(R x, R s2, R t2, R y) {
   const R dx = y - x;
   const R q = dx * dx;
   const R lg = det_log(s);
-  const R r = q / s;
+  const R r = div_rn(q, s);
   const R sum = lg + r;
   return (R)-0.5 * sum;
 }
+
+// Running maximum of log-likelihoods and whether one was NaN or +inf (such a
+// value is left out of the maximum; the cycle fails).  Binary64 keeps the
+// order-preserving signed integer of the value, so that neither the comparison
+// nor the check goes to the binary64 pipe.
+template <class R>
+struct MaxL {
+  float mx = -INFINITY;
+  bool bad = false;
+  __device__ __forceinline__ void take(float l) {
+    bad |= !(l < INFINITY);
+    mx = fmaxf(mx, l);
+  }
+  __device__ __forceinline__ float value() const { return mx; }
+};
+template <>
+struct MaxL<double> {
+  static constexpr long long NEG_INF = (long long)0x800FFFFFFFFFFFFFull;  // key of -inf
+  long long mx = NEG_INF;
+  bool bad = false;
+  static __device__ __forceinline__ long long key(long long b) { return b ^ (long long)((unsigned long long)(b >> 63) >> 1); }
+  __device__ __forceinline__ void take(double l) {
+    const long long b = __double_as_longlong(l);
+    // exponent field all ones: infinite or NaN; -inf is a weight of zero
+    const bool odd = (__double2hiint(l) & 0x7FF00000) == 0x7FF00000;
+    const long long v = key(b);
+    const bool wrong = odd && v != NEG_INF;
+    bad |= wrong;
+    if (!wrong && v > mx) mx = v;
+  }
+  __device__ __forceinline__ double value() const { return __longlong_as_double(key(mx)); }
+};
 
 __device__ __forceinline__ unsigned long long enc_max(float x) { return enc_f(x); }
 __device__ __forceinline__ unsigned long long enc_max(double x) { return enc_d(x); }
@@ -355,13 +387,11 @@ __global__ void __launch_bounds__(BLOCK, W_CTAS_PER_SM) k_weights(FilterArgs<R> 
   const int lane = threadIdx.x & 31;
   const uint64_t gw = (uint64_t)blockIdx.x * WARPS + (threadIdx.x >> 5);
   const uint64_t nw = (uint64_t)gridDim.x * WARPS;
-  R mx = (R)-INFINITY;
-  bool bad = false;
+  MaxL<R> top;
   auto weigh = [&](R x, R s2, R t2, R lam) {
     R l = log_pred<R>(x, s2, t2, yr);
     if constexpr (ESS) l = lam + l;
-    bad |= !(l < (R)INFINITY);  // NaN or +inf
-    mx = fmax(mx, l);
+    top.take(l);
     return l;
   };
   auto chunk = [&](uint64_t cb) {  // the warp's chunk of CHUNK particles from cb
@@ -411,8 +441,8 @@ __global__ void __launch_bounds__(BLOCK, W_CTAS_PER_SM) k_weights(FilterArgs<R> 
   } else {
     for (uint64_t cb = gw * CHUNK; cb < n; cb += nw * CHUNK) chunk(cb);
   }
-  if (bad) atomicOr(&a.ctl->err, ERR_NUMERIC);
-  mx = block_max<R>(mx, s_red);
+  if (top.bad) atomicOr(&a.ctl->err, ERR_NUMERIC);
+  const R mx = block_max<R>(top.value(), s_red);
   if (threadIdx.x == 0 && mx > (R)-INFINITY) atomicMax(&a.ctl->maxenc, enc_max(mx));
 }
 // CTAs of the weights kernel for n particles: the resident maximum `cap`, or
@@ -450,7 +480,7 @@ __global__ void __launch_bounds__(BLOCK) k_boot_pw(FilterArgs<R> a) {
   const uint64_t i = (uint64_t)blockIdx.x * BLOCK + threadIdx.x;
   if (i < a.n) {
     const R Z = bm_normal(draw(a.seed, a.filter, t, (uint32_t)i, P_BOOT_STATE, 0), (R)0);
-    const R sv = sqrt(st.t2[i]);
+    const R sv = sqrt_rn(st.t2[i]);
     const R xz = sv * Z;
     const R xp = st.x[i] + xz;
     st.x[i] = xp;
@@ -670,7 +700,7 @@ __global__ void __launch_bounds__(BLOCK, 4) k_scan(ScanArgs a) {
         if (MODE == FROM_LOGLIK) {
           R ex;
           const R dl = v[e] - m;
-          w = quant_exp<R>(dl, a.k, &ex);
+          w = quant_exp(dl, a.k, &ex);
           epart = epart + ex;
         } else {
           const float wf = (float)v[e];
@@ -1343,26 +1373,6 @@ __device__ __forceinline__ void bulk_wait_done() {
   asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
 
-// W = min(floor(e 2^k), 2^k) from e = exp(dl) as quant_exp returns it: e is
-// 0 or a normal number p 2^n, so e 2^k and p 2^(n + k) have the same bits
-// and the floor is the one quant_exp takes.
-__device__ __forceinline__ uint64_t quant_from_e(float e, int k) {
-  uint64_t W = 0;
-  if (e != 0.0f) {
-    const uint32_t eb = __float_as_uint(e);
-    const int sh = (int)(eb >> 23) - 150 + k;
-    const uint32_t m24 = (eb & 0x7fffffu) | 0x800000u;
-    W = sh >= 0 ? ((uint64_t)m24 << sh) : (uint64_t)(m24 >> (-sh < 31 ? -sh : 31));
-  }
-  const uint64_t cap = 1ull << k;
-  return W > cap ? cap : W;
-}
-__device__ __forceinline__ uint64_t quant_from_e(double e, int k) {
-  const uint64_t W = e != 0.0 ? f2u64_rz(e * pow2d(k)) : 0ull;
-  const uint64_t cap = 1ull << k;
-  return W > cap ? cap : W;
-}
-
 // The systematic resampling step writes each particle's slots into a
 // shared-memory window (an entry per slot of the tile, the particle's offset
 // in the tile + 1; the window starts at the tile's first slot rounded down to
@@ -1611,7 +1621,7 @@ __global__ void __launch_bounds__(BLOCK, PER == 8 ? 4 : 3) k_cdf_sys(FilterArgs<
             w = quant_from_e(ex, k);
           } else {
             const R dl = v[e] - m;
-            w = quant_exp<R>(dl, k, &ex);
+            w = quant_exp(dl, k, &ex);
           }
           ep = ep + ex;
           mx = ex > mx ? ex : mx;
@@ -2348,7 +2358,7 @@ __device__ __forceinline__ Gathered<R> gather_rec(const StateV<R>& src, uint32_t
 // new state back after the round's warp barrier.  Every value is the one the
 // weights kernel would give.
 template <class R, bool LEARN, bool FUSE = false, bool ESS = false>
-__global__ void __launch_bounds__(BLOCK, 5) k_propagate(FilterArgs<R> a) {
+__global__ void __launch_bounds__(BLOCK, 3) k_propagate(FilterArgs<R> a) {
   typedef GammaItem<R> Item;
   __shared__ Item s_q[WARPS][WQ_CAP];
   const Ctl* c = a.ctl;
@@ -2427,13 +2437,13 @@ __global__ void __launch_bounds__(BLOCK, 5) k_propagate(FilterArgs<R> a) {
       const R xa = cur.x, sa = cur.s2, ta = cur.t2;
       // V and mu share one correctly rounded reciprocal of s
       const R s = sa + ta;
-      const R ri = (R)1 / s;
+      const R ri = div_rn((R)1, s);
       const R p = sa * ta;
       const R V = p * ri;
       const R n2 = yr * ta;
       const R nn = fmaR(xa, sa, n2);
       const R mu = nn * ri;
-      const R sv = sqrt(V);
+      const R sv = sqrt_rn(V);
       R Z;
       theta_draws_rk<R>(a.rk, a.filter, t, (uint32_t)j, &Z, &Zs, &Us, &Zt, &Ut);
       xj = fmaR(sv, Z, mu);
@@ -2957,7 +2967,7 @@ __global__ void __launch_bounds__(BLOCK) k_estimate_w(FilterArgs<R> a) {
     const uint64_t i = base + e;
     if (i < a.n) {
       R wr;
-      (void)quant_exp<R>(a.lam[i], a.k, &wr);
+      (void)quant_exp(a.lam[i], a.k, &wr);
       const double w = (double)wr;
       const double dx = (double)(st.x[i] - c0), ds = (double)(st.s2[i] - c1),
                    dt = (double)(st.t2[i] - c2);
