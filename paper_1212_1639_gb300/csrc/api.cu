@@ -101,6 +101,7 @@ struct pf_filter {
   bool fp64 = false, learn = true;
   int scheme = 0;
   unsigned prop_grid = 0;  // persistent propagate grid
+  unsigned exp_grid = 0;   // binary64: grid of k_exp
   uint64_t w_cap = 1;      // resident CTAs of the weights kernel
   unsigned prop_grid_fuse = 0;  // the same for the propagation that also weighs
   unsigned cdf_grid = 0;   // cooperative CDF + systematic resampling grid (0: not used)
@@ -343,8 +344,12 @@ pf_status enqueue_cycle(pf_filter* f, KTimer* tm = nullptr, const double* y_src 
     else k_weights<R><<<wg, BLOCK, 0, s>>>(a);
     mark(tm, "weights", s);
   }
+  if constexpr (sizeof(R) == 8) {
+    k_exp<<<f->exp_grid, BLOCK, 0, s>>>(a);
+    mark(tm, "exp", s);
+  }
   ScanArgs sa;
-  sa.src = f->ell;
+  sa.src = f->fp64 ? (const void*)f->Q : f->ell;
   sa.Q = f->Q;
   sa.stat[0] = f->stat_w[0];
   sa.stat[1] = f->stat_w[1];
@@ -749,7 +754,7 @@ pf_status pf_create(const pf_config* cfg, pf_filter** out) {
   if (cudaGetLastError() != cudaSuccess) return bail(set_err(PF_ERR_CUDA, "init kernel launch failed"));
   {
     // persistent propagate grid: resident blocks per SM x SMs, at most one
-    // block per BLOCK slots
+    // block per 2 BLOCK slots (binary64: per 32, one warp's, see spread_slot)
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -761,9 +766,10 @@ pf_status pf_create(const pf_config* cfg, pf_filter** out) {
       e = f->learn ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_propagate2<true>, BLOCK, 0)
                    : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_propagate2<false>, BLOCK, 0);
     if (e != cudaSuccess || per_sm < 1 || sms < 1) return bail(set_err(PF_ERR_CUDA, "occupancy query failed"));
-    const uint64_t want = cdiv(n, f->fp64 ? (uint64_t)BLOCK : 2ull * BLOCK),
+    const uint64_t want = cdiv(n, f->fp64 ? 32ull : 2ull * BLOCK),
                    cap = (uint64_t)per_sm * (uint64_t)sms;
     f->prop_grid = (unsigned)(want < cap ? want : cap);
+    f->exp_grid = (unsigned)(want < 8ull * sms ? want : 8ull * sms);
     int per_sm_f = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_f, prop_fuse_fn(f), BLOCK, 0);
     if (e != cudaSuccess || per_sm_f < 1) return bail(set_err(PF_ERR_CUDA, "occupancy query failed"));

@@ -224,10 +224,10 @@ __device__ __forceinline__ void mt_constants(double a, double* d, double* c, dou
   const double SQZ = 0x1.698a4eea9073cp-6;
   const double dd = a - ONE_THIRD;
   const double nine_d = 9.0 * dd;
-  const double s = sqrt(nine_d);
+  const double s = sqrt_rn(nine_d);
   *d = dd;
-  *c = 1.0 / s;
-  *K = SQZ / dd;
+  *c = div_rn(1.0, s);
+  *K = div_rn(SQZ, dd);
 }
 // This cycle's constants for the propagation (observation and the
 // Marsaglia-Tsang constants of the shapes a0 + (t+1)/2), in both precisions.
@@ -348,6 +348,15 @@ __device__ __forceinline__ R block_max(R v, R* s_red) {
   return v;
 }
 
+// Binary64 kernels over single particles: warp w of CTA b takes 32 consecutive
+// ones at (w gridDim + b) 32, then steps by the grid's threads.  A sub-partition
+// takes 64 cycles per binary64 warp instruction, so a small filter finishes
+// sooner with one warp on each of many SMs than with the eight warps of a CTA
+// on one: N = 1024 weights 15.7 -> 11.2 us by events (all on one SM before).
+__device__ __forceinline__ uint64_t spread_slot() {
+  return ((uint64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32 + (threadIdx.x & 31);
+}
+
 // Persistent over the particles: per pass a warp takes a chunk of 64 16-byte
 // vectors of each array (2 x 32 x W_VEC particles), each load and store
 // instruction 512 contiguous bytes, two of each in flight per thread and array;
@@ -387,6 +396,7 @@ __global__ void __launch_bounds__(BLOCK, W_CTAS_PER_SM) k_weights(FilterArgs<R> 
   const int lane = threadIdx.x & 31;
   const uint64_t gw = (uint64_t)blockIdx.x * WARPS + (threadIdx.x >> 5);
   const uint64_t nw = (uint64_t)gridDim.x * WARPS;
+  (void)gw; (void)nw;
   MaxL<R> top;
   auto weigh = [&](R x, R s2, R t2, R lam) {
     R l = log_pred<R>(x, s2, t2, yr);
@@ -418,7 +428,12 @@ __global__ void __launch_bounds__(BLOCK, W_CTAS_PER_SM) k_weights(FilterArgs<R> 
     }
   };
   const uint64_t nchunks = (n + CHUNK - 1) / CHUNK;
-  if (nchunks >= 4 * nw) {
+  if constexpr (sizeof(R) == 8) {
+    // bound by the binary64 pipe, not by loads: one particle per lane, the
+    // warps of a CTA far apart, so that few particles still reach every SM
+    for (uint64_t i = spread_slot(); i < n; i += nw * 32)
+      a.ell[i] = weigh(st.x[i], st.s2[i], st.t2[i], ESS ? a.lam[i] : (R)0);
+  } else if (nchunks >= 4 * nw) {
     // Many chunks per warp: rounds of WARPS chunks (one per warp) go to
     // CTAs by ticket, each ticket taken a round ahead by thread 0, so that
     // CTAs on faster SMs take more rounds (the CTAs' finishing times under
@@ -449,7 +464,8 @@ __global__ void __launch_bounds__(BLOCK, W_CTAS_PER_SM) k_weights(FilterArgs<R> 
 // fewer when the particles make fewer chunks than the resident warps.
 template <class R>
 inline unsigned weights_grid(uint64_t n, uint64_t cap) {
-  const uint64_t per_cta = 64ull * WVec<R>::N * WARPS;  // one chunk per warp
+  // binary32: one chunk per warp; binary64: 32 particles, so that a CTA has one warp's work
+  const uint64_t per_cta = sizeof(R) == 8 ? 32ull : 64ull * WVec<R>::N * WARPS;
   const uint64_t ctas = (n + per_cta - 1) / per_cta;
   return (unsigned)(ctas < cap ? (ctas > 0 ? ctas : 1) : cap);
 }
@@ -544,6 +560,18 @@ template <class R> struct ESumT;
 template <> struct ESumT<float> { typedef ESum32 T; };
 template <> struct ESumT<double> { typedef ESum64 T; };
 
+// Binary64: e_i = exp(l_i - m) for every particle, into the space of the CDF
+// (the scan reads e and writes Q in its place; l stays for a propagation that
+// carries L - m).  The exponential is 21 of the CDF's 23 operations on the
+// binary64 pipe; here it runs one particle per lane on every SM, where a scan
+// tile would do 4096 of them on one: systematic cycle at N = 16384 70.7 -> 41.8
+// us, at N = 2^20 (256 tiles on 152 SMs) 329 -> 313 us.
+static __global__ void __launch_bounds__(BLOCK) k_exp(FilterArgs<double> a) {
+  const double m = dec_d(a.ctl->maxenc);
+  double* const E = reinterpret_cast<double*>(a.Q);
+  for (uint64_t i = spread_slot(); i < a.n; i += (uint64_t)gridDim.x * BLOCK) E[i] = exp_weight(a.ell[i] - m);
+}
+
 // Tile look-back by warp 0.  Returns the exclusive prefix of the tile (in
 // lane 0).  `total` is the tile aggregate.  Each round reads a window of 128
 // predecessors (four status words per lane, loads issued together), so a
@@ -622,7 +650,7 @@ __device__ __forceinline__ uint64_t lookback(uint64_t* stat, uint32_t tile, uint
 enum ScanMode { FROM_LOGLIK = 0, FROM_WEIGHTS = 1 };
 
 struct ScanArgs {
-  const void* src;          // l (R) or w (float)
+  const void* src;          // l (float), e (double, in Q's place) or w (float)
   uint64_t* Q;
   uint64_t* stat[2];        // tile status by cycle parity; the other parity's
                             // entries are cleared for the next cycle
@@ -699,8 +727,13 @@ __global__ void __launch_bounds__(BLOCK, 4) k_scan(ScanArgs a) {
       if (full || base + 4 * q + e < a.n) {
         if (MODE == FROM_LOGLIK) {
           R ex;
-          const R dl = v[e] - m;
-          w = quant_exp(dl, a.k, &ex);
+          if constexpr (sizeof(R) == 8) {  // src holds e (k_exp)
+            ex = v[e];
+            w = quant_from_e(ex, a.k);
+          } else {
+            const R dl = v[e] - m;
+            w = quant_exp(dl, a.k, &ex);
+          }
           epart = epart + ex;
         } else {
           const float wf = (float)v[e];
@@ -1490,7 +1523,9 @@ __global__ void __launch_bounds__(BLOCK, PER == 8 ? 4 : 3) k_cdf_sys(FilterArgs<
   // staged: phase 1 writes e = exp(l - m) back in l's place and phase 2
   // quantises from e (no second exponential); with ESS, or without
   // write-back, phase 2 quantises from l again
-  constexpr bool WB = STAGED && !ESS;
+  // binary64: e was computed by k_exp into the space of Q; both phases read it
+  constexpr bool PRE_E = sizeof(R) == 8;
+  constexpr bool WB = STAGED && !ESS && !PRE_E;
   constexpr int TP = BLOCK * PER;  // particles per tile
   typedef typename ESumT<R>::T ES;
   __shared__ uint64_t s_warp[WARPS + 1];
@@ -1528,6 +1563,8 @@ __global__ void __launch_bounds__(BLOCK, PER == 8 ? 4 : 3) k_cdf_sys(FilterArgs<
   if constexpr (sizeof(R) == 4) m = dec_f((uint32_t)c->maxenc);
   else m = dec_d(c->maxenc);
   const int k = a.k;
+  (void)m;
+  R* const wsrc = PRE_E ? reinterpret_cast<R*>(a.Q) : a.ell;  // l, or e
   // TMA rings (staged).  Phase 1: the CTA's tile i goes to ring buffer
   // i % NB1 with barrier i % NB1; phase 2: tile i to s_ell[i & 1] with
   // barrier NB1 + (i & 1).  The k-th copy through a barrier completes its
@@ -1561,7 +1598,7 @@ __global__ void __launch_bounds__(BLOCK, PER == 8 ? 4 : 3) k_cdf_sys(FilterArgs<
     const uint64_t cnt = n - first < (uint64_t)TP ? n - first : (uint64_t)TP;
     const uint32_t bytes = (uint32_t)((cnt * sizeof(R) + 15) & ~(uint64_t)15);
     fence_proxy_async_smem();  // (phase 2: the buffer held the previous tile's window)
-    tma_load_1d(dst, a.ell + first, bytes, &s_bar[bi]);
+    tma_load_1d(dst, wsrc + first, bytes, &s_bar[bi]);
     ++iss_b[bi];
   };
   // every thread: wait for the k-th copy through barrier bi
@@ -1624,7 +1661,7 @@ __global__ void __launch_bounds__(BLOCK, PER == 8 ? 4 : 3) k_cdf_sys(FilterArgs<
             w = quant_exp(dl, k, &ex);
           }
           ep = ep + ex;
-          mx = ex > mx ? ex : mx;
+          mx = pos_less(mx, ex) ? ex : mx;
         }
         ex4[e] = ex;
         exs[4 * q + e] = ex;
@@ -1709,7 +1746,7 @@ __global__ void __launch_bounds__(BLOCK, PER == 8 ? 4 : 3) k_cdf_sys(FilterArgs<
       // (with ESS l stays in place: a propagation that does not resample
       // carries L - m from it, so phase 2 quantises from l again)
       R emx;
-      quantP(tile, buf, W, &ep, &emx, WB ? 1 : 0);
+      quantP(tile, buf, W, &ep, &emx, PRE_E ? 2 : (WB ? 1 : 0));
       if (WB) fence_proxy_async_smem();  // e in buf, for the bulk store below
       mine += W[PER - 1];
       add_sq(W);
@@ -1737,7 +1774,7 @@ __global__ void __launch_bounds__(BLOCK, PER == 8 ? 4 : 3) k_cdf_sys(FilterArgs<
     for (uint32_t tile = tb; tile < te; ++tile) {
       uint64_t W[PER];
       R ep;
-      quantP(tile, a.ell + (uint64_t)tile * TP, W, &ep, &emx_keep, 0);
+      quantP(tile, wsrc + (uint64_t)tile * TP, W, &ep, &emx_keep, PRE_E ? 2 : 0);
       mine += W[PER - 1];
       add_sq(W);
 #pragma unroll
@@ -1852,7 +1889,7 @@ __global__ void __launch_bounds__(BLOCK, PER == 8 ? 4 : 3) k_cdf_sys(FilterArgs<
       // stored out), then this one
       if (threadIdx.x == 0 && tile + 1 < te) issue(NB1 + ((i2 + 1) & 1), s_ell[(i2 + 1) & 1], tile + 1);
       take(NB1 + (i2 & 1), i2 >> 1);
-      quantP(tile, s_ell[i2 & 1], W, &ep, &emx, WB ? 2 : 0);
+      quantP(tile, s_ell[i2 & 1], W, &ep, &emx, (WB || PRE_E) ? 2 : 0);
     }
     // the tile's first slot S0 = R(carry)
     // (a later tile starts where the previous one ended: no division)
@@ -2345,8 +2382,7 @@ __device__ __forceinline__ Gathered<R> gather_rec(const StateV<R>& src, uint32_t
   return g;
 }
 
-// Persistent grid: thread (block b, lane t) handles slots j = b*BLOCK + t +
-// k * stride.  The ancestor index is loaded two slots ahead and the ancestor's
+// Persistent grid: a thread handles the slots spread_slot() + k * stride.  The ancestor index is loaded two slots ahead and the ancestor's
 // record one slot ahead, so the dependent index -> gather latency overlaps the
 // arithmetic of the current slot.
 //
@@ -2421,7 +2457,7 @@ __global__ void __launch_bounds__(BLOCK, 3) k_propagate(FilterArgs<R> a) {
   auto weigh_late = [&](const Item& itm) {  // FUSE: the slot's state is final
     weigh_next<R>(a.ell, itm.j, dst.x[itm.j], dst.s2[itm.j], dst.t2[itm.j], yn, mxn, badn);
   };
-  uint64_t j = (uint64_t)blockIdx.x * BLOCK + threadIdx.x;
+  uint64_t j = spread_slot();
   uint32_t an = j < n ? ancx(j) : 0;
   uint32_t an_next = j + stride < n ? ancx(j + stride) : 0;
   Gathered<R> cur = gather_rec<R>(src, an);
