@@ -104,28 +104,21 @@ struct pf_filter {
   unsigned exp_grid = 0;   // binary64: grid of k_exp
   uint64_t w_cap = 1;      // resident CTAs of the weights kernel
   unsigned prop_grid_fuse = 0;  // the same for the propagation that also weighs
-  unsigned cdf_grid = 0;   // cooperative CDF + systematic resampling grid (0: not used)
-  bool cdf_staged = false; // its CTAs own several tiles: TMA-staged variant
-  int cdf_per = 16;         // particles per thread of its tiles (8: 2048-particle tiles)
   bool bootstrap = false;   // Algorithm "Particle Filtering" instead of particle learning
   uint32_t nparts = 0;      // log-ML partials per cycle
-  uint64_t* cta_tot = nullptr;
-  U128* cta_sq = nullptr;  // adaptive resampling: per-CTA sums of W^2 of the cooperative kernel
+  uint64_t* pre = nullptr;  // CDF tile prefixes (k_sums)
+  U128* sq = nullptr;       // adaptive resampling: per-CTA sums of W^2 (k_sums)
   std::vector<void*> allocs;
   void* x[2] = {}; void* s2[2] = {}; void* t2[2] = {}; void* bs[2] = {}; void* bt[2] = {};
   void* ell = nullptr;
-  // adaptive resampling (cfg.ess_frac > 0): carried log-weights, the grid of
-  // the decision kernel and its per-block partial sums
+  // adaptive resampling (cfg.ess_frac > 0): carried log-weights
   bool ess = false;
   void* lam = nullptr;
-  unsigned ess_grid = 0;
-  U128* ess_part = nullptr;
   uint64_t* Q = nullptr;
   uint64_t* S = nullptr;
   uint32_t* anc = nullptr;
   uint32_t* I = nullptr;
   uint64_t* splits = nullptr;  // merge-path partition
-  uint64_t* stat_w[2] = {};
   uint64_t* stat_e[2] = {};
   void* part = nullptr;
   double* part_est = nullptr;
@@ -188,13 +181,10 @@ FilterArgs<R> filter_args(pf_filter* f) {
     a.st[p].t2 = (R*)f->t2[p];
     a.st[p].bs = (B*)f->bs[p];
     a.st[p].bt = (B*)f->bt[p];
-    a.stat_w[p] = f->stat_w[p];
     a.stat_e[p] = f->stat_e[p];
   }
   a.ell = (R*)f->ell;
   a.lam = (R*)f->lam;
-  a.ess_frac = f->cfg.ess_frac;
-  a.ess_part = f->ess_part;
   a.Q = f->Q;
   a.S = f->S;
   a.anc = f->anc;
@@ -250,29 +240,19 @@ bool is_multinomial(int scheme) { return scheme == PF_MULTINOMIAL || scheme == P
 bool is_cutpoint(int scheme) { return scheme == PF_MULTINOMIAL_CUTPOINT || scheme == PF_SYSTEMATIC_CUTPOINT; }
 
 // Resampling kernels shared by the filter cycle and pf_resample: from a
-// finished CDF Q (and spacing prefix S) to ancestors.
+// finished CDF Q (and spacing prefix S) to ancestors (multinomial and the
+// cut-point schemes; systematic and stratified ancestors come from k_slots).
 inline uint32_t merge_chunks(uint64_t n) { return (uint32_t)cdiv(2 * n, MERGE_D); }
-inline uint32_t sys_chunks(uint64_t n) { return (uint32_t)cdiv(2 * n, SYS_D); }
 
 pf_status launch_resample(int scheme, const PosArgs& pa, uint64_t n, uint32_t* I,
                           uint64_t* splits, cudaStream_t s, KTimer* tm = nullptr) {
   const bool multi = is_multinomial(scheme);
-  if (scheme == PF_STRATIFIED) {
-    k_strat<<<(unsigned)cdiv(n, BLOCK), BLOCK, 0, s>>>(pa);
-    mark(tm, "stratified", s);
-  } else if (!is_cutpoint(scheme) && multi) {
+  if (!is_cutpoint(scheme) && multi) {
     const uint32_t chunks = merge_chunks(n);
     const unsigned pgrid = (unsigned)cdiv((uint64_t)(chunks + 1) * 32, BLOCK);
     k_partition<POS_MULTINOMIAL><<<pgrid, BLOCK, 0, s>>>(pa, splits, chunks + 1, MERGE_D);
     mark(tm, "partition", s);
     k_merge<POS_MULTINOMIAL><<<chunks, BLOCK, 0, s>>>(pa, splits);
-    mark(tm, "merge", s);
-  } else if (!is_cutpoint(scheme)) {
-    const uint32_t chunks = sys_chunks(n);
-    const unsigned pgrid = (unsigned)cdiv((uint64_t)(chunks + 1) * 32, BLOCK);
-    k_partition<POS_SYSTEMATIC><<<pgrid, BLOCK, 0, s>>>(pa, splits, chunks + 1, SYS_D);
-    mark(tm, "partition", s);
-    k_merge_sys<<<chunks, SYS_THREADS, 0, s>>>(pa, splits);
     mark(tm, "merge", s);
   } else {
     const unsigned grid = (unsigned)cdiv(n, BLOCK);
@@ -284,6 +264,69 @@ pf_status launch_resample(int scheme, const PosArgs& pa, uint64_t n, uint32_t* I
   }
   CK(cudaGetLastError());
   return PF_OK;
+}
+
+// Which slot map a scheme uses (SLOTS_NONE: its ancestors come from launch_resample).
+int slot_pos(int scheme) {
+  return scheme == PF_SYSTEMATIC ? SLOTS_SYS : scheme == PF_STRATIFIED ? SLOTS_STRAT : SLOTS_NONE;
+}
+template <int SRC>
+void launch_slots(int pos, const SlotArgs& a, cudaStream_t s) {
+  if (pos == SLOTS_SYS) k_slots<SRC, SLOTS_SYS><<<a.ntiles, BLOCK, 0, s>>>(a);
+  else if (pos == SLOTS_STRAT) k_slots<SRC, SLOTS_STRAT><<<a.ntiles, BLOCK, 0, s>>>(a);
+  else k_slots<SRC, SLOTS_NONE><<<a.ntiles, BLOCK, 0, s>>>(a);
+}
+inline unsigned sums_grid(uint64_t n) { return (unsigned)cdiv(n, SUM_TILE); }
+
+// The filter's CDF and, for the systematic and stratified schemes, its
+// ancestors: the tile sums (k_sums, also the log-ML and the adaptive decision),
+// then the tiles (k_slots).  Binary32 plain: k_sums leaves e in l's place;
+// adaptive: l stays (a propagation that does not resample carries L - max),
+// so k_slots takes the exponential again; binary64: e is in Q's space.
+template <class R>
+void launch_cdf(pf_filter* f, cudaStream_t s, KTimer* tm) {
+  SlotArgs a;
+  std::memset(&a, 0, sizeof(a));
+  a.Q = f->Q;
+  a.anc = f->anc;
+  a.pre = f->pre;
+  a.part = f->part;
+  a.sq = f->sq;
+  a.ctl = f->ctl;
+  a.t_dev = &f->ctl->t;
+  a.n = f->n;
+  a.ntiles = (uint32_t)cdiv(f->n, SLOT_TILE);
+  a.k = f->k;
+  a.seed = f->cfg.seed;
+  a.filter = f->cfg.filter_id;
+  a.ess_frac = f->cfg.ess_frac;
+  a.gate = f->ess ? &f->ctl->resamp : nullptr;
+  a.src_vec = a.anc_vec = 1;
+  const unsigned sg = sums_grid(f->n);
+  const int pos = slot_pos(f->scheme);
+  if (pos != SLOTS_NONE && !f->fp64) a.heavy = (char*)f->pre + pre_bytes(f->n);
+  if constexpr (sizeof(R) == 8) {
+    a.src = f->Q;
+    a.part_blk = f->part;
+    if (f->ess) k_sums<SRC_E64, true><<<sg, BLOCK, 0, s>>>(a);
+    else k_sums<SRC_E64, false><<<sg, BLOCK, 0, s>>>(a);
+    mark(tm, "cdf_sums", s);
+    launch_slots<SRC_E64>(pos, a, s);
+  } else {
+    a.src = f->ell;
+    a.part_blk = (char*)f->part + sizeof(ESum32);
+    if (f->ess) {
+      k_sums<SRC_LOG, true><<<sg, BLOCK, 0, s>>>(a);
+      mark(tm, "cdf_sums", s);
+      launch_slots<SRC_LOG>(pos, a, s);
+    } else {
+      a.e_out = (float*)f->ell;
+      k_sums<SRC_LOG, false><<<sg, BLOCK, 0, s>>>(a);
+      mark(tm, "cdf_sums", s);
+      launch_slots<SRC_E32>(pos, a, s);
+    }
+  }
+  mark(tm, pos == SLOTS_NONE ? "cdf" : "cdf_resample", s);
 }
 
 // One cycle (Steps 1-4), enqueued on f->stream; reads t and y on the device.
@@ -348,28 +391,7 @@ pf_status enqueue_cycle(pf_filter* f, KTimer* tm = nullptr, const double* y_src 
     k_exp<<<f->exp_grid, BLOCK, 0, s>>>(a);
     mark(tm, "exp", s);
   }
-  ScanArgs sa;
-  sa.src = f->fp64 ? (const void*)f->Q : f->ell;
-  sa.Q = f->Q;
-  sa.stat[0] = f->stat_w[0];
-  sa.stat[1] = f->stat_w[1];
-  sa.part = f->part;
-  sa.ctl = f->ctl;
-  sa.t_dev = &f->ctl->t;
-  sa.t_arg = 0;
-  sa.n = n;
-  sa.k = f->k;
-  sa.spin_limit = SPIN_LIMIT;
-  sa.withhold = NO_TILE;
-  sa.vec_ok = 1;
-  if (!f->cdf_grid) {
-    k_scan<FROM_LOGLIK, R><<<f->ntiles, BLOCK, 0, s>>>(sa);
-    mark(tm, "scan", s);
-  }
-  if (f->ess && !f->cdf_grid) {  // adaptive resampling: the decision from the finished CDF
-    k_ess<R><<<f->ess_grid, BLOCK, 0, s>>>(a);
-    mark(tm, "ess", s);
-  }
+  launch_cdf<R>(f, s, tm);
   if (fork) {
     CK(cudaStreamWaitEvent(s, f->ev_join, 0));
   } else if (is_multinomial(f->scheme)) {
@@ -388,33 +410,7 @@ pf_status enqueue_cycle(pf_filter* f, KTimer* tm = nullptr, const double* y_src 
   pa.n = n;
   pa.seed = f->cfg.seed;
   pa.filter = f->cfg.filter_id;
-  if (f->cdf_grid) {
-    // systematic: the CDF and the resampling in one cooperative launch
-    cudaLaunchConfig_t cfg;
-    std::memset(&cfg, 0, sizeof(cfg));
-    cfg.gridDim = dim3(f->cdf_grid, 1, 1);
-    cfg.blockDim = dim3(BLOCK, 1, 1);
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    U128* const sq = f->cta_sq;
-    if (f->cdf_staged) {
-      if (f->ess) CK(cudaLaunchKernelEx(&cfg, k_cdf_sys<R, true, 16, true>, a, f->cta_tot, sq));
-      else CK(cudaLaunchKernelEx(&cfg, k_cdf_sys<R, true, 16>, a, f->cta_tot, sq));
-    } else if (f->cdf_per == 8) {
-      if constexpr (sizeof(R) == 4) {
-        if (f->ess) CK(cudaLaunchKernelEx(&cfg, k_cdf_sys<float, false, 8, true>, a, f->cta_tot, sq));
-        else CK(cudaLaunchKernelEx(&cfg, k_cdf_sys<float, false, 8>, a, f->cta_tot, sq));
-      }
-    } else {
-      if (f->ess) CK(cudaLaunchKernelEx(&cfg, k_cdf_sys<R, false, 16, true>, a, f->cta_tot, sq));
-      else CK(cudaLaunchKernelEx(&cfg, k_cdf_sys<R, false, 16>, a, f->cta_tot, sq));
-    }
-    mark(tm, "cdf_resample", s);
-  } else {
+  if (slot_pos(f->scheme) == SLOTS_NONE) {
     pf_status st = launch_resample(f->scheme, pa, n, f->I, f->splits, s, tm);
     if (st != PF_OK) return st;
   }
@@ -461,20 +457,6 @@ pf_status enqueue_cycle(pf_filter* f, KTimer* tm = nullptr, const double* y_src 
   }
   CK(cudaGetLastError());
   return PF_OK;
-}
-
-// The cooperative CDF + systematic resampling kernel of a configuration.
-const void* cdf_fn(bool fp64, bool staged, int per, bool ess) {
-  if (per == 8)
-    return ess ? (const void*)k_cdf_sys<float, false, 8, true> : (const void*)k_cdf_sys<float, false, 8>;
-  if (fp64) {
-    if (staged)
-      return ess ? (const void*)k_cdf_sys<double, true, 16, true> : (const void*)k_cdf_sys<double, true, 16>;
-    return ess ? (const void*)k_cdf_sys<double, false, 16, true> : (const void*)k_cdf_sys<double, false, 16>;
-  }
-  if (staged)
-    return ess ? (const void*)k_cdf_sys<float, true, 16, true> : (const void*)k_cdf_sys<float, true, 16>;
-  return ess ? (const void*)k_cdf_sys<float, false, 16, true> : (const void*)k_cdf_sys<float, false, 16>;
 }
 
 // The propagation that also computes the next cycle's weights (binary32:
@@ -666,11 +648,9 @@ pf_status pf_create(const pf_config* cfg, pf_filter** out) {
     if ((st = dev_alloc(f, n * rs, &f->t2[p])) != PF_OK) return bail(st);
     if ((st = dev_alloc(f, n * 8, &f->bs[p])) != PF_OK) return bail(st);
     if ((st = dev_alloc(f, n * 8, &f->bt[p])) != PF_OK) return bail(st);
-    if ((st = dev_alloc(f, (size_t)f->ntiles * 8, (void**)&f->stat_w[p])) != PF_OK) return bail(st);
     if ((st = dev_alloc(f, (size_t)f->ntiles * 8, (void**)&f->stat_e[p])) != PF_OK) return bail(st);
   }
-  // l is moved by 16-byte bulk copies: its tail is padded to 16 bytes
-  if ((st = dev_alloc(f, (n * rs + 15) & ~(size_t)15, &f->ell)) != PF_OK) return bail(st);
+  if ((st = dev_alloc(f, n * rs, &f->ell)) != PF_OK) return bail(st);
   if ((st = dev_alloc(f, n * 8, (void**)&f->Q)) != PF_OK) return bail(st);
   if (is_multinomial(f->scheme)) {
     if ((st = dev_alloc(f, (n + 1) * 8, (void**)&f->S)) != PF_OK) return bail(st);
@@ -682,17 +662,16 @@ pf_status pf_create(const pf_config* cfg, pf_filter** out) {
   if ((st = dev_alloc(f, n * 4, (void**)&f->anc)) != PF_OK) return bail(st);
   if (is_cutpoint(f->scheme) && (st = dev_alloc(f, n * 4, (void**)&f->I)) != PF_OK) return bail(st);
   if ((st = dev_alloc(f, ((size_t)merge_chunks(n) + 1) * 8, (void**)&f->splits)) != PF_OK) return bail(st);
-  // log-ML partials: one per CDF tile (2048-particle tiles need twice as many)
-  if ((st = dev_alloc(f, (size_t)f->ntiles * 32, &f->part)) != PF_OK) return bail(st);
-  f->nparts = f->ntiles;
+  // log-ML partials.  Binary64: one per 4096 particles (rounded sums, folded in
+  // order); binary32: exact sums, folded into the first entry by k_sums
+  if ((st = dev_alloc(f, ((size_t)f->ntiles + 1) * sizeof(ESum32), &f->part)) != PF_OK) return bail(st);
+  f->nparts = f->fp64 ? f->ntiles : 1;
+  if ((st = dev_alloc(f, pre_heavy_bytes(n), (void**)&f->pre)) != PF_OK) return bail(st);
   const uint64_t est_blocks = cdiv(n, (uint64_t)BLOCK * EST_PER_THREAD);
   if ((st = dev_alloc(f, est_blocks * 8 * 8, (void**)&f->part_est)) != PF_OK) return bail(st);
   if (f->ess) {
     if ((st = dev_alloc(f, n * rs, &f->lam)) != PF_OK) return bail(st);
-    const uint64_t eb = cdiv(n, (uint64_t)BLOCK * ESS_PER_THREAD);
-    f->ess_grid = (unsigned)(eb < 1024 ? eb : 1024);
-    if ((st = dev_alloc(f, (size_t)f->ess_grid * sizeof(U128), (void**)&f->ess_part)) != PF_OK)
-      return bail(st);
+    if ((st = dev_alloc(f, (size_t)sums_grid(n) * sizeof(U128), (void**)&f->sq)) != PF_OK) return bail(st);
   }
   if ((st = dev_alloc(f, sizeof(Ctl), (void**)&f->ctl)) != PF_OK) return bail(st);
   if (cudaHostAlloc((void**)&f->ctl_host, sizeof(Ctl), cudaHostAllocMapped) != cudaSuccess) {
@@ -737,8 +716,7 @@ pf_status pf_create(const pf_config* cfg, pf_filter** out) {
   if (f->ess && cudaMemsetAsync(f->lam, 0, n * rs, f->stream) != cudaSuccess)
     return bail(set_err(PF_ERR_CUDA, "log-weight memset failed"));
   for (int p = 0; p < 2; ++p) {
-    if (cudaMemsetAsync(f->stat_w[p], 0, (size_t)f->ntiles * 8, f->stream) != cudaSuccess ||
-        cudaMemsetAsync(f->stat_e[p], 0, (size_t)f->ntiles * 8, f->stream) != cudaSuccess)
+    if (cudaMemsetAsync(f->stat_e[p], 0, (size_t)f->ntiles * 8, f->stream) != cudaSuccess)
       return bail(set_err(PF_ERR_CUDA, "status memset failed"));
   }
   const unsigned grid = (unsigned)cdiv(n, BLOCK);
@@ -780,41 +758,6 @@ pf_status pf_create(const pf_config* cfg, pf_filter** out) {
     if (e != cudaSuccess || per_sm_w < 1) return bail(set_err(PF_ERR_CUDA, "occupancy query failed"));
     f->w_cap = (uint64_t)per_sm_w * (uint64_t)sms;
     f->prop_grid_fuse = (unsigned)(want < cap_f ? want : cap_f);
-    if (f->scheme == PF_SYSTEMATIC) {
-      // cooperative grid: every CTA resident at once (it waits on the others).
-      // One tile per CTA when the tiles fit at once -- in binary32 2048-particle
-      // tiles (8 per thread) if those fit, for twice the parallelism -- else
-      // the staged variant over 4096-particle tiles.
-      int cdf_sm = 0;
-      uint64_t g = 0;
-      if (!f->fp64) {
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&cdf_sm, cdf_fn(false, false, 8, f->ess), BLOCK, 0);
-        if (e != cudaSuccess || cdf_sm < 1) return bail(set_err(PF_ERR_CUDA, "occupancy query failed"));
-        g = (uint64_t)cdf_sm * (uint64_t)sms;
-        if (cdiv(n, 8ull * BLOCK) <= g) {
-          f->cdf_per = 8;
-          f->nparts = (uint32_t)cdiv(n, 8ull * BLOCK);
-        }
-      }
-      if (f->cdf_per == 16) {
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&cdf_sm, cdf_fn(f->fp64, false, 16, f->ess), BLOCK, 0);
-        if (e != cudaSuccess || cdf_sm < 1) return bail(set_err(PF_ERR_CUDA, "occupancy query failed"));
-        g = (uint64_t)cdf_sm * (uint64_t)sms;
-        if (f->ntiles > g) {
-          f->cdf_staged = true;
-          e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&cdf_sm, cdf_fn(f->fp64, true, 16, f->ess), BLOCK, 0);
-          if (e != cudaSuccess || cdf_sm < 1) return bail(set_err(PF_ERR_CUDA, "occupancy query failed"));
-          g = (uint64_t)cdf_sm * (uint64_t)sms;
-        }
-      }
-      const uint64_t nt = f->cdf_per == 8 ? f->nparts : f->ntiles;
-      f->cdf_grid = (unsigned)(nt < g ? nt : g);
-      // the staged binary32 kernel leaves one exact log-ML partial per CTA
-      if (f->cdf_staged && !f->fp64) f->nparts = f->cdf_grid;
-      if ((st = dev_alloc(f, (size_t)f->cdf_grid * 8, (void**)&f->cta_tot)) != PF_OK) return bail(st);
-      if (f->ess && (st = dev_alloc(f, (size_t)f->cdf_grid * sizeof(U128), (void**)&f->cta_sq)) != PF_OK)
-        return bail(st);
-    }
   }
   if ((st = build_graph(f, CF_PLAIN)) != PF_OK) return bail(st);
   *out = f;
@@ -1250,6 +1193,7 @@ struct Scratch {
   uint64_t* S;
   uint32_t* I;
   uint64_t* splits;
+  uint64_t* pre;
   uint64_t* stat[2];
   uint64_t* stat_e[2];
   Ctl* ctl;
@@ -1277,6 +1221,7 @@ size_t scratch_layout(uint64_t n, bool need_Q, bool multi, bool cut, char* base,
   s->S = multi ? (uint64_t*)take((n + 1) * 8) : nullptr;
   s->I = cut ? (uint32_t*)take(n * 4) : nullptr;
   s->splits = (uint64_t*)take(((size_t)merge_chunks(n) + 1) * 8);
+  s->pre = (uint64_t*)take(pre_heavy_bytes(n));
   s->base = base;
   (void)zero_bytes;
   return off;
@@ -1299,14 +1244,38 @@ pf_status run_resample(const float* w, uint64_t n, uint64_t seed, uint32_t filte
                        int scheme, uint32_t* anc, uint64_t* Q_out, const Scratch& sc,
                        cudaStream_t s, WaitDiag dg = WaitDiag()) {
   const uint32_t ntiles = (uint32_t)cdiv(n, TILE);
-  const unsigned gmax = (unsigned)(cdiv(n, BLOCK) < 152 * 8 ? cdiv(n, BLOCK) : 152 * 8);
-  k_wmax<<<gmax, BLOCK, 0, s>>>(w, n, sc.ctl);
+  const uint64_t want = cdiv(n, 8 * BLOCK);
+  const unsigned gmax = (unsigned)(want < 152 * 8 ? want : 152 * 8);
+  k_wmax<<<gmax, BLOCK, 0, s>>>(w, n, sc.ctl, ((uintptr_t)w & 31) == 0);
+  if (anc) {
+    // tile sums, then the tiles: ancestors (systematic, stratified), or the CDF
+    SlotArgs a;
+    std::memset(&a, 0, sizeof(a));
+    const int pos = slot_pos(scheme);
+    a.src = w;
+    a.Q = pos == SLOTS_NONE ? sc.Q : nullptr;
+    a.anc = anc;
+    a.pre = sc.pre;
+      if (pos != SLOTS_NONE) a.heavy = (char*)sc.pre + pre_bytes(n);
+    a.ctl = sc.ctl;
+    a.t_arg = t;
+    a.n = n;
+    a.ntiles = (uint32_t)cdiv(n, SLOT_TILE);
+    a.k = cdf_shift(n);
+    a.seed = seed;
+    a.filter = filter;
+    a.src_vec = ((uintptr_t)w & 31) == 0;
+    a.anc_vec = ((uintptr_t)anc & 15) == 0;
+    k_sums<SRC_W, false><<<sums_grid(n), BLOCK, 0, s>>>(a);
+    launch_slots<SRC_W>(pos, a, s);
+    CK(cudaGetLastError());
+    if (pos != SLOTS_NONE) return PF_OK;
+  } else {
   ScanArgs sa;
   sa.src = w;
-  sa.Q = Q_out ? Q_out : sc.Q;
+  sa.Q = Q_out;
   sa.stat[0] = sc.stat[0];
   sa.stat[1] = sc.stat[1];
-  sa.part = nullptr;
   sa.ctl = sc.ctl;
   sa.t_dev = nullptr;
   sa.t_arg = 0;
@@ -1315,9 +1284,10 @@ pf_status run_resample(const float* w, uint64_t n, uint64_t seed, uint32_t filte
   sa.vec_ok = ((uintptr_t)w & 15) == 0;
   sa.spin_limit = dg.spin_limit;
   sa.withhold = dg.withhold;
-  k_scan<FROM_WEIGHTS, float><<<ntiles, BLOCK, 0, s>>>(sa);
+  k_scan<<<ntiles, BLOCK, 0, s>>>(sa);
   CK(cudaGetLastError());
-  if (!anc) return PF_OK;
+  return PF_OK;
+  }
   if (is_multinomial(scheme)) {
     SpacingArgs sp;
     sp.S = sc.S;
@@ -1333,7 +1303,7 @@ pf_status run_resample(const float* w, uint64_t n, uint64_t seed, uint32_t filte
   }
   PosArgs pa;
   pa.gate = nullptr;
-  pa.Q = sa.Q;
+  pa.Q = sc.Q;
   pa.S = sc.S;
   pa.anc = anc;
   pa.I = sc.I;
@@ -1438,7 +1408,8 @@ pf_status resample_common(const float* w, uint64_t n, uint64_t seed, uint32_t fi
     return resample_small(w, n, seed, filter, t, scheme, anc, s);
   Scratch sc;
   const bool multi = anc && is_multinomial(scheme), cut = anc && is_cutpoint(scheme);
-  const size_t bytes = scratch_layout(n, Q_out == nullptr, multi, cut, nullptr, &sc);
+  const bool need_Q = anc && slot_pos(scheme) == SLOTS_NONE;
+  const size_t bytes = scratch_layout(n, need_Q, multi, cut, nullptr, &sc);
   void* base = nullptr;
   cudaMemPool_t pool = nullptr;
   pf_status sp = scratch_pool(&pool);
@@ -1448,7 +1419,7 @@ pf_status resample_common(const float* w, uint64_t n, uint64_t seed, uint32_t fi
     cudaGetLastError();
     return set_err(PF_ERR_OOM, "cudaMallocFromPoolAsync(%zu): %s", bytes, cudaGetErrorString(e));
   }
-  scratch_layout(n, Q_out == nullptr, multi, cut, (char*)base, &sc);
+  scratch_layout(n, need_Q, multi, cut, (char*)base, &sc);
   pf_status st = PF_OK;
   if (cudaMemsetAsync(base, 0, scratch_zero_bytes(n), s) != cudaSuccess)
     st = set_err(PF_ERR_CUDA, "scratch memset failed");
@@ -1542,7 +1513,8 @@ constexpr uint64_t NOALLOC_TILES = (NOALLOC_N + TILE - 1) / TILE;
 constexpr size_t NOALLOC_BYTES =
     align256(sizeof(Ctl)) + 4 * align256(NOALLOC_TILES * 8) + align256(NOALLOC_N * 8) +
     align256((NOALLOC_N + 1) * 8) + align256(NOALLOC_N * 4) +
-    align256(((2 * NOALLOC_N + MERGE_D - 1) / MERGE_D + 1) * 8);
+    align256(((2 * NOALLOC_N + MERGE_D - 1) / MERGE_D + 1) * 8) +
+    align256(pre_heavy_bytes(NOALLOC_N));
 
 // The scratch itself: one copy per device, shared by every call on it.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[NOALLOC_BYTES];

@@ -53,7 +53,6 @@ struct Ctl {
   uint32_t ticket_e;      // spacing scan tile ticket
   uint32_t done_prop;     // last-block counter of k_propagate
   uint32_t done_est;      // last-block counter of k_estimate
-  uint32_t gbar;          // grid barrier of k_cdf_sys
   double logml;           // accumulated log marginal likelihood
   double est[8];          // t, x mean/var, sigma2 mean/var, tau2 mean/var, log_marglik
   // per-cycle constants written by k_weights (block 0) for k_propagate:
@@ -62,22 +61,25 @@ struct Ctl {
                           // squeeze coefficients K_sigma, K_tau ([4], [5]), binary64
   float yf;               // y rounded to binary32
   float mtf[6];           // the same constants rounded to binary32
-  // resampling key constants written by k_partition (block 0) for k_merge:
-  // T = Q_{n-1}, A (n or S_n) and the systematic offset r
+  // resampling key constants written by k_sums, or by k_partition (block 0) for
+  // k_merge: T = Q_{n-1}, A (n or S_n) and the systematic offset r
   uint64_t keyT, keyA, keyR;
   // the next cycle's maximum of l, gathered by a propagation that also
   // computes the next cycle's predictive weights (order-encoded, as maxenc)
   unsigned long long maxenc_nx;
-  // adaptive resampling: this cycle's decision (written by k_ess), the
-  // last-block counter of k_ess, and sum_i exp(lambda_i) of the carried
-  // log-weights (n after a resampling)
+  // adaptive resampling: this cycle's decision (written by k_sums) and
+  // sum_i exp(lambda_i) of the carried log-weights (n after a resampling)
   uint32_t resamp;
-  uint32_t done_ess;
   double slam;
   // binary32 propagation: the next unit of 64 slots to hand out
   unsigned long long prop_ticket;
   // weights kernel: the next round of WARPS chunks to hand out
   uint32_t w_ticket;
+  // k_sums: last-block counter, and the slot map's constants (SlotMap)
+  uint32_t done_sums;
+  int32_t slot_z;
+  uint64_t slot_rho, slot_r32;
+  uint32_t heavy_count, heavy_chunks;
 };
 
 // Tile status words carry their value and flag in one aligned 64-bit word and
@@ -142,7 +144,6 @@ struct FilterArgs {
   uint64_t* S;              // n+1 spacing prefix (multinomial)
   uint32_t* anc;
   uint32_t* I;              // cut-point table
-  uint64_t* stat_w[2];      // scan tile status, by parity
   uint64_t* stat_e[2];      // spacing scan tile status, by parity
   void* part;               // per-tile log-ML partial (U128 for FP32, double for FP64)
   double* part_est;         // per-block estimate partials
@@ -160,14 +161,10 @@ struct FilterArgs {
   // the next cycle's predictive weights (*y_nx_src when set, else y_nx_val)
   const double* y_nx_src;
   double y_nx_val;
-  // adaptive resampling: carried log-weights (NULL: resample every cycle),
-  // the ESS fraction and k_ess's per-block partial sums of W^2
-  R* lam;
-  double ess_frac;
-  U128* ess_part;
+  R* lam;                   // adaptive resampling: carried log-weights (NULL: resample every cycle)
   uint64_t n;
   uint32_t ntiles;
-  uint32_t nparts;          // log-ML partials written this cycle (one per CDF tile)
+  uint32_t nparts;          // log-ML partials written this cycle (binary64: one per 4096 particles)
   int k;                    // CDF shift: W <= 2^k
   uint64_t seed;
   uint32_t filter;
@@ -646,15 +643,22 @@ __device__ __forceinline__ uint64_t lookback(uint64_t* stat, uint32_t tile, uint
   return excl;
 }
 
-// Scan sources.
-enum ScanMode { FROM_LOGLIK = 0, FROM_WEIGHTS = 1 };
+// floor(w 2^s) of a caller's weight (negative and non-finite ones, which
+// k_wmax has flagged: 0); below 2^k by the choice of s
+__device__ __forceinline__ uint64_t quant_weight(float w, int s) {
+  const uint32_t b = __float_as_uint(w);
+  if (b >= 0x7F800000u) return 0;
+  const uint32_t E = b >> 23;
+  const uint32_t m = (b & 0x7fffffu) | (E ? 0x800000u : 0u);
+  const int sh = (int)(E ? E : 1u) - 150 + s;
+  return sh >= 0 ? (uint64_t)m << sh : (uint64_t)(m >> (-sh < 31 ? -sh : 31));
+}
 
 struct ScanArgs {
-  const void* src;          // l (float), e (double, in Q's place) or w (float)
+  const float* src;         // weights
   uint64_t* Q;
   uint64_t* stat[2];        // tile status by cycle parity; the other parity's
                             // entries are cleared for the next cycle
-  void* part;               // per-tile log-ML partial (FROM_LOGLIK)
   Ctl* ctl;
   const uint32_t* t_dev;    // cycle index in device memory, or NULL
   uint32_t t_arg;
@@ -670,14 +674,11 @@ struct ScanArgs {
 // the warp / block scans run once per 16 elements.
 constexpr int SCAN_PER = TILE / BLOCK;  // 16
 
-template <int MODE, class R>
-__global__ void __launch_bounds__(BLOCK, 4) k_scan(ScanArgs a) {
-  typedef typename ESumT<R>::T ES;
+static __global__ void __launch_bounds__(BLOCK, 4) k_scan(ScanArgs a) {
   __shared__ uint64_t s_stage[BLOCK * (SCAN_PER + 1)];
   __shared__ uint32_t s_tile;
   __shared__ uint64_t s_warp_tot[WARPS];
   __shared__ uint64_t s_excl;
-  __shared__ ES s_es[WARPS];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (threadIdx.x == 0) s_tile = atomicAdd(&a.ctl->ticket_w, 1u);
   __syncthreads();
@@ -686,62 +687,28 @@ __global__ void __launch_bounds__(BLOCK, 4) k_scan(ScanArgs a) {
   const uint32_t par = (a.t_dev ? *a.t_dev : a.t_arg) & 1u;
   uint64_t* const stat = par ? a.stat[1] : a.stat[0];
   uint64_t* const stat_next = par ? a.stat[0] : a.stat[1];
-
-  // the value that quantisation is relative to
-  R m = (R)0;
-  int escale = 0;
-  if (MODE == FROM_LOGLIK) {
-    if constexpr (sizeof(R) == 4) m = dec_f((uint32_t)a.ctl->maxenc);
-    else m = dec_d(a.ctl->maxenc);
-  } else {
-    int e;
-    (void)frexpf(__uint_as_float((uint32_t)a.ctl->maxenc), &e);
-    escale = a.k - e;
-  }
+  // quantisation is relative to the power of two of the largest weight
+  int e2;
+  (void)frexpf(__uint_as_float((uint32_t)a.ctl->maxenc), &e2);
+  const int escale = a.k - e2;
 
   const bool full = base + SCAN_PER <= a.n;
   uint64_t W[SCAN_PER];
-  R epart = (R)0;  // this thread's sum of exp(l - m), fixed order
   uint64_t run = 0;
 #pragma unroll
   for (int q = 0; q < SCAN_PER / 4; ++q) {
     // four values at a time, consumed as soon as they arrive
-    R v[4];
+    float v[4];
     if (full && a.vec_ok) {
-      if constexpr (sizeof(R) == 4) {
-        const float4 f = *reinterpret_cast<const float4*>((const float*)a.src + base + 4 * q);
-        v[0] = f.x; v[1] = f.y; v[2] = f.z; v[3] = f.w;
-      } else {
-        const double2 f0 = *reinterpret_cast<const double2*>((const double*)a.src + base + 4 * q);
-        const double2 f1 = *reinterpret_cast<const double2*>((const double*)a.src + base + 4 * q + 2);
-        v[0] = f0.x; v[1] = f0.y; v[2] = f1.x; v[3] = f1.y;
-      }
+      const float4 f = *reinterpret_cast<const float4*>(a.src + base + 4 * q);
+      v[0] = f.x; v[1] = f.y; v[2] = f.z; v[3] = f.w;
     } else {
 #pragma unroll
-      for (int e = 0; e < 4; ++e)
-        v[e] = (base + 4 * q + e < a.n) ? ((const R*)a.src)[base + 4 * q + e] : (R)0;
+      for (int e = 0; e < 4; ++e) v[e] = (base + 4 * q + e < a.n) ? a.src[base + 4 * q + e] : 0.0f;
     }
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-      uint64_t w = 0;
-      if (full || base + 4 * q + e < a.n) {
-        if (MODE == FROM_LOGLIK) {
-          R ex;
-          if constexpr (sizeof(R) == 8) {  // src holds e (k_exp)
-            ex = v[e];
-            w = quant_from_e(ex, a.k);
-          } else {
-            const R dl = v[e] - m;
-            w = quant_exp(dl, a.k, &ex);
-          }
-          epart = epart + ex;
-        } else {
-          const float wf = (float)v[e];
-          if (!(wf >= 0.0f) || !(wf < INFINITY)) atomicOr(&a.ctl->err, ERR_WEIGHTS);
-          else w = f2u64_rz(ldexpf(wf, escale));
-        }
-      }
-      run += w;
+      run += quant_weight(v[e], escale);
       W[4 * q + e] = run;  // inclusive running sum
     }
   }
@@ -749,14 +716,6 @@ __global__ void __launch_bounds__(BLOCK, 4) k_scan(ScanArgs a) {
   const uint64_t tt = W[SCAN_PER - 1];
   const uint64_t tincl = warp_incl_scan(tt, lane);
   if (lane == 31) s_warp_tot[warp] = tincl;
-  if (MODE == FROM_LOGLIK) {
-    ES es;
-    es.zero();
-    es.add(epart);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) es.add(es.shfl_xor(o));
-    if (lane == 0) s_es[warp] = es;
-  }
   __syncthreads();
   if (warp == 0) {
     uint64_t wt = lane < WARPS ? s_warp_tot[lane] : 0;
@@ -779,11 +738,6 @@ __global__ void __launch_bounds__(BLOCK, 4) k_scan(ScanArgs a) {
     if (lane == 0) {
       s_excl = excl;
       stat_next[tile] = 0;
-      if (MODE == FROM_LOGLIK) {
-        ES tot = s_es[0];
-        for (int w = 1; w < WARPS; ++w) tot.add(s_es[w]);
-        reinterpret_cast<ES*>(a.part)[tile] = tot;
-      }
     }
   }
   __syncthreads();
@@ -1085,22 +1039,10 @@ __global__ void __launch_bounds__(BLOCK) k_merge(PosArgs a, const uint64_t* spli
 }
 
 // ---------------------------------------------------------------------------
-// Systematic resampling by a per-thread walk.  Slot j's key is j T + r
-// (A = n), so slots are equally spaced and particle i owns the slots
-// [R_{i-1}, R_i) with R_i = #{j : j T + r < n Q_i}.  Each CTA takes one
-// merge-path tile (particles [i0, i1), slots [j0, j1), j0 <= R_i <= j1 for
-// its particles).  Thread t walks 16 consecutive particles: it finds its
-// first slot once (a division by T through a 64-bit reciprocal), then emits
-// a_j = i while j T + r < n Q_i, stepping the key by T.  A particle owning
-// more than SYS_CAP slots records a run that the whole CTA fills.  The
-// ancestors are staged in shared memory and written out coalesced.
+// Exact slot positions.  Systematic: slot j's key is j T + r (A = n), so slots
+// are equally spaced and particle i owns the slots [R_{i-1}, R_i) with
+// R_i = #{j : j T + r < n Q_i}.
 // ---------------------------------------------------------------------------
-constexpr int SYS_D = 8192;
-constexpr int SYS_THREADS = 512;
-constexpr int SYS_PER = 16;      // particles per thread (SYS_D / SYS_THREADS)
-constexpr int SYS_CAP = 8;       // slots emitted one by one per particle
-constexpr int SYS_MAX_RUNS = SYS_D / SYS_CAP + 2;
-constexpr int BB_RUNS = 512;     // k_cdf_sys: runs per tile held in shared memory
 
 __device__ __forceinline__ U128 sub128(U128 x, uint64_t y) {
   return U128{x.hi - (x.lo < y ? 1ull : 0ull), x.lo - y};
@@ -1170,114 +1112,6 @@ __device__ __forceinline__ uint64_t strat_first(uint64_t q, uint64_t n, uint64_t
   const U128 P = add128(mul64x32(T, (uint32_t)c), strat_offset(T, seed, filter, t, c));
   return lt128(P, X) ? c + 1 : c;
 }
-// One thread per particle: particle i owns the slots [first(n Q_{i-1}),
-// first(n Q_i)); the lower end comes from the neighbouring lane.  A warp
-// stores the ranges longer than 32 slots together.
-static __global__ void __launch_bounds__(BLOCK) k_strat(PosArgs a) {
-  if (gated_off(a)) return;
-  const uint64_t n = a.n;
-  const uint32_t t = a.t_dev ? *a.t_dev : a.t_arg;
-  const uint64_t T = a.Q[n - 1];
-  const uint64_t i = (uint64_t)blockIdx.x * BLOCK + threadIdx.x;
-  const int lane = threadIdx.x & 31;
-  if (T == 0) {  // empty CDF (flagged): keep every index in range
-    if (i == 0) atomicOr(&a.ctl->err, ERR_NUMERIC);
-    if (i < n) a.anc[i] = (uint32_t)i;
-    return;
-  }
-  const SysDiv dv = make_sysdiv(T);
-  const uint64_t j1 = i < n ? strat_first(a.Q[i], n, T, dv, a.seed, a.filter, t) : n;
-  uint64_t j0 = __shfl_up_sync(0xffffffffu, j1, 1);
-  if (lane == 0) j0 = i == 0 ? 0 : (i < n ? strat_first(a.Q[i - 1], n, T, dv, a.seed, a.filter, t) : n);
-  const uint64_t cnt = i < n ? j1 - j0 : 0;
-  if (cnt <= 32) {
-    for (uint64_t q = j0; q < j0 + cnt; ++q) a.anc[q] = (uint32_t)i;
-  }
-  uint32_t heavy = __ballot_sync(0xffffffffu, cnt > 32);
-  while (heavy) {
-    const int l = __ffs(heavy) - 1;
-    heavy &= heavy - 1;
-    const uint64_t s0 = __shfl_sync(0xffffffffu, j0, l), s1 = __shfl_sync(0xffffffffu, j1, l);
-    const uint32_t v = (uint32_t)__shfl_sync(0xffffffffu, i, l);
-    for (uint64_t q = s0 + lane; q < s1; q += 32) a.anc[q] = v;
-  }
-}
-
-static __global__ void __launch_bounds__(SYS_THREADS) k_merge_sys(PosArgs a, const uint64_t* splits) {
-  if (gated_off(a)) return;
-  __shared__ uint32_t s_anc[SYS_D];
-  __shared__ uint32_t s_run[SYS_MAX_RUNS][3];
-  __shared__ uint32_t s_nruns;
-  const uint64_t T = a.ctl->keyT, r = a.ctl->keyR, n = a.n;
-  if (T == 0) {  // empty CDF: flag, keep every index in range
-    if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&a.ctl->err, ERR_NUMERIC);
-    for (uint64_t j = (uint64_t)blockIdx.x * SYS_THREADS + threadIdx.x; j < n;
-         j += (uint64_t)gridDim.x * SYS_THREADS)
-      a.anc[j] = (uint32_t)j;
-    return;
-  }
-  const uint64_t total = 2 * n;
-  const uint64_t d0 = (uint64_t)blockIdx.x * SYS_D;
-  const uint64_t d1 = d0 + SYS_D < total ? d0 + SYS_D : total;
-  const uint64_t i0 = splits[blockIdx.x], i1 = splits[blockIdx.x + 1];
-  const uint64_t j0 = d0 - i0, j1 = d1 - i1;
-  const uint32_t nB = (uint32_t)(j1 - j0);
-  if (threadIdx.x == 0) s_nruns = 0;
-  __syncthreads();
-  const SysDiv dv = make_sysdiv(T);
-  auto add_run = [&](uint64_t st, uint64_t en, uint64_t val) {
-    const uint32_t k = atomicAdd(&s_nruns, 1u);
-    if (k < SYS_MAX_RUNS) {
-      s_run[k][0] = (uint32_t)(st - j0);
-      s_run[k][1] = (uint32_t)(en - j0);
-      s_run[k][2] = (uint32_t)val;
-    }
-  };
-  if (i0 == i1) {
-    if (threadIdx.x == 0 && nB) add_run(j0, j1, i0);  // every slot belongs to particle i0
-  } else {
-    const uint64_t ib = i0 + (uint64_t)threadIdx.x * SYS_PER;
-    if (ib < i1) {
-      const uint64_t ie = ib + SYS_PER < i1 ? ib + SYS_PER : i1;
-      uint64_t j = threadIdx.x == 0 ? j0 : sys_first_slot(a.Q[ib - 1], n, r, dv);
-      j = j < j0 ? j0 : (j > j1 ? j1 : j);
-      U128 KB = add128(mul64x32(T, (uint32_t)j), r);
-      for (uint64_t i = ib; i < ie; ++i) {
-        const uint64_t qi = a.Q[i];
-        const U128 KQ = mul64x32(qi, (uint32_t)n);
-        int emitted = 0;
-        while (j < j1 && lt128(KB, KQ)) {
-          if (emitted == SYS_CAP) {  // a heavy particle: jump to its last slot
-            uint64_t R = sys_first_slot(qi, n, r, dv);
-            R = R < j ? j : (R > j1 ? j1 : R);
-            add_run(j, R, i);
-            j = R;
-            KB = add128(mul64x32(T, (uint32_t)j), r);
-            break;
-          }
-          s_anc[j - j0] = (uint32_t)i;
-          ++j;
-          KB = add128(KB, T);
-          ++emitted;
-        }
-      }
-      if (ie == i1 && j < j1) add_run(j, j1, i1);  // remaining slots belong to particle i1
-    }
-  }
-  __syncthreads();
-  const uint32_t nr = s_nruns < SYS_MAX_RUNS ? s_nruns : SYS_MAX_RUNS;
-  if (s_nruns > SYS_MAX_RUNS && threadIdx.x == 0) atomicOr(&a.ctl->err, ERR_NUMERIC);
-  for (uint32_t k = 0; k < nr; ++k) {
-    const uint32_t st = s_run[k][0], en = s_run[k][1], v = s_run[k][2];
-    for (uint32_t q = st + threadIdx.x; q < en; q += SYS_THREADS) s_anc[q] = v;
-  }
-  __syncthreads();
-  for (uint32_t q = threadIdx.x; q < nB; q += SYS_THREADS) {
-    const uint32_t v = s_anc[q];
-    a.anc[j0 + q] = v < n ? v : (uint32_t)(n - 1);
-  }
-}
-
 // ---------------------------------------------------------------------------
 // The paper's Section 3.2 algorithms.
 // Parallelized Cut-Point Search: thread i computes L_i = ceil(n Q_i / T) and
@@ -1342,127 +1176,13 @@ static __global__ void __launch_bounds__(BLOCK) k_cutpoint_method_explicit(
   anc[j] = (uint32_t)(k < n ? k : n - 1);
 }
 
-// ---------------------------------------------------------------------------
-// Bulk asynchronous copies (TMA, cp.async.bulk) into shared memory, completed
-// on an mbarrier.  Waits are bounded: after SPIN_LIMIT polls they report
-// failure instead of hanging.
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-// make the barrier initialisation visible to the async proxy
-__device__ __forceinline__ void mbar_init_fence() {
-  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-}
-// order this thread's earlier shared-memory accesses before later async-proxy ones
-__device__ __forceinline__ void fence_proxy_async_smem() {
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
-// copy `bytes` (a multiple of 16; both addresses 16-byte aligned) from global
-// to shared memory, completing on `bar`, which expects exactly these bytes
-__device__ __forceinline__ void tma_load_1d(void* dst, const void* src, uint32_t bytes,
-                                            uint64_t* bar) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
-               ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-      ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
-}
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
-  const uint32_t addr = smem_u32(bar);
-  for (uint32_t i = 0; i < SPIN_LIMIT; ++i) {
-    uint32_t done;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(done) : "r"(addr), "r"(parity) : "memory");
-    if (done) return true;
-  }
-  return false;
-}
-
-// copy `bytes` (a multiple of 16; both addresses 16-byte aligned) from
-// shared to global memory as one bulk async-group
-__device__ __forceinline__ void tma_store_1d(void* dst, const void* src, uint32_t bytes) {
-  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
-               ::"l"(dst), "r"(smem_u32(src)), "r"(bytes) : "memory");
-  asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-}
-// wait until this thread's bulk stores have read their shared-memory source
-__device__ __forceinline__ void bulk_wait_read() {
-  asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-}
-// wait until all but the most recent of this thread's bulk store groups
-// have read their shared-memory source
-__device__ __forceinline__ void bulk_wait_read1() {
-  asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
-}
-// wait until this thread's bulk stores are complete
-__device__ __forceinline__ void bulk_wait_done() {
-  asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
-}
-
-// The systematic resampling step writes each particle's slots into a
-// shared-memory window (an entry per slot of the tile, the particle's offset
-// in the tile + 1; the window starts at the tile's first slot rounded down to
-// a multiple of four).  Entry of slot x: x with bits 1-3 XORed by bits 6-8, so
-// that threads writing slots about PER apart, and warps reading consecutive
-// slots, hit distinct banks.  The four slots 4g .. 4g + 3 keep one aligned
-// group of four entries (in the order 0 1 2 3, or 2 3 0 1 when bit 1 is
-// flipped), so the window is read out four slots per 8-byte load.
+// Entry of slot x (relative to the window's base, a multiple of four) in
+// k_slots' window of 16-bit entries: x with bits 1-3 XORed by bits 6-8, so that
+// threads writing slots about eight apart, and warps reading consecutive slots,
+// hit distinct banks.  The four slots 4g .. 4g + 3 keep one aligned group of four
+// entries (in the order 0 1 2 3, or 2 3 0 1 when bit 1 is flipped), so the window
+// is read out four slots per 8-byte load.
 __device__ __forceinline__ uint32_t win_entry(uint32_t x) { return x ^ (((x >> 6) & 7u) << 1); }
-// A run of the CTA's run list: slots [s0, s1) of ancestor v; with WRUN set in
-// v, window slots (relative to the tile's first slot) of mark v & 0xffff.
-constexpr uint32_t WRUN = 0x80000000u;
-
-// Rare paths of the systematic resampling step, kept out of line so that the
-// per-particle loop stays small: the slot count of a heavy particle (more than
-// three slots), and the slots of a particle that its `inl` in-line window
-// writes did not cover -- the rest of a heavy particle's run in the window
-// (by the whole CTA when long) and slots past the window (stored directly, or
-// by the whole CTA when long).
-static __device__ __noinline__ uint32_t sys_heavy_count(int64_t D, SysDiv dv) {
-  return (uint32_t)(sys_floor_div(U128{0, (uint64_t)D - 1}, dv) + 1);
-}
-static __device__ __noinline__ void sys_rest(uint32_t j, uint32_t c, uint32_t S0, uint32_t wslots,
-                                             uint16_t mk, uint32_t ig, uint16_t* win, uint32_t* anc,
-                                             uint32_t (*runs)[3], uint32_t* nruns, uint32_t inl = 2u) {
-  const uint32_t wend = S0 + wslots, e = j + c;
-  const uint32_t a = j + inl < e ? j + inl : e;  // window part [a, b)
-  const uint32_t b = e < wend ? e : wend;
-  if (b > a) {
-    bool queued = false;
-    if (b - a > (uint32_t)SYS_CAP) {
-      const uint32_t kr = atomicAdd(nruns, 1u);
-      if (kr < BB_RUNS) {
-        runs[kr][0] = a - S0;
-        runs[kr][1] = b - S0;
-        runs[kr][2] = WRUN | mk;
-        queued = true;
-      }
-    }
-    if (!queued)
-      for (uint32_t q = a; q < b; ++q) win[win_entry(q - S0)] = mk;
-  }
-  const uint32_t st = j > wend ? j : wend;  // past the window: [st, e)
-  if (e > st) {
-    if (e - st > (uint32_t)SYS_CAP) {
-      const uint32_t kr = atomicAdd(nruns, 1u);
-      if (kr < BB_RUNS) {
-        runs[kr][0] = st;
-        runs[kr][1] = e;
-        runs[kr][2] = ig;
-        return;
-      }
-    }
-    for (uint32_t q = st; q < e; ++q) anc[q] = ig;
-  }
-}
-
 // Correctly rounded conversion of a 128-bit integer to binary64: the top 64
 // significant bits with a sticky bit for the rest, rounded once, scaled by an
 // exact power of two.
@@ -1482,611 +1202,9 @@ __device__ __forceinline__ double u128_to_f64_rn(U128 v) {
   return d * __longlong_as_double((long long)(1023 + sh) << 52);
 }
 
-// ---------------------------------------------------------------------------
-// The CDF and systematic resampling in one cooperative launch (Steps 1b-1c
-// of the cycle for the systematic scheme).  Every CTA owns a contiguous range
-// of tiles of BLOCK x PER particles (thread t: particles [PER t, PER t + PER)):
-//   phase 1  the exact sum of its quantised weights W_i;
-//   barrier  all CTAs (the launch is cooperative, so all are resident; the
-//            wait is bounded and reports ERR_TIMEOUT);
-//   phase 2  its exclusive prefix and T from the CTA sums, then for each of
-//            its tiles the block scan of W with a carry -- thread t holds
-//            Q_i for its particles and Q before them in registers -- the CDF
-//            written out, and systematic resampling from those registers:
-//            each particle writes its slots into a shared-memory window, which
-//            the CTA then stores out coalesced.
-// The quantisation and the log-ML partials (sums over 16 consecutive
-// particles in a fixed order; with PER = 8 a lane pair shares one) are those
-// of k_scan, and the ancestors those of k_merge_sys: the results are the same
-// bits.  Instead of a look-back over tiles in flight, one grid-wide barrier.
-// PER = 8 (binary32) doubles the CTAs for the same particles where one tile
-// per CTA fits at once; the binary32 tile partials are exact, so the tile
-// size does not change them.
-// ---------------------------------------------------------------------------
-// STAGED: a CTA owns several tiles, copied by TMA into shared memory ahead of
-// use.  Phase 1 streams l through a ring of NB1 buffers (NB1 - 1 tiles in
-// flight: phase 1 is bound by the bytes in flight, and the CDF rows' space
-// is free until phase 2) and writes e = exp(l - m) back in l's place by bulk
-// stores, so phase 2 needs no exponentials; phase 2 reads e through a double
-// buffer; the CDF goes out through shared-memory rows, coalesced.  Otherwise
-// (one tile per CTA) l is read directly and the tile's W stay in shared
-// memory between the phases.
-//
-// With ESS (adaptive resampling) phase 1 also sums W^2 exactly per CTA
-// (cta_sq); after the grid barrier every CTA takes k_ess's decision from the
-// totals, CTA 0 publishes it, and a cycle that does not resample writes the
-// CDF and the log-ML partials but no ancestors.
-template <class R, bool STAGED, int PER, bool ESS = false>
-__global__ void __launch_bounds__(BLOCK, PER == 8 ? 4 : 3) k_cdf_sys(FilterArgs<R> a, uint64_t* cta_tot,
-                                                                    U128* cta_sq) {
-  static_assert(PER == 16 || (PER == 8 && !STAGED && sizeof(R) == 4), "tile shapes");
-  // staged: phase 1 writes e = exp(l - m) back in l's place and phase 2
-  // quantises from e (no second exponential); with ESS, or without
-  // write-back, phase 2 quantises from l again
-  // binary64: e was computed by k_exp into the space of Q; both phases read it
-  constexpr bool PRE_E = sizeof(R) == 8;
-  constexpr bool WB = STAGED && !ESS && !PRE_E;
-  constexpr int TP = BLOCK * PER;  // particles per tile
-  typedef typename ESumT<R>::T ES;
-  __shared__ uint64_t s_warp[WARPS + 1];
-  __shared__ uint64_t s_pre2[WARPS];
-  __shared__ ES s_es[WARPS];
-  __shared__ uint64_t s_bc[2];
-  __shared__ uint32_t s_run[BB_RUNS][3];
-  __shared__ uint32_t s_nruns;
-  // one tile per CTA: the tile's quantised weights and log-ML partials, kept
-  // from phase 1 for phase 2 (the CTA quantises once).  Staged: phase 1 uses
-  // this space as further TMA buffers and phase 2 as the rows of the CDF.
-  __shared__ alignas(128) uint64_t s_keep[BLOCK * (PER + 1)];
-  __shared__ R s_keep_ep[STAGED ? 1 : BLOCK];
-  // staged: l (phase 1) or e (phase 2) of the next tiles arrives by TMA while
-  // the CTA works on the current one; in phase 2 the buffer of the current
-  // tile, once quantised, is the tile's ancestor window (see below)
-  __shared__ alignas(128) R s_ell[2][STAGED ? TP : 4];
-  __shared__ alignas(16) uint16_t s_win[STAGED ? 8 : 2 * TP];
-  // phase 1's ring of NB1 buffers (s_ell[0], s_ell[1], then s_keep), so that
-  // NB1 - 1 tiles are in flight while one is quantised: four 16 KB tiles in
-  // binary32, three 32 KB tiles in binary64; phase 2's ring is s_ell
-  constexpr int NB1 = STAGED ? 2 + (int)(sizeof(uint64_t) * BLOCK * (PER + 1) / (sizeof(R) * TP)) : 1;
-  __shared__ alignas(8) uint64_t s_bar[NB1 + 2];
-  __shared__ uint32_t s_S[2];  // the tile's first slot and the slot after its last
-  __shared__ U128 s_sq[ESS ? WARPS : 1];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  Ctl* c = a.ctl;
-  const uint64_t n = a.n;
-  const uint32_t ntiles = (uint32_t)((n + TP - 1) / TP);
-  const uint32_t per = (ntiles + gridDim.x - 1) / gridDim.x;
-  const uint32_t tb = blockIdx.x * per < ntiles ? blockIdx.x * per : ntiles;
-  const uint32_t te = tb + per < ntiles ? tb + per : ntiles;
-  const uint32_t t = c->t;
-  R m;
-  if constexpr (sizeof(R) == 4) m = dec_f((uint32_t)c->maxenc);
-  else m = dec_d(c->maxenc);
-  const int k = a.k;
-  (void)m;
-  R* const wsrc = PRE_E ? reinterpret_cast<R*>(a.Q) : a.ell;  // l, or e
-  // TMA rings (staged).  Phase 1: the CTA's tile i goes to ring buffer
-  // i % NB1 with barrier i % NB1; phase 2: tile i to s_ell[i & 1] with
-  // barrier NB1 + (i & 1).  The k-th copy through a barrier completes its
-  // phase k, waited for with parity k & 1.
-  // After a wait that gave up (s_tmo set, ERR_TIMEOUT raised) the CTA issues
-  // no more copies and waits for none; its CDF and ancestors are then
-  // invalid, which the error word reports.  Before the CTA exits, thread 0
-  // waits once more, bounded, for every copy it issued that it has not seen
-  // complete, so that no copy into this CTA's shared memory outlives it.
-  __shared__ uint32_t s_tmo;
-  if (threadIdx.x == 0) {
-    s_tmo = 0;
-    if (STAGED) {
-      for (int b = 0; b < NB1 + 2; ++b) mbar_init(&s_bar[b], 1);
-      mbar_init_fence();
-    }
-  }
-  __syncthreads();
-  uint32_t iss_b[NB1 + 2], ok_b[NB1 + 2];  // thread 0: copies issued / seen complete per barrier
-#pragma unroll
-  for (int b = 0; b < NB1 + 2; ++b) iss_b[b] = ok_b[b] = 0;
-  // phase 1's ring buffer b
-  auto ring1 = [&](uint32_t b) -> R* {
-    return b < 2 ? s_ell[b] : reinterpret_cast<R*>(s_keep) + (b - 2) * TP;
-  };
-  // thread 0: copy tile `tile` of l (or e) into dst through barrier bi; dst
-  // is free (any bulk store from it has read it)
-  auto issue = [&](uint32_t bi, R* dst, uint32_t tile) {
-    if (*(volatile uint32_t*)&s_tmo) return;
-    const uint64_t first = (uint64_t)tile * TP;
-    const uint64_t cnt = n - first < (uint64_t)TP ? n - first : (uint64_t)TP;
-    const uint32_t bytes = (uint32_t)((cnt * sizeof(R) + 15) & ~(uint64_t)15);
-    fence_proxy_async_smem();  // (phase 2: the buffer held the previous tile's window)
-    tma_load_1d(dst, wsrc + first, bytes, &s_bar[bi]);
-    ++iss_b[bi];
-  };
-  // every thread: wait for the k-th copy through barrier bi
-  auto take = [&](uint32_t bi, uint32_t k) {
-    if (!*(volatile uint32_t*)&s_tmo) {
-      if (mbar_wait(&s_bar[bi], k & 1)) {
-        if (threadIdx.x == 0) ++ok_b[bi];
-      } else {
-        s_tmo = 1u;
-        atomicOr(&c->err, ERR_TIMEOUT);
-      }
-    }
-  };
-  auto drain_copies = [&]() {  // thread 0, at exit
-    if constexpr (STAGED) {
-      if (!*(volatile uint32_t*)&s_tmo) return;
-      for (int b = 0; b < NB1 + 2; ++b)
-        for (uint32_t k = ok_b[b]; k < iss_b[b]; ++k) (void)mbar_wait(&s_bar[b], k & 1);
-    }
-  };
-  // this thread's 16 weights of tile `tile` quantised, as inclusive running
-  // sums W, the partial sum of e = exp(l - m) and the largest e.  mode 0:
-  // from l in buf; 1: from l in buf (shared memory), writing e back in its
-  // place; 2: from e in buf (written back by phase 1).
-  auto quantP = [&](uint32_t tile, const R* buf, uint64_t* W, R* epart, R* emx, int mode) {
-    R exs[PER];
-    R mx = (R)0;
-    const uint64_t base = (uint64_t)tile * TP + (uint64_t)threadIdx.x * PER;
-    R* const row = const_cast<R*>(buf) + threadIdx.x * PER;
-    const bool full = base + PER <= n;
-    uint64_t run = 0;
-    R ep = (R)0;
-#pragma unroll
-    for (int q = 0; q < PER / 4; ++q) {
-      R v[4];
-      if (full) {
-        if constexpr (sizeof(R) == 4) {
-          const float4 f = *reinterpret_cast<const float4*>(row + 4 * q);
-          v[0] = f.x; v[1] = f.y; v[2] = f.z; v[3] = f.w;
-        } else {
-          const double2 f0 = *reinterpret_cast<const double2*>(row + 4 * q);
-          const double2 f1 = *reinterpret_cast<const double2*>(row + 4 * q + 2);
-          v[0] = f0.x; v[1] = f0.y; v[2] = f1.x; v[3] = f1.y;
-        }
-      } else {
-#pragma unroll
-        for (int e = 0; e < 4; ++e) v[e] = (base + 4 * q + e < n) ? row[4 * q + e] : (R)0;
-      }
-      R ex4[4];
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        uint64_t w = 0;
-        R ex = (R)0;
-        if (full || base + 4 * q + e < n) {
-          if (mode == 2) {
-            ex = v[e];
-            w = quant_from_e(ex, k);
-          } else {
-            const R dl = v[e] - m;
-            w = quant_exp(dl, k, &ex);
-          }
-          ep = ep + ex;
-          mx = pos_less(mx, ex) ? ex : mx;
-        }
-        ex4[e] = ex;
-        exs[4 * q + e] = ex;
-        run += w;
-        W[4 * q + e] = run;  // inclusive running sum
-      }
-      if (mode == 1) {
-        if constexpr (sizeof(R) == 4) {
-          *reinterpret_cast<float4*>(row + 4 * q) = make_float4(ex4[0], ex4[1], ex4[2], ex4[3]);
-        } else {
-          *reinterpret_cast<double2*>(row + 4 * q) = make_double2(ex4[0], ex4[1]);
-          *reinterpret_cast<double2*>(row + 4 * q + 2) = make_double2(ex4[2], ex4[3]);
-        }
-      }
-    }
-    if constexpr (PER == 8) {
-      // the log-ML partials are sums over 16 consecutive particles in
-      // order: the odd lane continues the even lane's sum over its own 8
-      const R prev = __shfl_xor_sync(0xffffffffu, ep, 1);
-      R acc = prev;
-#pragma unroll
-      for (int e = 0; e < PER; ++e) acc = acc + exs[e];  // e = 0 past n: adds nothing
-      ep = (threadIdx.x & 1) ? acc : (R)0;
-    }
-    *epart = ep;
-    *emx = mx;
-  };
-  // block sum of one value per thread, returned to every thread
-  auto block_sum = [&](uint64_t v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane == 0) s_warp[warp] = v;
-    __syncthreads();
-    uint64_t tot = 0;
-    for (int w = 0; w < WARPS; ++w) tot += s_warp[w];
-    __syncthreads();
-    return tot;
-  };
-
-  // block sum of one 128-bit value per thread, returned to every thread
-  auto block_sum128 = [&](U128 v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      U128 u;
-      u.hi = __shfl_xor_sync(0xffffffffu, v.hi, o);
-      u.lo = __shfl_xor_sync(0xffffffffu, v.lo, o);
-      v = add128(v, u);
-    }
-    if (lane == 0) s_sq[warp] = v;
-    __syncthreads();
-    U128 tot{0, 0};
-    for (int w = 0; w < WARPS; ++w) tot = add128(tot, s_sq[w]);
-    __syncthreads();
-    return tot;
-  };
-
-  // phase 1: this CTA's sum of W (and with ESS of W^2)
-  uint64_t mine = 0;
-  R emx_keep = (R)0;
-  U128 sq{0, 0};
-  auto add_sq = [&](const uint64_t* W) {
-    if constexpr (ESS) {
-      uint64_t prev = 0;
-#pragma unroll
-      for (int e = 0; e < PER; ++e) {
-        const uint64_t w = W[e] - prev;
-        prev = W[e];
-        sq = add128(sq, mul64(w, w));
-      }
-    }
-  };
-  if constexpr (STAGED) {
-    if (threadIdx.x == 0)
-      for (uint32_t b = 0; b + 1 < (uint32_t)NB1 && tb + b < te; ++b) issue(b, ring1(b), tb + b);
-    uint32_t i = 0;
-    for (uint32_t tile = tb; tile < te; ++tile, ++i) {
-      const uint32_t b = i % NB1;
-      R* const buf = ring1(b);
-      take(b, i / NB1);
-      uint64_t W[PER];
-      R ep;
-      // (with ESS l stays in place: a propagation that does not resample
-      // carries L - m from it, so phase 2 quantises from l again)
-      R emx;
-      quantP(tile, buf, W, &ep, &emx, PRE_E ? 2 : (WB ? 1 : 0));
-      if (WB) fence_proxy_async_smem();  // e in buf, for the bulk store below
-      mine += W[PER - 1];
-      add_sq(W);
-      __syncthreads();
-      if (threadIdx.x == 0) {
-        if (WB) {
-          // e goes back to l's place in global memory for phase 2, which
-          // then needs no exponentials
-          const uint64_t first = (uint64_t)tile * TP;
-          const uint64_t cnt = n - first < (uint64_t)TP ? n - first : (uint64_t)TP;
-          tma_store_1d(a.ell + first, buf, (uint32_t)((cnt * sizeof(R) + 15) & ~(uint64_t)15));
-        }
-        if (tile + NB1 - 1 < te) {
-          // the previous tile's buffer takes the tile NB1 - 1 ahead, once
-          // its bulk store has read it (this tile's may still be reading)
-          if (WB) bulk_wait_read1();
-          const uint32_t nb = (i + NB1 - 1) % NB1;
-          issue(nb, ring1(nb), tile + NB1 - 1);
-        }
-      }
-    }
-  } else {
-    // at most one tile: l read directly, its W (and this thread's largest e)
-    // kept for phase 2
-    for (uint32_t tile = tb; tile < te; ++tile) {
-      uint64_t W[PER];
-      R ep;
-      quantP(tile, wsrc + (uint64_t)tile * TP, W, &ep, &emx_keep, PRE_E ? 2 : 0);
-      mine += W[PER - 1];
-      add_sq(W);
-#pragma unroll
-      for (int e = 0; e < PER; ++e) s_keep[threadIdx.x * (PER + 1) + e] = W[e];
-      s_keep_ep[threadIdx.x] = ep;
-    }
-  }
-  mine = block_sum(mine);
-  if constexpr (ESS) sq = block_sum128(sq);
-  if (threadIdx.x == 0) {
-    st_status(&cta_tot[blockIdx.x], mine);
-    if constexpr (ESS) {
-      st_status(&cta_sq[blockIdx.x].hi, sq.hi);
-      st_status(&cta_sq[blockIdx.x].lo, sq.lo);
-    }
-    __threadfence();
-    atomicAdd(&c->gbar, 1u);
-    if (STAGED && tb < te) {  // phase 2's first tile from HBM: e stored, complete
-      bulk_wait_done();
-      issue(NB1, s_ell[0], tb);
-    }
-    uint32_t spins = 0;
-    while (ld_volatile_u32(&c->gbar) < gridDim.x) {
-      if (++spins > SPIN_LIMIT) {
-        atomicOr(&c->err, ERR_TIMEOUT);
-        break;
-      }
-      __nanosleep(64);
-    }
-    __threadfence();
-  }
-  __syncthreads();
-
-  // phase 2: this CTA's exclusive prefix and the total T
-  uint64_t pre = 0, all = 0;
-  for (uint32_t b = threadIdx.x; b < gridDim.x; b += BLOCK) {
-    const uint64_t v = ld_status(&cta_tot[b]);
-    all += v;
-    if (b < blockIdx.x) pre += v;
-  }
-  // both block sums in one pass (two block barriers)
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    pre += __shfl_xor_sync(0xffffffffu, pre, o);
-    all += __shfl_xor_sync(0xffffffffu, all, o);
-  }
-  if (lane == 0) {
-    s_warp[warp] = pre;
-    s_pre2[warp] = all;
-  }
-  __syncthreads();
-  pre = 0;
-  uint64_t T = 0;
-  for (int w = 0; w < WARPS; ++w) {
-    pre += s_warp[w];
-    T += s_pre2[w];
-  }
-  __syncthreads();
-  // adaptive resampling: the decision of k_ess, from the same exact sums
-  bool rs = true;
-  if constexpr (ESS) {
-    U128 B{0, 0};
-    for (uint32_t b = threadIdx.x; b < gridDim.x; b += BLOCK) {
-      U128 v;
-      v.hi = ld_status(&cta_sq[b].hi);
-      v.lo = ld_status(&cta_sq[b].lo);
-      B = add128(B, v);
-    }
-    B = block_sum128(B);
-    const double A = __ull2double_rn(T);
-    const double Bd = u128_to_f64_rn(B);
-    const double lhs = A * A;
-    const double f = a.ess_frac * (double)n;
-    const double rhs = f * Bd;
-    rs = lhs < rhs;
-    if (blockIdx.x == 0 && threadIdx.x == 0) c->resamp = rs ? 1u : 0u;
-  }
-  const U4 wr = draw(a.seed, a.filter, t, 0, P_SYS_OFFSET, 0);
-  const uint64_t r = __umul64hi(((uint64_t)wr.b << 32) | wr.a, T);
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    c->keyT = T;
-    c->keyA = n;
-    c->keyR = r;
-    if (T == 0) atomicOr(&c->err, ERR_NUMERIC);
-  }
-  const SysDiv dv = make_sysdiv(T > 0 ? T : 1);
-  // a particle with n W_i <= 2 T owns at most two slots, and e_i <= thr
-  // implies it: W_i <= e_i 2^k <= thr 2^k <= 2 T / n, every rounding of
-  // thr = T (1 / n) 2^(1 - k) taken downward
-  R thr;
-  if constexpr (sizeof(R) == 4)
-    thr = __fmul_rd(__fmul_rd(__ull2float_rd(T), __frcp_rd(__ull2float_ru(n))), pow2f(1 - k));
-  else
-    thr = __dmul_rd(__dmul_rd(__ull2double_rd(T), __drcp_rd((double)n)), pow2d(1 - k));
-  if (threadIdx.x == 0) s_nruns = 0;
-  __syncthreads();
-  uint64_t carry = pre;
-  uint32_t i2 = 0;
-  // the log-ML partial of the CTA's tiles (thread 0)
-  constexpr bool CTA_PART = STAGED && sizeof(R) == 4;
-  ES cta_es;
-  cta_es.zero();
-  for (uint32_t tile = tb; tile < te; ++tile, ++i2) {
-    uint64_t W[PER];
-    R ep, emx = emx_keep;
-    if constexpr (!STAGED) {  // this thread's own entries: no barrier needed
-#pragma unroll
-      for (int e = 0; e < PER; ++e) W[e] = s_keep[threadIdx.x * (PER + 1) + e];
-      ep = s_keep_ep[threadIdx.x];
-    } else {
-      // the next tile into the other buffer (the previous tile's window,
-      // stored out), then this one
-      if (threadIdx.x == 0 && tile + 1 < te) issue(NB1 + ((i2 + 1) & 1), s_ell[(i2 + 1) & 1], tile + 1);
-      take(NB1 + (i2 & 1), i2 >> 1);
-      quantP(tile, s_ell[i2 & 1], W, &ep, &emx, (WB || PRE_E) ? 2 : 0);
-    }
-    // the tile's first slot S0 = R(carry)
-    // (a later tile starts where the previous one ended: no division)
-    if (threadIdx.x == 0) s_S[0] = tile == tb ? (uint32_t)sys_first_slot(carry, n, r, dv) : s_S[1];
-    // The ancestors of the tile's slots [S0, S1) are built in a shared-memory
-    // window of one 16-bit entry per slot (a free l buffer when staged), at
-    // least two per particle of the tile, then stored out coalesced.
-    constexpr uint32_t WIN_SLOTS = STAGED ? TP * sizeof(R) / 2 : 2 * TP;
-    static_assert(WIN_SLOTS % 512 == 0 && WIN_SLOTS >= 2 * TP, "window");
-    uint16_t* const win = STAGED ? reinterpret_cast<uint16_t*>(s_ell[i2 & 1]) : s_win;
-    {
-      ES es;
-      es.zero();
-      es.add(ep);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) es.add(es.shfl_xor(o));
-      if (lane == 0) s_es[warp] = es;
-    }
-    // block exclusive scan of the thread totals
-    const uint64_t tt = W[PER - 1];
-    const uint64_t incl = warp_incl_scan(tt, lane);
-    if (lane == 31) s_warp[warp] = incl;
-    __syncthreads();
-    if (warp == 0) {
-      const uint64_t wt = lane < WARPS ? s_warp[lane] : 0;
-      const uint64_t wi = warp_incl_scan(wt, lane);
-      if (lane < WARPS) s_warp[lane] = wi - wt;
-      if (lane == WARPS - 1) s_bc[0] = wi;
-      if (lane == 0) {
-        ES tot = s_es[0];
-        for (int w = 1; w < WARPS; ++w) tot.add(s_es[w]);
-        // staged binary32: one exact partial per CTA (the sum of its tiles'),
-        // so that the propagation's final fold reads one per CTA
-        if constexpr (CTA_PART) cta_es.add(tot);
-        else reinterpret_cast<ES*>(a.part)[tile] = tot;
-      }
-    }
-    __syncthreads();
-    const uint64_t o = carry + s_warp[warp] + (incl - tt);  // Q just before this thread's particles
-    const uint64_t tile_tot = s_bc[0];
-    const uint64_t tbase = (uint64_t)tile * TP;
-    const uint64_t base = tbase + (uint64_t)threadIdx.x * PER;
-    const uint32_t S0 = s_S[0];
-    const uint32_t S0a = S0 & ~3u;  // the window's base: slots in aligned groups of four
-    // The CDF: this thread's values go to its shared-memory row (read by the
-    // resampling step below); staged (several tiles per CTA, where the store
-    // instructions add up) the rows are written out coalesced below,
-    // otherwise the values are stored directly.
-    uint64_t* const qrow = s_keep + threadIdx.x * (PER + 1);
-#pragma unroll
-    for (int e = 0; e < PER; ++e) qrow[e] = o + W[e];
-    if constexpr (!STAGED) {
-      if (base + PER <= n) {
-#pragma unroll
-        for (int e = 0; e < PER; e += 2)
-          *reinterpret_cast<ulonglong2*>(a.Q + base + e) = make_ulonglong2(o + W[e], o + W[e + 1]);
-      } else {
-#pragma unroll
-        for (int e = 0; e < PER; ++e)
-          if (base + e < n) a.Q[base + e] = o + W[e];
-      }
-    }
-    // Systematic resampling, one step per particle: with D = n Q_i - (j T + r)
-    // for particle i and its first slot j, i owns the c = ceil(D / T) slots
-    // j .. j + c - 1 (none if D <= 0); D then drops by c T into (-T, 0] and
-    // the next particle adds n w_{i+1} <= n 2^k <= 2^61 (T <= 2^61 too), so
-    // D is an int64.  A particle writes its offset in the tile + 1 into the
-    // window entries of its slots: the first three by predicated stores, any
-    // others (a heavy particle) and slots past the window out of line, in
-    // runs of the CTA when long.  c comes from three comparisons unless it is
-    // above 3 (a heavy particle, divided out): no branch for up to three slots,
-    // which covers all but a few particles in a hundred even when an outlying
-    // observation concentrates the weights.  Every slot of [S0, S1) is
-    // written exactly once, so the window needs no clearing.  A rolled loop
-    // over the row: the step's code stays small.
-    // a warp none of whose particles can own more than two slots takes the
-    // lean step; any other warp counts up to three slots without a branch
-    const bool light = !__any_sync(0xffffffffu, emx > thr);
-    if (rs && T > 0 && base < n) {
-      const uint32_t ecount = base + PER <= n ? (uint32_t)PER : (uint32_t)(n - base);
-      uint32_t j = threadIdx.x == 0 ? S0 : (base == 0 ? 0u : (uint32_t)sys_first_slot(o, n, r, dv));
-      const U128 X = mul64x32(o, (uint32_t)n);
-      const U128 KB = add128(mul64x32(T, j), r);
-      int64_t D = (int64_t)(X.lo - KB.lo);  // n Q - (j T + r) just before this thread's particles
-      const int64_t Ti = (int64_t)T, T2 = 2 * Ti, T3 = 3 * Ti;
-      const uint32_t off0 = (uint32_t)(base - tbase) + 1u;
-      const uint32_t n32 = (uint32_t)n;
-      uint64_t qprev = o;
-      if (light) {
-#pragma unroll 1
-        for (uint32_t e = 0; e < ecount; ++e) {
-          const uint64_t q = qrow[e];
-          const uint64_t w = q - qprev;
-          D += (int64_t)((uint64_t)(uint32_t)w * n32 + (((w >> 32) * n32) << 32));  // w n mod 2^64
-          qprev = q;
-          const uint32_t c = (uint32_t)(D > 0) + (uint32_t)(D > Ti);
-          const uint16_t mk = (uint16_t)(off0 + e);
-          const uint32_t x = j - S0a;
-          if (c >= 1u && x < WIN_SLOTS) win[win_entry(x)] = mk;
-          if (c >= 2u && x + 1u < WIN_SLOTS) win[win_entry(x + 1u)] = mk;
-          if (x + c > WIN_SLOTS)
-            sys_rest(j, c, S0a, WIN_SLOTS, mk, (uint32_t)base + e, win, a.anc, s_run, &s_nruns, 2u);
-          D -= c == 1u ? Ti : (int64_t)c * Ti;
-          j += c;
-        }
-      } else {
-#pragma unroll 1
-      for (uint32_t e = 0; e < ecount; ++e) {
-        const uint64_t q = qrow[e];
-        const uint64_t w = q - qprev;
-        D += (int64_t)((uint64_t)(uint32_t)w * n32 + (((w >> 32) * n32) << 32));  // w n mod 2^64
-        qprev = q;
-        uint32_t c = (uint32_t)(D > 0) + (uint32_t)(D > Ti) + (uint32_t)(D > T2);
-        if (D > T3) c = sys_heavy_count(D, dv);
-        const uint16_t mk = (uint16_t)(off0 + e);
-        const uint32_t x = j - S0a;
-        if (c >= 1u && x < WIN_SLOTS) win[win_entry(x)] = mk;
-        if (c >= 2u && x + 1u < WIN_SLOTS) win[win_entry(x + 1u)] = mk;
-        if (c >= 3u && x + 2u < WIN_SLOTS) win[win_entry(x + 2u)] = mk;
-        if (c > 3u || x + c > WIN_SLOTS)
-          sys_rest(j, c, S0a, WIN_SLOTS, mk, (uint32_t)base + e, win, a.anc, s_run, &s_nruns, 3u);
-        D -= c == 1u ? Ti : (int64_t)c * Ti;
-        j += c;
-      }
-      }
-      if (base + PER >= n || threadIdx.x == BLOCK - 1) s_S[1] = j;  // the tile's end slot
-    }
-    __syncthreads();
-    // window runs of heavy particles, by the whole CTA
-    const uint32_t nr = s_nruns < BB_RUNS ? s_nruns : BB_RUNS;
-    bool wr = false;
-    for (uint32_t q = 0; q < nr; ++q) {
-      const uint32_t v = s_run[q][2];
-      if (!(v & WRUN)) continue;
-      wr = true;
-      for (uint32_t x = s_run[q][0] + threadIdx.x; x < s_run[q][1]; x += BLOCK)
-        win[win_entry(x)] = (uint16_t)v;
-    }
-    if (wr) __syncthreads();  // (wr is the same in every thread)
-    if constexpr (STAGED) {  // the CDF rows, written out coalesced
-      const uint64_t tcnt = n - tbase < (uint64_t)TP ? n - tbase : (uint64_t)TP;
-      for (uint32_t p = 2 * threadIdx.x; p < tcnt; p += 2 * BLOCK) {
-        const uint64_t q0 = s_keep[(p / PER) * (PER + 1) + (p % PER)];
-        if (p + 1 < tcnt) {
-          const uint64_t q1 = s_keep[(p / PER) * (PER + 1) + (p % PER) + 1];
-          *reinterpret_cast<ulonglong2*>(a.Q + tbase + p) = make_ulonglong2(q0, q1);
-        } else {
-          a.Q[tbase + p] = q0;
-        }
-      }
-    }
-    // the window's slots [S0, wend), stored out coalesced, four per 16-byte
-    // store (the partial groups at either end slot by slot)
-    {
-      const uint32_t S1 = s_S[1];
-      const uint32_t wend = (rs && T > 0) ? (S1 - S0a < WIN_SLOTS ? S1 : S0a + WIN_SLOTS) : S0;
-      const uint32_t tb32 = (uint32_t)tbase - 1u;
-      const uint32_t ng = wend > S0 ? (wend - S0a + 3u) >> 2 : 0u;
-      for (uint32_t g = threadIdx.x; g < ng; g += BLOCK) {
-        const uint32_t x0 = g << 2;
-        const uint32_t sw = ((x0 >> 6) & 7u) << 1;
-        const uint2 v = *reinterpret_cast<const uint2*>(win + (x0 ^ (sw & 12u)));
-        const uint32_t lo = (sw & 2u) ? v.y : v.x, hi = (sw & 2u) ? v.x : v.y;
-        const uint32_t slot = S0a + x0;
-        const uint4 o4 = make_uint4(tb32 + (lo & 0xffffu), tb32 + (lo >> 16), tb32 + (hi & 0xffffu),
-                                    tb32 + (hi >> 16));
-        if (slot >= S0 && slot + 4u <= wend) {
-          *reinterpret_cast<uint4*>(a.anc + slot) = o4;
-        } else {
-          if (slot >= S0 && slot < wend) a.anc[slot] = o4.x;
-          if (slot + 1u >= S0 && slot + 1u < wend) a.anc[slot + 1u] = o4.y;
-          if (slot + 2u >= S0 && slot + 2u < wend) a.anc[slot + 2u] = o4.z;
-          if (slot + 3u >= S0 && slot + 3u < wend) a.anc[slot + 3u] = o4.w;
-        }
-      }
-    }
-    // runs past the window, by the whole CTA
-    for (uint32_t q = 0; q < nr; ++q) {
-      const uint32_t st = s_run[q][0], en = s_run[q][1], v = s_run[q][2];
-      if (v & WRUN) continue;
-      for (uint32_t jj = st + threadIdx.x; jj < en; jj += BLOCK) a.anc[jj] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) s_nruns = 0;
-    carry += tile_tot;
-  }
-  if (CTA_PART && threadIdx.x == 0) reinterpret_cast<ES*>(a.part)[blockIdx.x] = cta_es;
-  if (T == 0) {  // empty CDF (flagged): keep every index in range
-    for (uint64_t j = (uint64_t)blockIdx.x * BLOCK + threadIdx.x; j < n;
-         j += (uint64_t)gridDim.x * BLOCK)
-      a.anc[j] = (uint32_t)j;
-  }
-  if (STAGED && threadIdx.x == 0) {
-    drain_copies();
-    bulk_wait_done();
-  }
-}
+}  // namespace pfk
+#include "slots.cuh"
+namespace pfk {
 
 // ---------------------------------------------------------------------------
 // Steps 2-4: propagate x, update the sufficient statistics, draw theta.
@@ -2105,89 +1223,6 @@ __device__ __forceinline__ double esum_value(const ESum32& e) {
   return __ull2double_rn(e.s.hi) * 0x1p-32 + __ull2double_rn(e.s.lo) * 0x1p-96;
 }
 __device__ __forceinline__ double esum_value(const ESum64& e) { return e.s; }
-
-// ---------------------------------------------------------------------------
-// Adaptive resampling decision (not in the paper, which resamples every
-// cycle): ESS = (sum W)^2 / sum W^2 of the quantised weights against
-// ess_frac * n (Kong, Liu & Wong 1994).  sum W^2 is summed exactly in 128
-// bits from the finished CDF (W_i = Q_i - Q_{i-1}); sum W = Q_{n-1}.  The
-// comparison is A * A < (ess_frac * n) * B in binary64, A and B the two sums
-// each rounded to nearest once.  The last block writes the decision.
-// ---------------------------------------------------------------------------
-constexpr int ESS_PER_THREAD = 8;
-
-template <class R>
-__global__ void __launch_bounds__(BLOCK) k_ess(FilterArgs<R> a) {
-  __shared__ U128 s_red[WARPS];
-  __shared__ bool s_last;
-  const uint64_t n = a.n;
-  U128 acc{0, 0};
-  const uint64_t stride = (uint64_t)gridDim.x * BLOCK;
-  // ESS_PER_THREAD strided elements per pass, their loads issued together
-  for (uint64_t i0 = (uint64_t)blockIdx.x * BLOCK + threadIdx.x; i0 < n;
-       i0 += stride * ESS_PER_THREAD) {
-    uint64_t q[ESS_PER_THREAD], qp[ESS_PER_THREAD];
-#pragma unroll
-    for (int e = 0; e < ESS_PER_THREAD; ++e) {
-      const uint64_t i = i0 + (uint64_t)e * stride;
-      q[e] = i < n ? a.Q[i] : 0ull;
-      qp[e] = (i < n && i > 0) ? a.Q[i - 1] : 0ull;
-    }
-#pragma unroll
-    for (int e = 0; e < ESS_PER_THREAD; ++e) {
-      const uint64_t W = q[e] - qp[e];
-      acc = add128(acc, mul64(W, W));
-    }
-  }
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    U128 v;
-    v.hi = __shfl_xor_sync(0xffffffffu, acc.hi, o);
-    v.lo = __shfl_xor_sync(0xffffffffu, acc.lo, o);
-    acc = add128(acc, v);
-  }
-  if (lane == 0) s_red[warp] = acc;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    U128 b = s_red[0];
-    for (int w = 1; w < WARPS; ++w) b = add128(b, s_red[w]);
-    a.ess_part[blockIdx.x] = b;
-    __threadfence();
-    s_last = atomicAdd(&a.ctl->done_ess, 1u) == gridDim.x - 1;
-  }
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-  // fold the block partials across the block: an exact integer sum, so the
-  // order does not matter
-  U128 B{0, 0};
-  for (uint32_t b = threadIdx.x; b < gridDim.x; b += BLOCK) {
-    U128 v;
-    v.hi = __ldcg(&a.ess_part[b].hi);
-    v.lo = __ldcg(&a.ess_part[b].lo);
-    B = add128(B, v);
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    U128 v;
-    v.hi = __shfl_xor_sync(0xffffffffu, B.hi, o);
-    v.lo = __shfl_xor_sync(0xffffffffu, B.lo, o);
-    B = add128(B, v);
-  }
-  if (lane == 0) s_red[warp] = B;
-  __syncthreads();
-  if (threadIdx.x != 0) return;
-  B = s_red[0];
-  for (int w = 1; w < WARPS; ++w) B = add128(B, s_red[w]);
-  const double A = __ull2double_rn(a.Q[n - 1]);
-  const double Bd = u128_to_f64_rn(B);
-  const double lhs = A * A;
-  const double f = a.ess_frac * (double)n;
-  const double rhs = f * Bd;
-  a.ctl->resamp = lhs < rhs ? 1u : 0u;
-  a.ctl->done_ess = 0;
-}
 
 // Run by the last warp of k_propagate: fold the per-tile log-ML partials
 // (lane-strided, then butterfly: a fixed order), accumulate the increment
@@ -2255,7 +1290,6 @@ __device__ void fold_cycle_warp(const FilterArgs<R>& a, uint32_t t) {
     c->ticket_w = 0;
     c->ticket_e = 0;
     c->done_prop = 0;
-    c->gbar = 0;
     c->prop_ticket = 0;
     c->w_ticket = 0;
     __threadfence();
@@ -3093,7 +2127,7 @@ __global__ void __launch_bounds__(SMALL_THREADS) k_resample_small(const float* w
   for (int e = 0; e < SMALL_PER; ++e) {
     v[e] = ((uint32_t)e < per && base + e < n) ? w[base + e] : 0.0f;
     if (!(v[e] >= 0.0f) || !(v[e] < INFINITY)) bad = true;
-    else mx = max(mx, __float_as_uint(v[e]));
+    else mx = max(mx, __float_as_uint(fabsf(v[e])));  // (-0 is a zero weight)
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
@@ -3182,17 +2216,31 @@ __global__ void __launch_bounds__(SMALL_THREADS) k_resample_small(const float* w
 }
 
 // Maximum of binary32 input weights (pf_resample): non-negative floats order
-// as their bit patterns.
-static __global__ void __launch_bounds__(BLOCK) k_wmax(const float* w, uint64_t n, Ctl* ctl) {
+// as their bit patterns (-0 is a zero weight).  With vec, 32-byte aligned w: a
+// thread's eight weights per load, two loads in flight.
+static __global__ void __launch_bounds__(BLOCK) k_wmax(const float* w, uint64_t n, Ctl* ctl, int vec) {
   __shared__ uint32_t s_red[WARPS];
   uint32_t mx = 0;
   bool bad = false;
-  for (uint64_t i = (uint64_t)blockIdx.x * BLOCK + threadIdx.x; i < n;
-       i += (uint64_t)gridDim.x * BLOCK) {
-    const float v = w[i];
+  auto take = [&](float v) {
     if (!(v >= 0.0f) || !(v < INFINITY)) bad = true;
-    else mx = max(mx, __float_as_uint(v));
+    else mx = max(mx, __float_as_uint(fabsf(v)));
+  };
+  const uint64_t nt = (uint64_t)gridDim.x * BLOCK, id = (uint64_t)blockIdx.x * BLOCK + threadIdx.x;
+  const uint64_t n8 = vec ? n / 8 : 0;
+  for (uint64_t i = id; i < n8; i += 2 * nt) {
+    float v[16];
+    const bool two = i + nt < n8;
+    ld8(w + 8 * i, v);
+    if (two) ld8(w + 8 * (i + nt), v + 8);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) take(v[e]);
+    if (two) {
+#pragma unroll
+      for (int e = 8; e < 16; ++e) take(v[e]);
+    }
   }
+  for (uint64_t i = 8 * n8 + id; i < n; i += nt) take(w[i]);
   if (bad) atomicOr(&ctl->err, ERR_WEIGHTS);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
