@@ -183,7 +183,7 @@ struct BatchSmem {
   typedef typename ESumT<R>::T ES;
   uint64_t warp[NT / 32 + 1];
   R red[NT / 32];
-  ES es[NT / 32];
+  ES es[2][NT / 32];             // by round parity: thread 0 reads a round's while others write the next's
   ES fold[32];                   // log-ML tile partials, lane-strided (group rank 0)
   uint32_t run[BB_MAX_RUNS][3];
   GammaItem<R> wq[NT / 32][WQ_CAP];   // per-warp queues of deferred gamma draws
@@ -373,7 +373,7 @@ __device__ __forceinline__ void batch_filter(const BatchArgs<R>& a, const BatchI
       es.add(epart);
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) es.add(es.shfl_xor(o));
-      if (lane == 0) sm.es[warp] = es;
+      if (lane == 0) sm.es[par][warp] = es;
     }
     uint64_t total;
     const uint64_t excl = block_excl_scan<NW>(run, sm.warp, &total);  // its barriers publish sm.es
@@ -381,8 +381,8 @@ __device__ __forceinline__ void batch_filter(const BatchArgs<R>& a, const BatchI
       // each tile's partial: its 8 warps in order
 #pragma unroll
       for (int tp = 0; tp < TPP; ++tp) {
-        ES tot = sm.es[tp * WARPS];
-        for (int q = 1; q < WARPS; ++q) tot.add(sm.es[tp * WARPS + q]);
+        ES tot = sm.es[par][tp * WARPS];
+        for (int q = 1; q < WARPS; ++q) tot.add(sm.es[par][tp * WARPS + q]);
         sm.ues[par][tp] = tot;
       }
     }
