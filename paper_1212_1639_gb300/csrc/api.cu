@@ -17,6 +17,7 @@
 #include "../../include/pf.h"
 #include "../../include/pf_diag.h"
 #include "kernels.cuh"
+#include "small.cuh"
 
 using namespace pfk;
 
@@ -102,6 +103,7 @@ struct pf_filter {
   int scheme = 0;
   unsigned prop_grid = 0;  // persistent propagate grid
   unsigned exp_grid = 0;   // binary64: grid of k_exp
+  bool small = false;      // whole cycles by one cluster (k_small)
   uint64_t w_cap = 1;      // resident CTAs of the weights kernel
   unsigned prop_grid_fuse = 0;  // the same for the propagation that also weighs
   bool bootstrap = false;   // Algorithm "Particle Filtering" instead of particle learning
@@ -539,6 +541,72 @@ void set_obs(unsigned char* args, bool next, const double* src, double val) {
   }
 }
 
+// Largest filters whose cycles run in one cluster launch (k_small), where that
+// is the faster (small.cuh has both sides' times): binary32 as many as the
+// cluster holds, binary64 half of that.
+constexpr uint64_t SMALL_N32 = (uint64_t)SMALL_M * SMALL_GMAX;
+constexpr uint64_t SMALL_N64 = SMALL_N32 / 2;
+
+template <class R>
+void small_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr, cudaStream_t s) {
+  std::memset(cfg, 0, sizeof(*cfg));
+  cfg->gridDim = dim3(SMALL_GMAX, 1, 1);
+  cfg->blockDim = dim3(BLOCK, 1, 1);
+  cfg->stream = s;
+  attr->id = cudaLaunchAttributeClusterDimension;
+  attr->val.clusterDim.x = SMALL_GMAX;
+  attr->val.clusterDim.y = 1;
+  attr->val.clusterDim.z = 1;
+  cfg->attrs = attr;
+  cfg->numAttrs = 1;
+}
+template <class R>
+bool small_fits() {
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr[1];
+  small_config<R>(&cfg, attr, nullptr);
+  int clusters = 0;
+  if (cudaOccupancyMaxActiveClusters(&clusters, k_small<R>, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return clusters >= 1;
+}
+
+// `steps` cycles of a small filter in one launch (steps <= SMALL_Y for host
+// observations y); with est the summaries follow the last cycle.
+template <class R>
+pf_status launch_small(pf_filter* f, const double* y_dev, const double* y, uint32_t steps, bool est) {
+  FilterArgs<R> a = filter_args<R>(f);
+  SmallArgs sa;
+  std::memset(&sa, 0, sizeof(sa));
+  sa.pos = is_multinomial(f->scheme) ? SP_MULTI : f->scheme == PF_STRATIFIED ? SP_STRAT : SP_SYS;
+  sa.learn = f->learn;
+  sa.ess = f->ess;
+  sa.est = est && !f->ess;
+  sa.m = (uint32_t)(cdiv(cdiv(f->n, SMALL_GMAX), 32) * 32);
+  sa.steps = steps;
+  sa.ess_frac = f->cfg.ess_frac;
+  sa.y_dev = y_dev;
+  if (!y_dev) std::memcpy(sa.y, y, steps * sizeof(double));
+  if (est) a.io = f->io_dev;
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr[1];
+  small_config<R>(&cfg, attr, f->stream);
+  CK(cudaLaunchKernelEx(&cfg, k_small<R>, a, sa));
+  if (est && f->ess) {
+    k_estimate_w<R><<<(unsigned)cdiv(f->n, (uint64_t)BLOCK * EST_PER_THREAD), BLOCK, 0, f->stream>>>(a);
+    CK(cudaGetLastError());
+  }
+  if (est && !a.ctl_mirror)
+    CK(cudaMemcpyAsync(f->ctl_host, f->ctl, offsetof(Ctl, y), cudaMemcpyDeviceToHost, f->stream));
+  return PF_OK;
+}
+pf_status launch_small(pf_filter* f, const double* y_dev, const double* y, uint32_t steps, bool est) {
+  return f->fp64 ? launch_small<double>(f, y_dev, y, steps, est)
+                 : launch_small<float>(f, y_dev, y, steps, est);
+}
+
 // One cycle of the given form: its graph (captured on first use), with this
 // cycle's observation in the weights node and the next one in the fused
 // propagation node.
@@ -547,6 +615,8 @@ pf_status launch_cycle(pf_filter* f, const double* y_src, double y_val, int form
   // the bootstrap filter's weights follow its own blind propagation;
   // adaptive resampling carries weights the fused propagation does not add
   if ((f->bootstrap || f->ess) && form != CF_EST) form = CF_PLAIN;
+  if (f->small && (form == CF_PLAIN || form == CF_EST))
+    return launch_small(f, y_src, &y_val, 1, form == CF_EST);
   CycleGraph& G = f->cg[form];
   if (!G.exec) {
     pf_status st = build_graph(f, form);
@@ -759,7 +829,9 @@ pf_status pf_create(const pf_config* cfg, pf_filter** out) {
     f->w_cap = (uint64_t)per_sm_w * (uint64_t)sms;
     f->prop_grid_fuse = (unsigned)(want < cap_f ? want : cap_f);
   }
-  if ((st = build_graph(f, CF_PLAIN)) != PF_OK) return bail(st);
+  f->small = !f->bootstrap && n <= (f->fp64 ? SMALL_N64 : SMALL_N32) &&
+             (f->fp64 ? small_fits<double>() : small_fits<float>());
+  if (!f->small && (st = build_graph(f, CF_PLAIN)) != PF_OK) return bail(st);
   *out = f;
   return PF_OK;
 }
@@ -806,8 +878,17 @@ pf_status pf_run(pf_filter* f, const double* y, uint32_t n_steps) {
     dev = attr.type == cudaMemoryTypeDevice || attr.type == cudaMemoryTypeManaged;
   cudaGetLastError();
   if (!dev) {
-    for (uint32_t i = 0; i < n_steps; ++i)
-      if ((st = pf_step(f, y[i])) != PF_OK) return st;
+    uint32_t i = 0;
+    if (f->ahead && n_steps && (st = pf_step(f, y[i++])) != PF_OK) return st;
+    for (uint32_t k; i < n_steps; i += k) {
+      k = 1;
+      if (f->small) {  // several cycles per launch
+        k = n_steps - i < SMALL_Y ? n_steps - i : SMALL_Y;
+        if ((st = launch_small(f, nullptr, y + i, k, false)) != PF_OK) return f->sticky = st;
+      } else if ((st = pf_step(f, y[i])) != PF_OK) {
+        return st;
+      }
+    }
     return PF_OK;
   }
   // device-resident observations cannot be compared with an announced one
@@ -815,8 +896,15 @@ pf_status pf_run(pf_filter* f, const double* y, uint32_t n_steps) {
     return set_err(PF_ERR_INVALID,
                    "pf_run with device-resident observations after pf_step_ahead: pass the "
                    "announced observation to pf_step first");
-  for (uint32_t i = 0; i < n_steps; ++i)
-    if ((st = launch_cycle(f, y + i, 0.0)) != PF_OK) return f->sticky = st;
+  for (uint32_t i = 0, k; i < n_steps; i += k) {
+    k = 1;
+    if (f->small) {
+      k = n_steps - i < 1024u ? n_steps - i : 1024u;  // (a bounded kernel)
+      if ((st = launch_small(f, y + i, nullptr, k, false)) != PF_OK) return f->sticky = st;
+    } else if ((st = launch_cycle(f, y + i, 0.0)) != PF_OK) {
+      return f->sticky = st;
+    }
+  }
   return PF_OK;
 }
 

@@ -23,6 +23,7 @@
 // filter with the same configuration bit for bit.
 #pragma once
 #include "kernels.cuh"
+#include "small.cuh"
 
 namespace pfk {
 
@@ -137,11 +138,6 @@ __device__ __forceinline__ uint64_t multi_first_slot(const uint64_t* S, uint64_t
 // shared memory and meet at cluster barriers (release / acquire at cluster
 // scope, which also orders their global-memory writes).
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t cluster_ctarank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
 // Barrier over the G CTAs processing one filter (G = 1: the CTA itself).
 __device__ __forceinline__ void group_sync(uint32_t G) {
   if (G > 1)
@@ -149,12 +145,6 @@ __device__ __forceinline__ void group_sync(uint32_t G) {
                  "barrier.cluster.wait.acquire.aligned;" ::: "memory");
   else
     __syncthreads();
-}
-__device__ __forceinline__ uint32_t dsm_addr(const void* p, uint32_t rank) {
-  const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
-  return r;
 }
 // Read a shared variable of CTA `rank` of this cluster.
 template <class T>

@@ -1906,7 +1906,8 @@ __device__ __forceinline__ void publish_done(EstIO* io) {
 // per quantity) over n particles, one reciprocal of n.
 __device__ __forceinline__ void est_finish(const double* tot, double n, const double* cs,
                                            double* out) {
-  const double inv_n = 1.0 / n;
+  const double inv_n = div_rn(1.0, n);
+#pragma unroll
   for (int q = 0; q < 3; ++q) {
     const double m1 = tot[2 * q] * inv_n;
     const double m2 = tot[2 * q + 1] * inv_n;
@@ -1923,25 +1924,23 @@ __device__ __forceinline__ void est_add(R* loc, R v0, R v1, R v2, R c0, R c1, R 
   loc[4] += dt; loc[5] += dt * dt;
 }
 
+// The sums of block b of BLOCK x EST_PER_THREAD particles, to part_est (the
+// state is read through L2: the caller may have written it in this launch).
 template <class R>
-__global__ void __launch_bounds__(BLOCK) k_estimate(FilterArgs<R> a) {
-  __shared__ double s_sum[6][WARPS];
-  __shared__ bool s_last;
-  const uint32_t t = a.ctl->t;
-  const StateV<R> st = (t & 1) ? a.st[1] : a.st[0];
-  const R c0 = st.x[0], c1 = st.s2[0], c2 = st.t2[0];
+__device__ __forceinline__ void est_block(const StateV<R>& st, uint64_t n, uint32_t b, R c0, R c1,
+                                          R c2, double (*s_sum)[WARPS], double* part_est) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   {
     R loc[6] = {0, 0, 0, 0, 0, 0};
-    const uint64_t base = ((uint64_t)blockIdx.x * BLOCK + threadIdx.x) * EST_PER_THREAD;
+    const uint64_t base = ((uint64_t)b * BLOCK + threadIdx.x) * EST_PER_THREAD;
     if constexpr (sizeof(R) == 4) {
-      if (base + EST_PER_THREAD <= a.n) {
+      if (base + EST_PER_THREAD <= n) {
         float4 X[EST_PER_THREAD / 4], S[EST_PER_THREAD / 4], T[EST_PER_THREAD / 4];
 #pragma unroll
         for (int q = 0; q < EST_PER_THREAD / 4; ++q) {
-          X[q] = *reinterpret_cast<const float4*>(st.x + base + 4 * q);
-          S[q] = *reinterpret_cast<const float4*>(st.s2 + base + 4 * q);
-          T[q] = *reinterpret_cast<const float4*>(st.t2 + base + 4 * q);
+          X[q] = __ldcg(reinterpret_cast<const float4*>(st.x + base + 4 * q));
+          S[q] = __ldcg(reinterpret_cast<const float4*>(st.s2 + base + 4 * q));
+          T[q] = __ldcg(reinterpret_cast<const float4*>(st.t2 + base + 4 * q));
         }
 #pragma unroll
         for (int q = 0; q < EST_PER_THREAD / 4; ++q) {
@@ -1951,13 +1950,14 @@ __global__ void __launch_bounds__(BLOCK) k_estimate(FilterArgs<R> a) {
           est_add<float>(loc, X[q].w, S[q].w, T[q].w, c0, c1, c2);
         }
       } else {
-        for (uint64_t i = base; i < a.n; ++i) est_add<R>(loc, st.x[i], st.s2[i], st.t2[i], c0, c1, c2);
+        for (uint64_t i = base; i < n; ++i)
+          est_add<R>(loc, __ldcg(st.x + i), __ldcg(st.s2 + i), __ldcg(st.t2 + i), c0, c1, c2);
       }
     } else {
 #pragma unroll 4
       for (int e = 0; e < EST_PER_THREAD; ++e) {
         const uint64_t i = base + e;
-        if (i < a.n) est_add<R>(loc, st.x[i], st.s2[i], st.t2[i], c0, c1, c2);
+        if (i < n) est_add<R>(loc, __ldcg(st.x + i), __ldcg(st.s2 + i), __ldcg(st.t2 + i), c0, c1, c2);
       }
     }
 #pragma unroll
@@ -1972,39 +1972,43 @@ __global__ void __launch_bounds__(BLOCK) k_estimate(FilterArgs<R> a) {
   if (threadIdx.x < 6) {
     double v = 0;
     for (int w = 0; w < WARPS; ++w) v += s_sum[threadIdx.x][w];
-    a.part_est[(uint64_t)blockIdx.x * 6 + threadIdx.x] = v;
+    part_est[(uint64_t)b * 6 + threadIdx.x] = v;
   }
-  if (threadIdx.x == 0) {
-    __threadfence();
-    s_last = atomicAdd(&a.ctl->done_est, 1u) == gridDim.x - 1;
-  }
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-  // fold the block partials: thread i sums blocks i, i + BLOCK, ... (a fixed
-  // assignment), then a shuffle tree per warp and the warps in order
-  {
+  __syncthreads();  // (s_sum is reused; the sums are visible to the block)
+}
+
+// The block sums folded and the summaries written and published: thread i sums
+// blocks i, i + BLOCK, ... (a fixed assignment), then a shuffle tree per warp
+// and the warps in order.
+template <class R>
+__device__ __forceinline__ void est_fold(const FilterArgs<R>& a, uint32_t t, uint32_t nblk, R c0, R c1,
+                                         R c2, double (*s_sum)[WARPS], double* s_tot) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // (a warp without a block adds zeros, which change no sum: it is left out)
+  const int nw = nblk >= BLOCK ? WARPS : (int)((nblk + 31) / 32);
+  if (warp < nw) {
     double v[6] = {0, 0, 0, 0, 0, 0};
-    for (uint32_t b = threadIdx.x; b < gridDim.x; b += BLOCK) {
+    for (uint32_t b = threadIdx.x; b < nblk; b += BLOCK) {
 #pragma unroll
       for (int q = 0; q < 6; ++q) v[q] += __ldcg(a.part_est + (uint64_t)b * 6 + q);
     }
+    if (nblk > 1) {
 #pragma unroll
-    for (int q = 0; q < 6; ++q) {
+      for (int q = 0; q < 6; ++q) {
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
+        for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
+      }
     }
-    __syncthreads();  // s_sum is reused
+    // (s_sum was last read before the caller's barrier)
     if (lane == 0) {
 #pragma unroll
       for (int q = 0; q < 6; ++q) s_sum[q][warp] = v[q];
     }
   }
   __syncthreads();
-  __shared__ double s_tot[6];
   if (threadIdx.x < 6) {  // the warps in order, one quantity per thread
     double v = 0;
-    for (int w = 0; w < WARPS; ++w) v += s_sum[threadIdx.x][w];
+    for (int w = 0; w < nw; ++w) v += s_sum[threadIdx.x][w];
     s_tot[threadIdx.x] = v;
   }
   __syncthreads();
@@ -2018,6 +2022,25 @@ __global__ void __launch_bounds__(BLOCK) k_estimate(FilterArgs<R> a) {
   __syncthreads();
   publish_summary(a.ctl, a.ctl_mirror);
   publish_done(a.io);
+}
+
+template <class R>
+__global__ void __launch_bounds__(BLOCK) k_estimate(FilterArgs<R> a) {
+  __shared__ double s_sum[6][WARPS];
+  __shared__ double s_tot[6];
+  __shared__ bool s_last;
+  const uint32_t t = a.ctl->t;
+  const StateV<R> st = (t & 1) ? a.st[1] : a.st[0];
+  const R c0 = st.x[0], c1 = st.s2[0], c2 = st.t2[0];
+  est_block<R>(st, a.n, blockIdx.x, c0, c1, c2, s_sum, a.part_est);
+  if (threadIdx.x == 0) {  // (the block's sums were written before its last barrier)
+    __threadfence();
+    s_last = atomicAdd(&a.ctl->done_est, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  est_fold<R>(a, t, gridDim.x, c0, c1, c2, s_sum, s_tot);
 }
 
 // Posterior summaries under adaptive resampling: the particles weighted by
