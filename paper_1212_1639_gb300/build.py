@@ -14,7 +14,7 @@ CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 LIB = os.path.join(HERE, "libpf.so")
 SOURCES = ["api.cu", "batch_f32.cu", "batch_f64.cu"]
-DEPS = ["api.cu", "batch_f32.cu", "batch_f64.cu", "kernels.cuh", "device.cuh", "slots.cuh", "small.cuh", "batch.cuh",
+DEPS = ["api.cu", "batch_f32.cu", "batch_f64.cu", "kernels.cuh", "device.cuh", "slots.cuh", "multi.cuh", "small.cuh", "batch.cuh",
         "batch_launch.h", "batch_kernels.cuh", "batch_api.cuh", "server_api.cuh"]
 ARCH = "-gencode=arch=compute_103a,code=sm_103a"
 

@@ -117,11 +117,10 @@ struct pf_filter {
   bool ess = false;
   void* lam = nullptr;
   uint64_t* Q = nullptr;
-  uint64_t* S = nullptr;
   uint32_t* anc = nullptr;
   uint32_t* I = nullptr;
-  uint64_t* splits = nullptr;  // merge-path partition
-  uint64_t* stat_e[2] = {};
+  uint64_t* spre = nullptr;    // multinomial: slot tile prefixes (k_spacing_sums)
+  uint32_t* splits = nullptr;  // and the particles below each tile (k_multi_split)
   void* part = nullptr;
   double* part_est = nullptr;
   Ctl* ctl = nullptr;
@@ -183,12 +182,10 @@ FilterArgs<R> filter_args(pf_filter* f) {
     a.st[p].t2 = (R*)f->t2[p];
     a.st[p].bs = (B*)f->bs[p];
     a.st[p].bt = (B*)f->bt[p];
-    a.stat_e[p] = f->stat_e[p];
   }
   a.ell = (R*)f->ell;
   a.lam = (R*)f->lam;
   a.Q = f->Q;
-  a.S = f->S;
   a.anc = f->anc;
   a.I = f->I;
   a.part = f->part;
@@ -241,36 +238,48 @@ inline void mark(KTimer* tm, const char* name, cudaStream_t s) {
 bool is_multinomial(int scheme) { return scheme == PF_MULTINOMIAL || scheme == PF_MULTINOMIAL_CUTPOINT; }
 bool is_cutpoint(int scheme) { return scheme == PF_MULTINOMIAL_CUTPOINT || scheme == PF_SYSTEMATIC_CUTPOINT; }
 
-// Resampling kernels shared by the filter cycle and pf_resample: from a
-// finished CDF Q (and spacing prefix S) to ancestors (multinomial and the
-// cut-point schemes; systematic and stratified ancestors come from k_slots).
-inline uint32_t merge_chunks(uint64_t n) { return (uint32_t)cdiv(2 * n, MERGE_D); }
+// Tiles of k_slots and k_multi.
+inline uint32_t slot_tiles(uint64_t n) { return (uint32_t)cdiv(n, SLOT_TILE); }
 
-pf_status launch_resample(int scheme, const PosArgs& pa, uint64_t n, uint32_t* I,
-                          uint64_t* splits, cudaStream_t s, KTimer* tm = nullptr) {
-  const bool multi = is_multinomial(scheme);
-  if (!is_cutpoint(scheme) && multi) {
-    const uint32_t chunks = merge_chunks(n);
-    const unsigned pgrid = (unsigned)cdiv((uint64_t)(chunks + 1) * 32, BLOCK);
-    k_partition<POS_MULTINOMIAL><<<pgrid, BLOCK, 0, s>>>(pa, splits, chunks + 1, MERGE_D);
-    mark(tm, "partition", s);
-    k_merge<POS_MULTINOMIAL><<<chunks, BLOCK, 0, s>>>(pa, splits);
-    mark(tm, "merge", s);
-  } else {
-    const unsigned grid = (unsigned)cdiv(n, BLOCK);
-    k_cutpoint_search<<<grid, BLOCK, 0, s>>>(pa.Q, n, I);
-    mark(tm, "cutpoint_search", s);
-    if (multi) k_cutpoint_method<POS_MULTINOMIAL><<<grid, BLOCK, 0, s>>>(pa);
-    else k_cutpoint_method<POS_SYSTEMATIC><<<grid, BLOCK, 0, s>>>(pa);
+// From a finished CDF to ancestors, for the schemes that k_slots does not
+// finish: multinomial (with the spacings' tile prefixes) and, with the table
+// that k_slots left in I, the cut-point method.
+pf_status launch_resample(int scheme, const MultiArgs& ma, const uint32_t* I, cudaStream_t s,
+                          KTimer* tm = nullptr) {
+  if (scheme == PF_SYSTEMATIC_CUTPOINT) {
+    PosArgs pa;
+    pa.Q = ma.Q;
+    pa.anc = ma.anc;
+    pa.I = I;
+    pa.ctl = ma.ctl;
+    pa.t_dev = ma.t_dev;
+    pa.t_arg = ma.t_arg;
+    pa.n = ma.n;
+    pa.seed = ma.seed;
+    pa.filter = ma.filter;
+    pa.gate = ma.gate;
+    k_cutpoint_method_sys<<<(unsigned)cdiv(ma.n, BLOCK), BLOCK, 0, s>>>(pa);
     mark(tm, "cutpoint_method", s);
+  } else if (scheme == PF_MULTINOMIAL_CUTPOINT) {
+    k_multi_split<<<1, BLOCK, 0, s>>>(ma);  // its constants only
+    mark(tm, "split", s);
+    k_multi<true><<<ma.ntiles, BLOCK, 0, s>>>(ma);
+    mark(tm, "cutpoint_method", s);
+  } else {
+    k_multi_split<<<(unsigned)cdiv(ma.ntiles + 1, WARPS), BLOCK, 0, s>>>(ma);
+    mark(tm, "split", s);
+    k_multi<false><<<ma.ntiles, BLOCK, 0, s>>>(ma);
+    mark(tm, "merge", s);
   }
   CK(cudaGetLastError());
   return PF_OK;
 }
 
-// Which slot map a scheme uses (SLOTS_NONE: its ancestors come from launch_resample).
+// Which slot map a scheme uses (the cut-point schemes: for their table;
+// SLOTS_NONE: the CDF alone).
 int slot_pos(int scheme) {
-  return scheme == PF_SYSTEMATIC ? SLOTS_SYS : scheme == PF_STRATIFIED ? SLOTS_STRAT : SLOTS_NONE;
+  return scheme == PF_SYSTEMATIC || is_cutpoint(scheme) ? SLOTS_SYS
+         : scheme == PF_STRATIFIED                      ? SLOTS_STRAT : SLOTS_NONE;
 }
 template <int SRC>
 void launch_slots(int pos, const SlotArgs& a, cudaStream_t s) {
@@ -290,7 +299,8 @@ void launch_cdf(pf_filter* f, cudaStream_t s, KTimer* tm) {
   SlotArgs a;
   std::memset(&a, 0, sizeof(a));
   a.Q = f->Q;
-  a.anc = f->anc;
+  a.cut = is_cutpoint(f->scheme);
+  a.anc = a.cut ? f->I : f->anc;
   a.pre = f->pre;
   a.part = f->part;
   a.sq = f->sq;
@@ -328,7 +338,7 @@ void launch_cdf(pf_filter* f, cudaStream_t s, KTimer* tm) {
       launch_slots<SRC_E32>(pos, a, s);
     }
   }
-  mark(tm, pos == SLOTS_NONE ? "cdf" : "cdf_resample", s);
+  mark(tm, pos == SLOTS_NONE ? "cdf" : a.cut ? "cutpoint_search" : "cdf_resample", s);
 }
 
 // One cycle (Steps 1-4), enqueued on f->stream; reads t and y on the device.
@@ -361,19 +371,23 @@ pf_status enqueue_cycle(pf_filter* f, KTimer* tm = nullptr, const double* y_src 
   // on the seed, the filter and t, so outside a timed cycle it runs on the
   // side stream beside the weights and the CDF scan
   const bool fork = is_multinomial(f->scheme) && !tm;
-  auto spacing = [&](cudaStream_t on) {
-    SpacingArgs sp;
-    sp.S = f->S;
-    sp.stat[0] = f->stat_e[0];
-    sp.stat[1] = f->stat_e[1];
-    sp.ctl = f->ctl;
-    sp.t_dev = &f->ctl->t;
-    sp.t_arg = 0;
-    sp.n = n;
-    sp.seed = f->cfg.seed;
-    sp.filter = f->cfg.filter_id;
-    k_spacing_scan<<<f->ntiles, BLOCK, 0, on>>>(sp);
-  };
+  MultiArgs ma;
+  std::memset(&ma, 0, sizeof(ma));
+  ma.Q = f->Q;
+  ma.pre = f->pre;
+  ma.spre = f->spre;
+  ma.splits = f->splits;
+  ma.anc = f->anc;
+  ma.I = f->I;
+  ma.ctl = f->ctl;
+  ma.t_dev = &f->ctl->t;
+  ma.ntiles = slot_tiles(n);
+  ma.n = n;
+  ma.seed = f->cfg.seed;
+  ma.filter = f->cfg.filter_id;
+  ma.gate = f->ess ? &f->ctl->resamp : nullptr;
+  ma.anc_vec = 1;
+  auto spacing = [&](cudaStream_t on) { k_spacing_sums<<<ma.ntiles, BLOCK, 0, on>>>(ma); };
   if (fork) {
     CK(cudaEventRecord(f->ev_fork, s));
     CK(cudaStreamWaitEvent(f->side, f->ev_fork, 0));
@@ -398,22 +412,10 @@ pf_status enqueue_cycle(pf_filter* f, KTimer* tm = nullptr, const double* y_src 
     CK(cudaStreamWaitEvent(s, f->ev_join, 0));
   } else if (is_multinomial(f->scheme)) {
     spacing(s);
-    mark(tm, "spacing_scan", s);
+    mark(tm, "spacing_sums", s);
   }
-  PosArgs pa;
-  pa.gate = f->ess ? &f->ctl->resamp : nullptr;
-  pa.Q = f->Q;
-  pa.S = f->S;
-  pa.anc = f->anc;
-  pa.I = f->I;
-  pa.ctl = f->ctl;
-  pa.t_dev = &f->ctl->t;
-  pa.t_arg = 0;
-  pa.n = n;
-  pa.seed = f->cfg.seed;
-  pa.filter = f->cfg.filter_id;
-  if (slot_pos(f->scheme) == SLOTS_NONE) {
-    pf_status st = launch_resample(f->scheme, pa, n, f->I, f->splits, s, tm);
+  if (is_multinomial(f->scheme) || is_cutpoint(f->scheme)) {
+    pf_status st = launch_resample(f->scheme, ma, f->I, s, tm);
     if (st != PF_OK) return st;
   }
   const bool fuse = !f->bootstrap && !f->ess && form_fuses(form);
@@ -718,12 +720,12 @@ pf_status pf_create(const pf_config* cfg, pf_filter** out) {
     if ((st = dev_alloc(f, n * rs, &f->t2[p])) != PF_OK) return bail(st);
     if ((st = dev_alloc(f, n * 8, &f->bs[p])) != PF_OK) return bail(st);
     if ((st = dev_alloc(f, n * 8, &f->bt[p])) != PF_OK) return bail(st);
-    if ((st = dev_alloc(f, (size_t)f->ntiles * 8, (void**)&f->stat_e[p])) != PF_OK) return bail(st);
   }
   if ((st = dev_alloc(f, n * rs, &f->ell)) != PF_OK) return bail(st);
   if ((st = dev_alloc(f, n * 8, (void**)&f->Q)) != PF_OK) return bail(st);
   if (is_multinomial(f->scheme)) {
-    if ((st = dev_alloc(f, (n + 1) * 8, (void**)&f->S)) != PF_OK) return bail(st);
+    if ((st = dev_alloc(f, pre_bytes(n), (void**)&f->spre)) != PF_OK) return bail(st);
+    if ((st = dev_alloc(f, ((size_t)slot_tiles(n) + 1) * 4, (void**)&f->splits)) != PF_OK) return bail(st);
     if (cudaStreamCreateWithFlags(&f->side, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&f->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&f->ev_join, cudaEventDisableTiming) != cudaSuccess)
@@ -731,7 +733,6 @@ pf_status pf_create(const pf_config* cfg, pf_filter** out) {
   }
   if ((st = dev_alloc(f, n * 4, (void**)&f->anc)) != PF_OK) return bail(st);
   if (is_cutpoint(f->scheme) && (st = dev_alloc(f, n * 4, (void**)&f->I)) != PF_OK) return bail(st);
-  if ((st = dev_alloc(f, ((size_t)merge_chunks(n) + 1) * 8, (void**)&f->splits)) != PF_OK) return bail(st);
   // log-ML partials.  Binary64: one per 4096 particles (rounded sums, folded in
   // order); binary32: exact sums, folded into the first entry by k_sums
   if ((st = dev_alloc(f, ((size_t)f->ntiles + 1) * sizeof(ESum32), &f->part)) != PF_OK) return bail(st);
@@ -785,10 +786,6 @@ pf_status pf_create(const pf_config* cfg, pf_filter** out) {
     return bail(set_err(PF_ERR_CUDA, "control block upload failed"));
   if (f->ess && cudaMemsetAsync(f->lam, 0, n * rs, f->stream) != cudaSuccess)
     return bail(set_err(PF_ERR_CUDA, "log-weight memset failed"));
-  for (int p = 0; p < 2; ++p) {
-    if (cudaMemsetAsync(f->stat_e[p], 0, (size_t)f->ntiles * 8, f->stream) != cudaSuccess)
-      return bail(set_err(PF_ERR_CUDA, "status memset failed"));
-  }
   const unsigned grid = (unsigned)cdiv(n, BLOCK);
   if (f->fp64) {
     FilterArgs<double> a = filter_args<double>(f);
@@ -1278,49 +1275,46 @@ namespace {
 
 struct Scratch {
   uint64_t* Q;
-  uint64_t* S;
   uint32_t* I;
-  uint64_t* splits;
-  uint64_t* pre;
-  uint64_t* stat[2];
-  uint64_t* stat_e[2];
+  uint64_t* pre;          // CDF tile prefixes, then the heavy list
+  uint64_t* spre;
+  uint32_t* splits;
+  uint64_t* stat[2];      // pf_cdf: tile status of the scan
   Ctl* ctl;
-  void* base;
 };
 
 constexpr size_t align256(size_t b) { return (b + 255) & ~size_t(255); }
 
+// What a scheme's resampling (cdf: pf_cdf) needs.
+inline bool scheme_needs_Q(int scheme) { return is_multinomial(scheme) || is_cutpoint(scheme); }
+
 // Lay out the scratch of pf_resample / pf_cdf inside one allocation.
-size_t scratch_layout(uint64_t n, bool need_Q, bool multi, bool cut, char* base, Scratch* s) {
+size_t scratch_layout(uint64_t n, int scheme, bool cdf, char* base, Scratch* s) {
   const uint64_t ntiles = cdiv(n, TILE);
   size_t off = 0;
-  auto take = [&](size_t bytes) {
+  auto take = [&](bool need, size_t bytes) -> char* {
+    if (!need) return nullptr;
     char* p = base ? base + off : nullptr;
     off += align256(bytes);
     return p;
   };
-  s->ctl = (Ctl*)take(sizeof(Ctl));
-  s->stat[0] = (uint64_t*)take(ntiles * 8);
-  s->stat[1] = (uint64_t*)take(ntiles * 8);
-  s->stat_e[0] = (uint64_t*)take(ntiles * 8);
-  s->stat_e[1] = (uint64_t*)take(ntiles * 8);
-  const size_t zero_bytes = off;  // everything above must start at zero
-  s->Q = need_Q ? (uint64_t*)take(n * 8) : nullptr;
-  s->S = multi ? (uint64_t*)take((n + 1) * 8) : nullptr;
-  s->I = cut ? (uint32_t*)take(n * 4) : nullptr;
-  s->splits = (uint64_t*)take(((size_t)merge_chunks(n) + 1) * 8);
-  s->pre = (uint64_t*)take(pre_heavy_bytes(n));
-  s->base = base;
-  (void)zero_bytes;
+  s->ctl = (Ctl*)take(true, sizeof(Ctl));
+  s->stat[0] = (uint64_t*)take(cdf, ntiles * 8);
+  s->stat[1] = (uint64_t*)take(cdf, ntiles * 8);
+  s->pre = (uint64_t*)take(!cdf, pre_heavy_bytes(n));
+  s->spre = (uint64_t*)take(!cdf && is_multinomial(scheme), pre_bytes(n));
+  s->splits = (uint32_t*)take(!cdf && is_multinomial(scheme), ((size_t)slot_tiles(n) + 1) * 4);
+  s->Q = (uint64_t*)take(!cdf && scheme_needs_Q(scheme), n * 8);
+  s->I = (uint32_t*)take(!cdf && is_cutpoint(scheme), n * 4);
   return off;
 }
 
-size_t scratch_zero_bytes(uint64_t n) {
-  const uint64_t ntiles = cdiv(n, TILE);
-  return align256(sizeof(Ctl)) + 4 * align256(ntiles * 8);
+// The leading bytes that must start at zero.
+size_t scratch_zero_bytes(uint64_t n, bool cdf) {
+  return align256(sizeof(Ctl)) + (cdf ? 2 * align256(cdiv(n, TILE) * 8) : 0);
 }
 
-// Weights -> Q (and S for multinomial) -> ancestors, on stream s with the
+// Weights -> ancestors, or the CDF, on stream s with the
 // given scratch (already zeroed in its first scratch_zero_bytes bytes).
 // Wait settings of the scan: the normal bound, or a failure-detection test's.
 struct WaitDiag {
@@ -1331,7 +1325,6 @@ struct WaitDiag {
 pf_status run_resample(const float* w, uint64_t n, uint64_t seed, uint32_t filter, uint32_t t,
                        int scheme, uint32_t* anc, uint64_t* Q_out, const Scratch& sc,
                        cudaStream_t s, WaitDiag dg = WaitDiag()) {
-  const uint32_t ntiles = (uint32_t)cdiv(n, TILE);
   const uint64_t want = cdiv(n, 8 * BLOCK);
   const unsigned gmax = (unsigned)(want < 152 * 8 ? want : 152 * 8);
   k_wmax<<<gmax, BLOCK, 0, s>>>(w, n, sc.ctl, ((uintptr_t)w & 31) == 0);
@@ -1341,10 +1334,11 @@ pf_status run_resample(const float* w, uint64_t n, uint64_t seed, uint32_t filte
     std::memset(&a, 0, sizeof(a));
     const int pos = slot_pos(scheme);
     a.src = w;
-    a.Q = pos == SLOTS_NONE ? sc.Q : nullptr;
-    a.anc = anc;
+    a.Q = sc.Q;
+    a.cut = is_cutpoint(scheme);
+    a.anc = a.cut ? sc.I : anc;
     a.pre = sc.pre;
-      if (pos != SLOTS_NONE) a.heavy = (char*)sc.pre + pre_bytes(n);
+    if (pos != SLOTS_NONE) a.heavy = (char*)sc.pre + pre_bytes(n);
     a.ctl = sc.ctl;
     a.t_arg = t;
     a.n = n;
@@ -1353,12 +1347,29 @@ pf_status run_resample(const float* w, uint64_t n, uint64_t seed, uint32_t filte
     a.seed = seed;
     a.filter = filter;
     a.src_vec = ((uintptr_t)w & 31) == 0;
-    a.anc_vec = ((uintptr_t)anc & 15) == 0;
+    a.anc_vec = ((uintptr_t)a.anc & 15) == 0;
     k_sums<SRC_W, false><<<sums_grid(n), BLOCK, 0, s>>>(a);
     launch_slots<SRC_W>(pos, a, s);
     CK(cudaGetLastError());
-    if (pos != SLOTS_NONE) return PF_OK;
-  } else {
+    if (!scheme_needs_Q(scheme)) return PF_OK;
+    MultiArgs ma;
+    std::memset(&ma, 0, sizeof(ma));
+    ma.Q = sc.Q;
+    ma.pre = sc.pre;
+    ma.spre = sc.spre;
+    ma.splits = sc.splits;
+    ma.anc = anc;
+    ma.I = sc.I;
+    ma.ctl = sc.ctl;
+    ma.t_arg = t;
+    ma.ntiles = slot_tiles(n);
+    ma.n = n;
+    ma.seed = seed;
+    ma.filter = filter;
+    ma.anc_vec = ((uintptr_t)anc & 31) == 0;
+    if (is_multinomial(scheme)) k_spacing_sums<<<ma.ntiles, BLOCK, 0, s>>>(ma);
+    return launch_resample(scheme, ma, sc.I, s);
+  }
   ScanArgs sa;
   sa.src = w;
   sa.Q = Q_out;
@@ -1372,36 +1383,9 @@ pf_status run_resample(const float* w, uint64_t n, uint64_t seed, uint32_t filte
   sa.vec_ok = ((uintptr_t)w & 15) == 0;
   sa.spin_limit = dg.spin_limit;
   sa.withhold = dg.withhold;
-  k_scan<<<ntiles, BLOCK, 0, s>>>(sa);
+  k_scan<<<(unsigned)cdiv(n, TILE), BLOCK, 0, s>>>(sa);
   CK(cudaGetLastError());
   return PF_OK;
-  }
-  if (is_multinomial(scheme)) {
-    SpacingArgs sp;
-    sp.S = sc.S;
-    sp.stat[0] = sc.stat_e[0];
-    sp.stat[1] = sc.stat_e[1];
-    sp.ctl = sc.ctl;
-    sp.t_dev = nullptr;
-    sp.t_arg = t;
-    sp.n = n;
-    sp.seed = seed;
-    sp.filter = filter;
-    k_spacing_scan<<<ntiles, BLOCK, 0, s>>>(sp);
-  }
-  PosArgs pa;
-  pa.gate = nullptr;
-  pa.Q = sc.Q;
-  pa.S = sc.S;
-  pa.anc = anc;
-  pa.I = sc.I;
-  pa.ctl = sc.ctl;
-  pa.t_dev = nullptr;
-  pa.t_arg = t;
-  pa.n = n;
-  pa.seed = seed;
-  pa.filter = filter;
-  return launch_resample(scheme, pa, n, sc.I, sc.splits, s);
 }
 
 pf_status finish_and_check(const Scratch& sc, cudaStream_t s) {
@@ -1495,9 +1479,8 @@ pf_status resample_common(const float* w, uint64_t n, uint64_t seed, uint32_t fi
       (scheme == PF_SYSTEMATIC || scheme == PF_STRATIFIED))
     return resample_small(w, n, seed, filter, t, scheme, anc, s);
   Scratch sc;
-  const bool multi = anc && is_multinomial(scheme), cut = anc && is_cutpoint(scheme);
-  const bool need_Q = anc && slot_pos(scheme) == SLOTS_NONE;
-  const size_t bytes = scratch_layout(n, need_Q, multi, cut, nullptr, &sc);
+  const bool cdf = !anc;
+  const size_t bytes = scratch_layout(n, scheme, cdf, nullptr, &sc);
   void* base = nullptr;
   cudaMemPool_t pool = nullptr;
   pf_status sp = scratch_pool(&pool);
@@ -1507,9 +1490,9 @@ pf_status resample_common(const float* w, uint64_t n, uint64_t seed, uint32_t fi
     cudaGetLastError();
     return set_err(PF_ERR_OOM, "cudaMallocFromPoolAsync(%zu): %s", bytes, cudaGetErrorString(e));
   }
-  scratch_layout(n, need_Q, multi, cut, (char*)base, &sc);
+  scratch_layout(n, scheme, cdf, (char*)base, &sc);
   pf_status st = PF_OK;
-  if (cudaMemsetAsync(base, 0, scratch_zero_bytes(n), s) != cudaSuccess)
+  if (cudaMemsetAsync(base, 0, scratch_zero_bytes(n, cdf), s) != cudaSuccess)
     st = set_err(PF_ERR_CUDA, "scratch memset failed");
   if (st == PF_OK) st = run_resample(w, n, seed, filter, t, scheme, anc, Q_out, sc, s, dg);
   pf_status st2 = PF_OK;
@@ -1597,12 +1580,9 @@ pf_status pf_cutpoint_method(const uint64_t* Q_dev, uint64_t n, const uint32_t* 
 namespace {
 
 constexpr uint64_t NOALLOC_N = PF_NOALLOC_MAX_PARTICLES;
-constexpr uint64_t NOALLOC_TILES = (NOALLOC_N + TILE - 1) / TILE;
 constexpr size_t NOALLOC_BYTES =
-    align256(sizeof(Ctl)) + 4 * align256(NOALLOC_TILES * 8) + align256(NOALLOC_N * 8) +
-    align256((NOALLOC_N + 1) * 8) + align256(NOALLOC_N * 4) +
-    align256(((2 * NOALLOC_N + MERGE_D - 1) / MERGE_D + 1) * 8) +
-    align256(pre_heavy_bytes(NOALLOC_N));
+    align256(sizeof(Ctl)) + align256(pre_heavy_bytes(NOALLOC_N)) + align256(pre_bytes(NOALLOC_N)) +
+    align256((NOALLOC_N / SLOT_TILE + 2) * 4) + align256(NOALLOC_N * 8) + align256(NOALLOC_N * 4);
 
 // The scratch itself: one copy per device, shared by every call on it.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[NOALLOC_BYTES];
@@ -1644,12 +1624,11 @@ extern "C" pf_status pf_resample_noalloc(const float* w_dev, uint64_t n, uint64_
   pf_status st = noalloc_scratch(&base);
   if (st != PF_OK) return st;
   Scratch sc;
-  const size_t bytes =
-      scratch_layout(n, true, is_multinomial(scheme), is_cutpoint(scheme), nullptr, &sc);
-  if (bytes > NOALLOC_BYTES) return set_err(PF_ERR_INVALID, "scratch layout exceeds the static array");
-  scratch_layout(n, true, is_multinomial(scheme), is_cutpoint(scheme), base, &sc);
-  // the control block and tile status words must start at zero each call
-  CK(cudaMemsetAsync(base, 0, scratch_zero_bytes(n), s));
+  if (scratch_layout(n, scheme, false, nullptr, &sc) > NOALLOC_BYTES)
+    return set_err(PF_ERR_INVALID, "scratch layout exceeds the static array");
+  scratch_layout(n, scheme, false, base, &sc);
+  // the control block must start at zero each call
+  CK(cudaMemsetAsync(base, 0, scratch_zero_bytes(n, false), s));
   if ((st = run_resample(w_dev, n, seed, filter_id, t, scheme, anc_dev, nullptr, sc, s)) != PF_OK)
     return st;
   return finish_and_check(sc, s);

@@ -79,6 +79,8 @@ struct BatchArgs {
   int commit;               // 0: a trial cycle that leaves t, log-ML and err untouched
 };
 
+enum PosKind { POS_MULTINOMIAL = 0, POS_SYSTEMATIC = 1 };  // a batch's resampling positions
+
 constexpr int BB = BLOCK;                 // threads per CTA of the init and summary kernels
 constexpr int BATCH_EST_ROW = 9;          // t, 6 summaries, log-ML, error bits
 constexpr int BB_CAP = 32;                // slots emitted per particle before a run

@@ -30,8 +30,6 @@ constexpr int WARPS = BLOCK / 32;
 constexpr int CHUNK = 128;                 // elements per warp per chunk (4 per lane)
 constexpr int CHUNKS = 4;                  // chunks per warp
 constexpr int TILE = WARPS * CHUNKS * CHUNK;  // 4096 elements per scan tile
-constexpr int MERGE_D = 2048;              // merged elements per merge CTA
-constexpr int MERGE_E = MERGE_D / BLOCK;   // merged elements per thread
 
 constexpr uint64_t FLAG_A = 1ull << 62;    // tile aggregate published
 constexpr uint64_t FLAG_P = 2ull << 62;    // tile inclusive prefix published
@@ -50,7 +48,6 @@ struct Ctl {
   uint32_t err;           // ErrBits
   unsigned long long maxenc;  // order-encoded max of l (or of the input weights)
   uint32_t ticket_w;      // scan tile ticket
-  uint32_t ticket_e;      // spacing scan tile ticket
   uint32_t done_prop;     // last-block counter of k_propagate
   uint32_t done_est;      // last-block counter of k_estimate
   double logml;           // accumulated log marginal likelihood
@@ -61,9 +58,8 @@ struct Ctl {
                           // squeeze coefficients K_sigma, K_tau ([4], [5]), binary64
   float yf;               // y rounded to binary32
   float mtf[6];           // the same constants rounded to binary32
-  // resampling key constants written by k_sums, or by k_partition (block 0) for
-  // k_merge: T = Q_{n-1}, A (n or S_n) and the systematic offset r
-  uint64_t keyT, keyA, keyR;
+  // resampling constants written by k_sums: T = Q_{n-1} and the systematic offset r
+  uint64_t keyT, keyR;
   // the next cycle's maximum of l, gathered by a propagation that also
   // computes the next cycle's predictive weights (order-encoded, as maxenc)
   unsigned long long maxenc_nx;
@@ -80,6 +76,11 @@ struct Ctl {
   int32_t slot_z;
   uint64_t slot_rho, slot_r32;
   uint32_t heavy_count, heavy_chunks;
+  // multinomial: last-block counter of k_spacing_sums, S_n, and the constants of
+  // the slots' positions (k_multi_split)
+  uint32_t done_spc;
+  int32_t multi_z;
+  uint64_t keyS, multi_rho, bucket_rho;
 };
 
 // Tile status words carry their value and flag in one aligned 64-bit word and
@@ -141,10 +142,8 @@ struct FilterArgs {
   StateV<R> st[2];          // ping-pong by cycle parity
   R* ell;
   uint64_t* Q;
-  uint64_t* S;              // n+1 spacing prefix (multinomial)
   uint32_t* anc;
   uint32_t* I;              // cut-point table
-  uint64_t* stat_e[2];      // spacing scan tile status, by parity
   void* part;               // per-tile log-ML partial (U128 for FP32, double for FP64)
   double* part_est;         // per-block estimate partials
   Ctl* ctl;
@@ -757,12 +756,8 @@ static __global__ void __launch_bounds__(BLOCK, 4) k_scan(ScanArgs a) {
   }
 }
 
-// ---------------------------------------------------------------------------
-// Multinomial positions: exponential spacings (Carpenter, Clifford &
-// Fearnhead 1999).  E_l = floor(-log(u_l) 2^31), u_l from draw
-// (seed, filter, t, l >> 2, SPACING) word l & 3; S = inclusive scan of E over
-// l = 0..n-1 by the same look-back scan, and S[n] = S[n-1] + E_n.
-// ---------------------------------------------------------------------------
+// Multinomial positions: spacing E_l = floor(-log(u_l) 2^31), u_l from draw
+// (seed, filter, t, l >> 2, SPACING) word l & 3 (multi.cuh).
 __device__ __forceinline__ uint64_t spacing_E(uint64_t seed, uint32_t filter, uint32_t t,
                                               uint64_t l, const U4& w) {
   const uint32_t word = (l & 3) == 0 ? w.a : (l & 3) == 1 ? w.b : (l & 3) == 2 ? w.c : w.d;
@@ -770,272 +765,6 @@ __device__ __forceinline__ uint64_t spacing_E(uint64_t seed, uint32_t filter, ui
   const float L = det_log(u);
   const float x = -L * 0x1p31f;
   return f2u64_rz(x);
-}
-
-struct SpacingArgs {
-  uint64_t* S;
-  uint64_t* stat[2];
-  Ctl* ctl;
-  const uint32_t* t_dev;    // cycle index in device memory, or NULL
-  uint32_t t_arg;
-  uint64_t n;
-  uint64_t seed;
-  uint32_t filter;
-};
-
-static __global__ void __launch_bounds__(BLOCK, 3) k_spacing_scan(SpacingArgs a) {
-  __shared__ uint32_t s_tile;
-  __shared__ uint64_t s_warp_tot[WARPS];
-  __shared__ uint64_t s_excl;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (threadIdx.x == 0) s_tile = atomicAdd(&a.ctl->ticket_e, 1u);
-  __syncthreads();
-  const uint32_t tile = s_tile;
-  const uint32_t t = a.t_dev ? *a.t_dev : a.t_arg;
-  const uint64_t wbase = (uint64_t)tile * TILE + (uint64_t)warp * (CHUNKS * CHUNK);
-  uint64_t W[CHUNKS][4];
-#pragma unroll
-  for (int c = 0; c < CHUNKS; ++c) {
-    const uint64_t i0 = wbase + (uint64_t)c * CHUNK + 4 * lane;  // multiple of 4
-    const U4 w = draw(a.seed, a.filter, t, (uint32_t)(i0 >> 2), P_SPACING, 0);
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      uint64_t v = 0;
-      if (i0 + e < a.n) {
-        const uint32_t word = e == 0 ? w.a : e == 1 ? w.b : e == 2 ? w.c : w.d;
-        const float u = unif_f32(word);
-        const float L = det_log(u);
-        const float x = -L * 0x1p31f;
-        v = f2u64_rz(x);
-      }
-      W[c][e] = v;
-    }
-  }
-  uint64_t carry = 0;
-#pragma unroll
-  for (int c = 0; c < CHUNKS; ++c) {
-    W[c][1] += W[c][0];
-    W[c][2] += W[c][1];
-    W[c][3] += W[c][2];
-    const uint64_t incl = warp_incl_scan(W[c][3], lane);
-    const uint64_t excl_l = incl - W[c][3] + carry;
-#pragma unroll
-    for (int e = 0; e < 4; ++e) W[c][e] += excl_l;
-    carry += __shfl_sync(0xffffffffu, incl, 31);
-  }
-  if (lane == 0) s_warp_tot[warp] = carry;
-  __syncthreads();
-  if (warp == 0) {
-    uint64_t wt = lane < WARPS ? s_warp_tot[lane] : 0;
-    const uint64_t wincl = warp_incl_scan(wt, lane);
-    if (lane < WARPS) s_warp_tot[lane] = wincl - wt;
-    const uint64_t total = __shfl_sync(0xffffffffu, wincl, 31);
-    uint64_t* const stat = (t & 1u) ? a.stat[1] : a.stat[0];
-    uint64_t* const stat_next = (t & 1u) ? a.stat[0] : a.stat[1];
-    const uint64_t excl = lookback(stat, tile, total, &a.ctl->err);
-    if (lane == 0) {
-      s_excl = excl;
-      stat_next[tile] = 0;
-    }
-  }
-  __syncthreads();
-  const uint64_t off = s_excl + s_warp_tot[warp];
-#pragma unroll
-  for (int c = 0; c < CHUNKS; ++c) {
-    const uint64_t i0 = wbase + (uint64_t)c * CHUNK + 4 * lane;
-    if (i0 + 4 <= a.n) {
-      *reinterpret_cast<ulonglong2*>(a.S + i0) = make_ulonglong2(W[c][0] + off, W[c][1] + off);
-      *reinterpret_cast<ulonglong2*>(a.S + i0 + 2) = make_ulonglong2(W[c][2] + off, W[c][3] + off);
-    }
-    if (i0 + 4 > a.n) {
-#pragma unroll
-      for (int e = 0; e < 4; ++e)
-        if (i0 + e < a.n) a.S[i0 + e] = W[c][e] + off;
-    }
-  }
-  // S[n] = S[n-1] + E_n, by the thread holding element n-1
-  const uint64_t last = a.n - 1;
-  const uint64_t lb = last - wbase;  // position of n-1 in this warp's 512 elements
-  if (last >= wbase && lb < CHUNKS * CHUNK && ((lb % CHUNK) >> 2) == (uint64_t)lane) {
-    const int c = (int)(lb / CHUNK), e = (int)(lb & 3);
-    uint64_t v = 0;
-#pragma unroll
-    for (int cc = 0; cc < CHUNKS; ++cc)
-#pragma unroll
-      for (int ee = 0; ee < 4; ++ee)
-        if (cc == c && ee == e) v = W[cc][ee];
-    const uint64_t ln = a.n;
-    const U4 w = draw(a.seed, a.filter, t, (uint32_t)(ln >> 2), P_SPACING, 0);
-    a.S[ln] = v + off + spacing_E(a.seed, a.filter, t, ln, w);
-  }
-}
-
-// ---------------------------------------------------------------------------
-// Resampling by merge (paper Section 3.1, multinomial with sorted uniforms;
-// systematic): the merged order of the CDF keys KQ_i = Q_i * A and the
-// position keys KB_j is cut into equal diagonals (merge path, Green, McColl
-// & Bader 2012).  Each CTA finds its two diagonal splits with a warp-wide
-// 32-ary search, stages both key ranges in shared memory and merges.
-// Ties go to the CDF (Q_i * A <= B_j means particle i lies below slot j).
-// ---------------------------------------------------------------------------
-enum PosKind { POS_MULTINOMIAL = 0, POS_SYSTEMATIC = 1 };
-
-struct PosArgs {
-  const uint64_t* Q;
-  const uint64_t* S;      // multinomial: spacing prefix, n+1 entries
-  uint32_t* anc;
-  const uint32_t* I;      // cut-point table (cut-point kernels)
-  Ctl* ctl;
-  const uint32_t* t_dev;
-  uint32_t t_arg;
-  uint64_t n;
-  uint64_t seed;
-  uint32_t filter;
-  // adaptive resampling: when set and *gate == 0 this cycle does not
-  // resample, and the resampling kernels return at once (NULL: always run)
-  const uint32_t* gate;
-};
-
-__device__ __forceinline__ bool gated_off(const PosArgs& a) { return a.gate && *a.gate == 0u; }
-
-template <int POS>
-struct PosKeys {
-  const uint64_t* Q;
-  const uint64_t* S;
-  uint64_t n, T, A, r;
-  __device__ __forceinline__ U128 kq(uint64_t i) const {
-    if (POS == POS_SYSTEMATIC) return mul64x32(Q[i], (uint32_t)A);  // A = n < 2^32
-    return mul64(Q[i], A);
-  }
-  __device__ __forceinline__ U128 kb(uint64_t j) const {
-    if (POS == POS_SYSTEMATIC) return add128(mul64x32(T, (uint32_t)j), r);
-    return mul64(S[j], T);
-  }
-};
-
-template <int POS>
-__device__ __forceinline__ PosKeys<POS> make_keys(const PosArgs& a) {
-  PosKeys<POS> K;
-  K.Q = a.Q;
-  K.S = a.S;
-  K.n = a.n;
-  K.T = a.Q[a.n - 1];
-  const uint32_t t = a.t_dev ? *a.t_dev : a.t_arg;
-  if (POS == POS_SYSTEMATIC) {
-    K.A = a.n;
-    const U4 w = draw(a.seed, a.filter, t, 0, P_SYS_OFFSET, 0);
-    const uint64_t R = ((uint64_t)w.b << 32) | w.a;
-    K.r = __umul64hi(R, K.T);
-  } else {
-    K.A = a.S[a.n];
-    K.r = 0;
-  }
-  return K;
-}
-
-// Number of CDF elements among the first d merged elements, by warp-wide
-// 32-ary search.  P(i) = (KQ_{i-1} <= KB_{d-i}) is true then false in i.
-template <int POS>
-__device__ __forceinline__ uint64_t warp_split(const PosKeys<POS>& K, uint64_t d) {
-  const int lane = threadIdx.x & 31;
-  uint64_t lo = d > K.n ? d - K.n : 0;
-  uint64_t hi = d < K.n ? d : K.n;
-  while (hi > lo) {
-    const uint64_t span = hi - lo;
-    const uint64_t q = lo + 1 + (span * (uint64_t)lane) / 32;
-    const bool p = le128(K.kq(q - 1), K.kb(d - q));
-    const uint32_t m = __ballot_sync(0xffffffffu, p);
-    if (m == 0) {
-      hi = lo;
-    } else {
-      const int kstar = 31 - __clz(m);  // trues form a prefix: last true lane
-      const uint64_t qk = __shfl_sync(0xffffffffu, q, kstar);
-      const uint64_t qn = __shfl_sync(0xffffffffu, q, kstar < 31 ? kstar + 1 : 31);
-      lo = qk;
-      if (kstar < 31) hi = qn - 1;
-    }
-  }
-  return lo;
-}
-
-// Merge-path partition: the split of diagonal d = c * MERGE_D, one warp per
-// split, all splits searched concurrently.  Block 0 also publishes the key
-// constants (T, A, r) for k_merge.
-template <int POS>
-__global__ void __launch_bounds__(BLOCK) k_partition(PosArgs a, uint64_t* splits,
-                                                     uint32_t nsplits, uint32_t tile) {
-  if (gated_off(a)) return;
-  const PosKeys<POS> K = make_keys<POS>(a);
-  const int lane = threadIdx.x & 31;
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    a.ctl->keyT = K.T;
-    a.ctl->keyA = K.A;
-    a.ctl->keyR = K.r;
-  }
-  const uint32_t wid = (uint32_t)(((uint64_t)blockIdx.x * BLOCK + threadIdx.x) >> 5);
-  if (wid >= nsplits) return;  // uniform per warp
-  const uint64_t total = 2 * a.n;
-  const uint64_t d = (uint64_t)wid * tile < total ? (uint64_t)wid * tile : total;
-  uint64_t sp;
-  if (K.T == 0 || K.A == 0) {
-    sp = d < a.n ? d : a.n;  // empty CDF: any monotone split; k_merge flags it
-  } else {
-    sp = warp_split<POS>(K, d);
-  }
-  if (lane == 0) splits[wid] = sp;
-}
-
-template <int POS>
-__global__ void __launch_bounds__(BLOCK) k_merge(PosArgs a, const uint64_t* splits) {
-  if (gated_off(a)) return;
-  __shared__ U128 s_key[MERGE_D];
-  PosKeys<POS> K;
-  K.Q = a.Q;
-  K.S = a.S;
-  K.n = a.n;
-  K.T = a.ctl->keyT;
-  K.A = a.ctl->keyA;
-  K.r = a.ctl->keyR;
-  if (K.T == 0 || K.A == 0) {  // empty CDF: flag, keep every index in range
-    if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&a.ctl->err, ERR_NUMERIC);
-    for (uint64_t j = (uint64_t)blockIdx.x * BLOCK + threadIdx.x; j < a.n;
-         j += (uint64_t)gridDim.x * BLOCK)
-      a.anc[j] = (uint32_t)j;
-    return;
-  }
-  const uint64_t total = 2 * a.n;
-  const uint64_t d0 = (uint64_t)blockIdx.x * MERGE_D;
-  const uint64_t d1 = d0 + MERGE_D < total ? d0 + MERGE_D : total;
-  const uint64_t i0 = splits[blockIdx.x], i1 = splits[blockIdx.x + 1];
-  const uint64_t j0 = d0 - i0, j1 = d1 - i1;
-  const int nA = (int)(i1 - i0), nB = (int)(j1 - j0);
-  for (int e = threadIdx.x; e < nA; e += BLOCK) s_key[e] = K.kq(i0 + e);
-  for (int e = threadIdx.x; e < nB; e += BLOCK) s_key[nA + e] = K.kb(j0 + e);
-  __syncthreads();
-  // this thread's diagonal range within the CTA's merge
-  const int dl0 = threadIdx.x * MERGE_E;
-  const int len = nA + nB;
-  if (dl0 >= len) return;
-  const int dl1 = dl0 + MERGE_E < len ? dl0 + MERGE_E : len;
-  // local split on diagonal dl0: largest ia with ia == lo or A[ia-1] <= B[dl0-ia]
-  int lo = dl0 > nB ? dl0 - nB : 0;
-  int hi = dl0 < nA ? dl0 : nA;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (le128(s_key[mid - 1], s_key[nA + dl0 - mid])) lo = mid;
-    else hi = mid - 1;
-  }
-  int ia = lo, jb = dl0 - lo;
-  for (int d = dl0; d < dl1; ++d) {
-    const bool takeA = jb >= nB || (ia < nA && le128(s_key[ia], s_key[nA + jb]));
-    if (takeA) {
-      ++ia;
-    } else {
-      const uint64_t an = i0 + ia;  // < n whenever T > 0
-      a.anc[j0 + jb] = (uint32_t)(an < a.n ? an : a.n - 1);
-      ++jb;
-    }
-  }
 }
 
 // ---------------------------------------------------------------------------
@@ -1114,51 +843,69 @@ __device__ __forceinline__ uint64_t strat_first(uint64_t q, uint64_t n, uint64_t
 }
 // ---------------------------------------------------------------------------
 // The paper's Section 3.2 algorithms.
-// Parallelized Cut-Point Search: thread i computes L_i = ceil(n Q_i / T) and
-// writes I_k = i for L_{i-1} <= k < L_i.
+// Parallelized Cut-Point Search: L_i = ceil(n Q_i / T), and I_k = i for
+// L_{i-1} <= k < L_i.  One thread per particle; L_{i-1} comes from the lane
+// below, and a warp stores the ranges longer than 32 together.  (Inside a
+// resampling k_slots builds the same table: L_i is its slot map with r = 0.)
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ uint64_t ceil_nq_over_t(uint64_t n, uint64_t q, uint64_t T) {
-  const U128 X = mul64(n, q);
-  const uint64_t f = div128_small(X, T);
-  const U128 p = mul64(f, T);
-  return (p.hi == X.hi && p.lo == X.lo) ? f : f + 1;
-}
-
 static __global__ void __launch_bounds__(BLOCK) k_cutpoint_search(const uint64_t* Q, uint64_t n,
                                                            uint32_t* I) {
   const uint64_t i = (uint64_t)blockIdx.x * BLOCK + threadIdx.x;
-  if (i >= n) return;
   const uint64_t T = Q[n - 1];
+  const int lane = threadIdx.x & 31;
   if (T == 0) {
-    I[i] = (uint32_t)i;
+    if (i < n) I[i] = (uint32_t)i;
     return;
   }
-  uint64_t Li = ceil_nq_over_t(n, Q[i], T);
-  uint64_t Lp = i == 0 ? 0 : ceil_nq_over_t(n, Q[i - 1], T);
-  Li = Li < n ? Li : n;  // L_i <= n whenever Q_i <= T
-  Lp = Lp < n ? Lp : n;
-  for (uint64_t k = Lp; k < Li; ++k) I[k] = (uint32_t)i;
+  const SysDiv dv = make_sysdiv(T);
+  auto L = [&](uint64_t q) { return sys_first_slot(q, n, 0, dv); };  // at most n
+  const uint64_t l1 = i < n ? L(Q[i]) : n;
+  uint64_t l0 = __shfl_up_sync(0xffffffffu, l1, 1);
+  if (lane == 0) l0 = i == 0 ? 0 : (i < n ? L(Q[i - 1]) : n);
+  const uint64_t cnt = i < n && l1 > l0 ? l1 - l0 : 0;
+  if (cnt <= 32)
+    for (uint64_t k = l0; k < l0 + cnt; ++k) I[k] = (uint32_t)i;
+  uint32_t heavy = __ballot_sync(0xffffffffu, cnt > 32);
+  while (heavy) {
+    const int l = __ffs(heavy) - 1;
+    heavy &= heavy - 1;
+    const uint64_t s0 = __shfl_sync(0xffffffffu, l0, l), s1 = __shfl_sync(0xffffffffu, l1, l);
+    const uint32_t v = (uint32_t)__shfl_sync(0xffffffffu, i, l);
+    for (uint64_t k = s0 + lane; k < s1; k += 32) I[k] = v;
+  }
 }
 
-// Parallelized Cut-Point Method for the scheme's positions: bucket b_j
-// (systematic: j; multinomial: floor(n S_j / S_n)), start at I_{b_j}, climb
-// while KQ_k <= KB_j.
-template <int POS>
-__global__ void __launch_bounds__(BLOCK) k_cutpoint_method(PosArgs a) {
-  if (gated_off(a)) return;
+// Parallelized Cut-Point Method for the systematic positions j T + r (bucket
+// j): start at I_j, climb while n Q_k <= j T + r.  (Multinomial: k_multi.)
+struct PosArgs {
+  const uint64_t* Q;
+  uint32_t* anc;
+  const uint32_t* I;      // cut-point table
+  Ctl* ctl;
+  const uint32_t* t_dev;
+  uint32_t t_arg;
+  uint64_t n;
+  uint64_t seed;
+  uint32_t filter;
+  // adaptive resampling: when set and *gate == 0 this cycle does not
+  // resample, and the kernel returns at once (NULL: always run)
+  const uint32_t* gate;
+};
+static __global__ void __launch_bounds__(BLOCK) k_cutpoint_method_sys(PosArgs a) {
+  if (a.gate && *a.gate == 0u) return;
   const uint64_t j = (uint64_t)blockIdx.x * BLOCK + threadIdx.x;
   if (j >= a.n) return;
-  const PosKeys<POS> K = make_keys<POS>(a);
-  if (K.T == 0 || K.A == 0) {
-    if (j == 0) atomicOr(&a.ctl->err, ERR_NUMERIC);
+  const uint64_t T = a.ctl->keyT;
+  if (T == 0) {  // empty CDF (flagged): keep every index in range
     a.anc[j] = (uint32_t)j;
     return;
   }
-  uint64_t b = j;
-  if (POS == POS_MULTINOMIAL) b = div128_small(mul64(a.n, a.S[j]), K.A);
-  uint64_t k = a.I[b < a.n ? b : a.n - 1];
-  const U128 kb = K.kb(j);
-  while (k < a.n && le128(K.kq(k), kb)) ++k;
+  const uint32_t t = a.t_dev ? *a.t_dev : a.t_arg;
+  const U4 w = draw(a.seed, a.filter, t, 0, P_SYS_OFFSET, 0);
+  const uint64_t r = __umul64hi(((uint64_t)w.b << 32) | w.a, T);
+  uint64_t k = a.I[j];
+  const U128 kb = add128(mul64x32(T, (uint32_t)j), r);
+  while (k < a.n && le128(mul64x32(a.Q[k], (uint32_t)a.n), kb)) ++k;
   a.anc[j] = (uint32_t)(k < a.n ? k : a.n - 1);
 }
 
@@ -1170,7 +917,7 @@ static __global__ void __launch_bounds__(BLOCK) k_cutpoint_method_explicit(
   if (j >= m) return;
   const uint64_t T = Q[n - 1];
   const uint64_t u = U[j];
-  const uint64_t b = T ? div128_small(mul64(n, u), T) : 0;
+  const uint64_t b = T == 0 ? 0 : u < T ? sys_floor_div(mul64x32(u, (uint32_t)n), make_sysdiv(T)) : n;
   uint64_t k = I[b < n ? b : n - 1];
   while (k < n && Q[k] <= u) ++k;
   anc[j] = (uint32_t)(k < n ? k : n - 1);
@@ -1204,6 +951,7 @@ __device__ __forceinline__ double u128_to_f64_rn(U128 v) {
 
 }  // namespace pfk
 #include "slots.cuh"
+#include "multi.cuh"
 namespace pfk {
 
 // ---------------------------------------------------------------------------
@@ -1288,7 +1036,6 @@ __device__ void fold_cycle_warp(const FilterArgs<R>& a, uint32_t t) {
       c->maxenc = ninf;
     }
     c->ticket_w = 0;
-    c->ticket_e = 0;
     c->done_prop = 0;
     c->prop_ticket = 0;
     c->w_ticket = 0;

@@ -62,6 +62,7 @@ struct SlotArgs {
   uint32_t filter;
   double ess_frac;
   void* heavy;            // heavy list, or NULL (no further windows: NONE and binary64)
+  int cut;                // k_slots builds the cut-point table in anc: the slot map with r = 0
   const uint32_t* gate;   // *gate == 0: this cycle does not resample (NULL: it does)
   int src_vec, anc_vec;   // src is 32-byte and anc 16-byte aligned
 };
@@ -321,7 +322,6 @@ static __device__ __noinline__ void sums_last(const SlotArgs& a, uint64_t* s_tot
   if (threadIdx.x == 0) {
     c->done_sums = 0;
     c->keyT = T;
-    c->keyA = a.n;
     if (T == 0) atomicOr(&c->err, ERR_NUMERIC);
     if constexpr (HAS_E && sizeof(R) == 4) {
       es = s_es[0];
@@ -358,7 +358,7 @@ static __device__ __noinline__ void sums_last(const SlotArgs& a, uint64_t* s_tot
   if (threadIdx.x == 96) {
     const uint32_t t = a.t_dev ? *a.t_dev : a.t_arg;
     const U4 wr = draw(a.seed, a.filter, t, 0, P_SYS_OFFSET, 0);
-    const uint64_t r = __umul64hi(((uint64_t)wr.b << 32) | wr.a, T);
+    const uint64_t r = a.cut ? 0ull : __umul64hi(((uint64_t)wr.b << 32) | wr.a, T);
     c->keyR = r;
     c->slot_r32 = div_2by1((r << z) >> 32, (r << z) << 32, Tz);
   }
