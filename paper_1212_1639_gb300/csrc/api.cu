@@ -261,8 +261,6 @@ pf_status launch_resample(int scheme, const MultiArgs& ma, const uint32_t* I, cu
     k_cutpoint_method_sys<<<(unsigned)cdiv(ma.n, BLOCK), BLOCK, 0, s>>>(pa);
     mark(tm, "cutpoint_method", s);
   } else if (scheme == PF_MULTINOMIAL_CUTPOINT) {
-    k_multi_split<<<1, BLOCK, 0, s>>>(ma);  // its constants only
-    mark(tm, "split", s);
     k_multi<true><<<ma.ntiles, BLOCK, 0, s>>>(ma);
     mark(tm, "cutpoint_method", s);
   } else {
@@ -300,6 +298,7 @@ void launch_cdf(pf_filter* f, cudaStream_t s, KTimer* tm) {
   std::memset(&a, 0, sizeof(a));
   a.Q = f->Q;
   a.cut = is_cutpoint(f->scheme);
+  a.multi = is_multinomial(f->scheme);
   a.anc = a.cut ? f->I : f->anc;
   a.pre = f->pre;
   a.part = f->part;
@@ -407,13 +406,13 @@ pf_status enqueue_cycle(pf_filter* f, KTimer* tm = nullptr, const double* y_src 
     k_exp<<<f->exp_grid, BLOCK, 0, s>>>(a);
     mark(tm, "exp", s);
   }
-  launch_cdf<R>(f, s, tm);
   if (fork) {
     CK(cudaStreamWaitEvent(s, f->ev_join, 0));
   } else if (is_multinomial(f->scheme)) {
     spacing(s);
     mark(tm, "spacing_sums", s);
   }
+  launch_cdf<R>(f, s, tm);
   if (is_multinomial(f->scheme) || is_cutpoint(f->scheme)) {
     pf_status st = launch_resample(f->scheme, ma, f->I, s, tm);
     if (st != PF_OK) return st;
@@ -549,7 +548,6 @@ void set_obs(unsigned char* args, bool next, const double* src, double val) {
 constexpr uint64_t SMALL_N32 = (uint64_t)SMALL_M * SMALL_GMAX;
 constexpr uint64_t SMALL_N64 = SMALL_N32 / 2;
 
-template <class R>
 void small_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr, cudaStream_t s) {
   std::memset(cfg, 0, sizeof(*cfg));
   cfg->gridDim = dim3(SMALL_GMAX, 1, 1);
@@ -566,7 +564,7 @@ template <class R>
 bool small_fits() {
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[1];
-  small_config<R>(&cfg, attr, nullptr);
+  small_config(&cfg, attr, nullptr);
   int clusters = 0;
   if (cudaOccupancyMaxActiveClusters(&clusters, k_small<R>, &cfg) != cudaSuccess) {
     cudaGetLastError();
@@ -594,7 +592,7 @@ pf_status launch_small(pf_filter* f, const double* y_dev, const double* y, uint3
   if (est) a.io = f->io_dev;
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[1];
-  small_config<R>(&cfg, attr, f->stream);
+  small_config(&cfg, attr, f->stream);
   CK(cudaLaunchKernelEx(&cfg, k_small<R>, a, sa));
   if (est && f->ess) {
     k_estimate_w<R><<<(unsigned)cdiv(f->n, (uint64_t)BLOCK * EST_PER_THREAD), BLOCK, 0, f->stream>>>(a);
@@ -1324,7 +1322,23 @@ struct WaitDiag {
 
 pf_status run_resample(const float* w, uint64_t n, uint64_t seed, uint32_t filter, uint32_t t,
                        int scheme, uint32_t* anc, uint64_t* Q_out, const Scratch& sc,
-                       cudaStream_t s, WaitDiag dg = WaitDiag()) {
+                       cudaStream_t s, WaitDiag dg = WaitDiag(), uint32_t* host_err = nullptr) {
+  MultiArgs ma;
+  std::memset(&ma, 0, sizeof(ma));
+  ma.Q = sc.Q;
+  ma.pre = sc.pre;
+  ma.spre = sc.spre;
+  ma.splits = sc.splits;
+  ma.anc = anc;
+  ma.I = sc.I;
+  ma.ctl = sc.ctl;
+  ma.t_arg = t;
+  ma.ntiles = slot_tiles(n);
+  ma.n = n;
+  ma.seed = seed;
+  ma.filter = filter;
+  ma.anc_vec = ((uintptr_t)anc & 31) == 0;
+  if (anc && is_multinomial(scheme)) k_spacing_sums<<<ma.ntiles, BLOCK, 0, s>>>(ma);
   const uint64_t want = cdiv(n, 8 * BLOCK);
   const unsigned gmax = (unsigned)(want < 152 * 8 ? want : 152 * 8);
   k_wmax<<<gmax, BLOCK, 0, s>>>(w, n, sc.ctl, ((uintptr_t)w & 31) == 0);
@@ -1336,6 +1350,8 @@ pf_status run_resample(const float* w, uint64_t n, uint64_t seed, uint32_t filte
     a.src = w;
     a.Q = sc.Q;
     a.cut = is_cutpoint(scheme);
+    a.multi = is_multinomial(scheme);
+    a.host_err = host_err;
     a.anc = a.cut ? sc.I : anc;
     a.pre = sc.pre;
     if (pos != SLOTS_NONE) a.heavy = (char*)sc.pre + pre_bytes(n);
@@ -1352,22 +1368,6 @@ pf_status run_resample(const float* w, uint64_t n, uint64_t seed, uint32_t filte
     launch_slots<SRC_W>(pos, a, s);
     CK(cudaGetLastError());
     if (!scheme_needs_Q(scheme)) return PF_OK;
-    MultiArgs ma;
-    std::memset(&ma, 0, sizeof(ma));
-    ma.Q = sc.Q;
-    ma.pre = sc.pre;
-    ma.spre = sc.spre;
-    ma.splits = sc.splits;
-    ma.anc = anc;
-    ma.I = sc.I;
-    ma.ctl = sc.ctl;
-    ma.t_arg = t;
-    ma.ntiles = slot_tiles(n);
-    ma.n = n;
-    ma.seed = seed;
-    ma.filter = filter;
-    ma.anc_vec = ((uintptr_t)anc & 31) == 0;
-    if (is_multinomial(scheme)) k_spacing_sums<<<ma.ntiles, BLOCK, 0, s>>>(ma);
     return launch_resample(scheme, ma, sc.I, s);
   }
   ScanArgs sa;
@@ -1451,19 +1451,35 @@ pf_status small_err_word(uint32_t** host, uint32_t** dev) {
   return PF_OK;
 }
 
-// Systematic and stratified resampling of up to SMALL_N weights: one CTA, one
-// launch, no scratch (k_resample_small), the same ancestors as the general path.
+// Resampling of up to RES_N weights: one cluster, one launch, no scratch
+// (k_small_resample), the same ancestors as the general path.
+bool small_resample_fits() {
+  static const bool fits = [] {
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[1];
+    small_config(&cfg, attr, nullptr);
+    int clusters = 0;
+    if (cudaOccupancyMaxActiveClusters(&clusters, k_small_resample, &cfg) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    return clusters >= 1;
+  }();
+  return fits;
+}
 pf_status resample_small(const float* w, uint64_t n, uint64_t seed, uint32_t filter, uint32_t t,
                          int scheme, uint32_t* anc, cudaStream_t s) {
   uint32_t *eh = nullptr, *ed = nullptr;
   pf_status st = small_err_word(&eh, &ed);
   if (st != PF_OK) return st;
   *(volatile uint32_t*)eh = 0u;
-  if (scheme == PF_STRATIFIED)
-    k_resample_small<true><<<1, SMALL_THREADS, 0, s>>>(w, (uint32_t)n, seed, filter, t, anc, ed);
-  else
-    k_resample_small<false><<<1, SMALL_THREADS, 0, s>>>(w, (uint32_t)n, seed, filter, t, anc, ed);
-  CK(cudaGetLastError());
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr[1];
+  small_config(&cfg, attr, s);
+  const int pos = is_multinomial(scheme) ? SP_MULTI : scheme == PF_STRATIFIED ? SP_STRAT : SP_SYS;
+  const uint32_t m = (uint32_t)(cdiv(cdiv(n, SMALL_GMAX), 32) * 32);
+  CK(cudaLaunchKernelEx(&cfg, k_small_resample, w, (uint32_t)n, m, pos, cdf_shift(n), seed, filter, t,
+                        anc, ed));
   CK(cudaStreamSynchronize(s));
   return map_err(*(volatile uint32_t*)eh);
 }
@@ -1475,11 +1491,16 @@ pf_status resample_common(const float* w, uint64_t n, uint64_t seed, uint32_t fi
   if (n < 1 || n > PF_MAX_PARTICLES) return set_err(PF_ERR_INVALID, "n must be in [1, 2^26]");
   if (scheme < 0 || scheme > 4) return set_err(PF_ERR_INVALID, "bad scheme");
   cudaStream_t s = (cudaStream_t)stream;
-  if (anc && !Q_out && n <= SMALL_N && dg.withhold == NO_TILE &&
-      (scheme == PF_SYSTEMATIC || scheme == PF_STRATIFIED))
+  if (anc && !Q_out && n <= RES_N && dg.withhold == NO_TILE && small_resample_fits())
     return resample_small(w, n, seed, filter, t, scheme, anc, s);
   Scratch sc;
   const bool cdf = !anc;
+  uint32_t *eh = nullptr, *ed = nullptr;
+  if (!cdf) {
+    pf_status se = small_err_word(&eh, &ed);
+    if (se != PF_OK) return se;
+    *(volatile uint32_t*)eh = 0u;
+  }
   const size_t bytes = scratch_layout(n, scheme, cdf, nullptr, &sc);
   void* base = nullptr;
   cudaMemPool_t pool = nullptr;
@@ -1494,13 +1515,21 @@ pf_status resample_common(const float* w, uint64_t n, uint64_t seed, uint32_t fi
   pf_status st = PF_OK;
   if (cudaMemsetAsync(base, 0, scratch_zero_bytes(n, cdf), s) != cudaSuccess)
     st = set_err(PF_ERR_CUDA, "scratch memset failed");
-  if (st == PF_OK) st = run_resample(w, n, seed, filter, t, scheme, anc, Q_out, sc, s, dg);
-  pf_status st2 = PF_OK;
-  if (st == PF_OK) st2 = finish_and_check(sc, s);
+  if (st == PF_OK) st = run_resample(w, n, seed, filter, t, scheme, anc, Q_out, sc, s, dg, ed);
+  if (cdf) {
+    pf_status st2 = PF_OK;
+    if (st == PF_OK) st2 = finish_and_check(sc, s);
+    cudaFreeAsync(base, s);
+    if (st == PF_OK && cudaStreamSynchronize(s) != cudaSuccess)
+      st = set_err(PF_ERR_CUDA, "stream synchronisation failed");
+    return st != PF_OK ? st : st2;
+  }
+  // the scratch goes back in stream order; one synchronisation, after which
+  // the error word (written by the tile sums' last CTA) is complete
   cudaFreeAsync(base, s);
-  if (st == PF_OK && cudaStreamSynchronize(s) != cudaSuccess)
-    st = set_err(PF_ERR_CUDA, "stream synchronisation failed");
-  return st != PF_OK ? st : st2;
+  if (cudaStreamSynchronize(s) != cudaSuccess && st == PF_OK)
+    st = set_err(PF_ERR_CUDA, "stream: %s", cudaGetErrorString(cudaGetLastError()));
+  return st != PF_OK ? st : map_err(*(volatile uint32_t*)eh);
 }
 
 pf_status read_total(const uint64_t* Q, uint64_t n, cudaStream_t s, uint64_t* T) {

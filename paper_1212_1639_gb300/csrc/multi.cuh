@@ -15,6 +15,7 @@
 // weights and the CDF).
 #pragma once
 #include "device.cuh"
+#include "slots.cuh"
 
 namespace pfk {
 
@@ -149,25 +150,11 @@ __device__ __forceinline__ uint64_t warp_last(uint64_t lo, uint64_t hi, F below)
 
 // splits[s] = #{i : Q_i S_n <= S T} for S the spacings before slot tile s, one
 // warp per tile: the CDF tile by its prefix, then the particle in the tile.
-// CTA 0 also writes the constants of the slots' positions: with A = S_n,
-// P = floor((S 2^z) rho / 2^64), rho = floor(T 2^64 / (A 2^z)), A 2^z in
-// [2^63, 2^64); and for the cut-point bucket floor(n S / A) likewise.
 static __global__ void __launch_bounds__(BLOCK) k_multi_split(MultiArgs a) {
   if (a.gate && *a.gate == 0u) return;
-  Ctl* const c = a.ctl;
-  const uint64_t T = c->keyT, A = c->keyS, n = a.n;
+  const uint64_t T = a.ctl->keyT, A = a.ctl->keyS, n = a.n;
   const int lane = threadIdx.x & 31;
-  if (T == 0) {  // empty CDF (flagged)
-    return;
-  }
-  if (blockIdx.x == 0 && lane == 0) {
-    const int z = __clzll((long long)A);
-    if (threadIdx.x == 0) {
-      c->multi_z = z;
-      c->multi_rho = div_2by1(T, 0, A << z);
-    }
-    if (threadIdx.x == 32) c->bucket_rho = div_2by1(n << 32, 0, A << z);
-  }
+  if (T == 0) return;  // empty CDF (flagged)
   const uint32_t s = blockIdx.x * WARPS + (threadIdx.x >> 5);
   if (s > a.ntiles) return;
   const U128 key = mul64(s < a.ntiles ? a.spre[s] : A, T);

@@ -62,6 +62,8 @@ struct SlotArgs {
   uint32_t filter;
   double ess_frac;
   void* heavy;            // heavy list, or NULL (no further windows: NONE and binary64)
+  uint32_t* host_err;     // mapped host word for pf_resample's errors, or NULL
+  int multi;              // multinomial: S_n is known (k_spacing_sums ran before)
   int cut;                // k_slots builds the cut-point table in anc: the slot map with r = 0
   const uint32_t* gate;   // *gate == 0: this cycle does not resample (NULL: it does)
   int src_vec, anc_vec;   // src is 32-byte and anc 16-byte aligned
@@ -323,6 +325,7 @@ static __device__ __noinline__ void sums_last(const SlotArgs& a, uint64_t* s_tot
     c->done_sums = 0;
     c->keyT = T;
     if (T == 0) atomicOr(&c->err, ERR_NUMERIC);
+    if (SRC == SRC_W && a.host_err) *a.host_err = c->err | (c->maxenc == 0 ? ERR_WEIGHTS : 0u);
     if constexpr (HAS_E && sizeof(R) == 4) {
       es = s_es[0];
       for (int w = 1; w < WARPS; ++w) es.add(s_es[w]);
@@ -361,6 +364,19 @@ static __device__ __noinline__ void sums_last(const SlotArgs& a, uint64_t* s_tot
     const uint64_t r = a.cut ? 0ull : __umul64hi(((uint64_t)wr.b << 32) | wr.a, T);
     c->keyR = r;
     c->slot_r32 = div_2by1((r << z) >> 32, (r << z) << 32, Tz);
+  }
+  // multinomial: the constants of the slots' positions (k_multi).  With A = S_n,
+  // P = floor((S 2^z) rho / 2^64), rho = floor(T 2^64 / (A 2^z)), A 2^z in
+  // [2^63, 2^64); and the cut-point bucket n S / A in units of 2^-32 likewise
+  if (a.multi && (threadIdx.x == 128 || threadIdx.x == 160)) {
+    const uint64_t A = c->keyS;
+    const int az = __clzll((long long)A);
+    if (threadIdx.x == 128) {
+      c->multi_z = az;
+      c->multi_rho = div_2by1(T, 0, A << az);
+    } else {
+      c->bucket_rho = div_2by1(a.n << 32, 0, A << az);
+    }
   }
   if (!a.heavy) return;
   const bool any = __syncthreads_or(heavy);  // (the prefixes and constants are written)

@@ -90,6 +90,51 @@ __device__ __forceinline__ uint64_t small_scan(uint64_t v, uint64_t* s, uint64_t
   return off + incl - v;
 }
 
+// The number of particles whose key Q A is not above each of K slots' keys,
+// for Q in the cluster's distributed shared memory (m per CTA, q): first over
+// the CTAs by their last values cum, then by bisection in that CTA's part.  The
+// K bisections go step by step together, so that their loads overlap.
+template <int K, class F>
+__device__ __forceinline__ void cluster_search(const uint64_t* q, const uint64_t* cum, uint32_t G,
+                                               uint32_t m, uint32_t n, const U128* kb, F above,
+                                               uint32_t* out) {
+  uint32_t at[K], lo[K], hi[K];
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    lo[k] = 0;
+    hi[k] = G - 1;
+  }
+  for (uint32_t w = G - 1; w; w >>= 1) {
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      const uint32_t mid = (lo[k] + hi[k]) >> 1;
+      const bool up = lo[k] < hi[k], ab = above(cum[mid], kb[k]);
+      if (up && ab) hi[k] = mid;
+      if (up && !ab) lo[k] = mid + 1;
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    const uint32_t rr = lo[k], b = rr * m;
+    at[k] = dsm_addr(q, rr);
+    out[k] = b;
+    lo[k] = 0;
+    hi[k] = b < n ? (b + m < n ? m : n - b) : 0u;
+  }
+  for (uint32_t w = m; w; w >>= 1) {
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      const uint32_t mid = (lo[k] + hi[k]) >> 1;
+      const bool up = lo[k] < hi[k];
+      const bool ab = up && above(dsm_u64(at[k] + 8 * mid), kb[k]);
+      if (up && ab) hi[k] = mid;
+      if (up && !ab) lo[k] = mid + 1;
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < K; ++k) out[k] = out[k] + lo[k] < n ? out[k] + lo[k] : n - 1;
+}
+
 template <class R>
 struct SmallSmem {
   R e[SMALL_M];                 // e_i
@@ -325,28 +370,33 @@ __global__ void __launch_bounds__(BLOCK) k_small(FilterArgs<R> a, SmallArgs sa) 
       return lt128(kb, multi ? mul64(q, A) : mul64x32(q, n));
     };
     uint32_t an[SMALL_K];
+    if (rs && T > 0) {
+      U128 kb[SMALL_K];
+#pragma unroll
+      for (int k = 0; k < SMALL_K; ++k) {
+        const uint32_t i = tid + k * BLOCK, j = lo + i;
+        kb[k] = U128{0, 0};
+        if (i < cnt) {
+          if (sa.pos == SP_SYS) kb[k] = add128(mul64x32(T, j), r);
+          else if (sa.pos == SP_STRAT) kb[k] = add128(mul64x32(T, j), strat_offset(T, a.seed, a.filter, t, j));
+          else kb[k] = mul64(sm.s[i], T);
+        }
+      }
+      if (m <= BLOCK) {
+        cluster_search<1>(sm.q, sm.cum, G, m, n, kb, above, an);
+      } else {
+#pragma unroll
+        for (int k = 0; k < SMALL_K; k += 2)
+          if (k * BLOCK < m) cluster_search<2>(sm.q, sm.cum, G, m, n, kb + k, above, an + k);
+      }
+    } else {
+#pragma unroll
+      for (int k = 0; k < SMALL_K; ++k) an[k] = lo + tid + k * BLOCK;
+    }
 #pragma unroll
     for (int k = 0; k < SMALL_K; ++k) {
-      const uint32_t i = tid + k * BLOCK, j = lo + i;
-      an[k] = j;
-      if (i < cnt && rs && T > 0) {
-        U128 kb;
-        if (sa.pos == SP_SYS) kb = add128(mul64x32(T, j), r);
-        else if (sa.pos == SP_STRAT) kb = add128(mul64x32(T, j), strat_offset(T, a.seed, a.filter, t, j));
-        else kb = mul64(sm.s[i], T);
-        uint32_t rr = 0;
-        while (rr + 1 < G && !above(sm.cum[rr], kb)) ++rr;
-        const uint32_t qa = dsm_addr(sm.q, rr);
-        uint32_t x0 = 0, x1 = rr * m < n ? (rr * m + m < n ? m : n - rr * m) : 0u;
-        while (x0 < x1) {
-          const uint32_t mid = (x0 + x1) >> 1;
-          if (above(dsm_u64(qa + 8 * mid), kb)) x1 = mid;
-          else x0 = mid + 1;
-        }
-        const uint32_t v = rr * m + x0;
-        an[k] = v < n ? v : n - 1;
-      }
-      if (i < cnt) a.anc[j] = an[k];
+      const uint32_t i = tid + k * BLOCK;
+      if (i < cnt) a.anc[lo + i] = an[k];
     }
     const R ds = (R)sm.c[0], cs = (R)sm.c[1], dt = (R)sm.c[2], ct = (R)sm.c[3];
     const R ks = (R)sm.c[4], kt = (R)sm.c[5];
@@ -433,6 +483,142 @@ __global__ void __launch_bounds__(BLOCK) k_small(FilterArgs<R> a, SmallArgs sa) 
   if (nblk > 1) cluster_sync_all();
   if (rank != 0) return;
   est_fold<R>(a, t1, nblk, c0, c1, c2, sm.est_sum, sm.est_tot);
+}
+
+// ---------------------------------------------------------------------------
+// Resampling of a small weight vector (n <= RES_N) by one cluster, all schemes:
+// the quantisation (W_i = floor(w_i 2^(k - e)), max w = f 2^e), the exact CDF and
+// the positions of the general path, each slot's ancestor by the same search as
+// above -- one launch instead of three to six, no scratch.  Errors go to *err
+// (negative / non-finite / all-zero weights: ERR_WEIGHTS).
+// ---------------------------------------------------------------------------
+constexpr int RES_K = 8;
+constexpr uint32_t RES_M = RES_K * BLOCK;
+constexpr uint64_t RES_N = (uint64_t)RES_M * SMALL_GMAX;
+
+static __global__ void __launch_bounds__(BLOCK) k_small_resample(const float* w, uint32_t n, uint32_t m,
+                                                          int pos, int kshift, uint64_t seed,
+                                                          uint32_t filter, uint32_t t, uint32_t* anc,
+                                                          uint32_t* err) {
+  __shared__ uint64_t s_q[RES_M], s_s[RES_M];
+  __shared__ uint64_t s_warp[WARPS], s_warp2[WARPS], s_cum[SMALL_GMAX];
+  __shared__ uint64_t s_tot, s_stot, s_En;
+  __shared__ uint32_t s_red[WARPS], s_max;  // s_max: the CTA's largest weight; ~0: a bad one
+  const uint32_t tid = threadIdx.x;
+  const int lane = tid & 31, warp = tid >> 5;
+  const uint32_t rank = cluster_ctarank(), G = cluster_nctarank();
+  const uint32_t lo = rank * m < n ? rank * m : n;
+  const uint32_t cnt = lo + m < n ? m : n - lo;
+  float v[RES_K];
+  uint32_t mx = 0;
+#pragma unroll
+  for (int k = 0; k < RES_K; ++k) {
+    const uint32_t i = tid + k * BLOCK;
+    v[k] = i < cnt ? w[lo + i] : 0.0f;
+    mx = max(mx, (!(v[k] >= 0.0f) || !(v[k] < INFINITY)) ? ~0u : __float_as_uint(fabsf(v[k])));
+  }
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  if (lane == 0) s_red[warp] = mx;
+  // meanwhile: multinomial spacings of the CTA's slots (thread t: 8 t .. 8 t + 7)
+  uint64_t Es[RES_K], er = 0;
+  if (pos == SP_MULTI) {
+#pragma unroll
+    for (int h = 0; h < RES_K / 4; ++h) {
+      const uint32_t l0 = lo + RES_K * tid + 4 * h;  // a multiple of four
+      U4 d = {0, 0, 0, 0};
+      if (RES_K * tid + 4 * h < cnt) d = draw(seed, filter, t, l0 >> 2, P_SPACING, 0);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        if (RES_K * tid + 4 * h + e < cnt) er += spacing_E(seed, filter, t, l0 + e, d);
+        Es[4 * h + e] = er;
+      }
+    }
+    if (tid == BLOCK - 1) s_En = spacing_E(seed, filter, t, n, draw(seed, filter, t, n >> 2, P_SPACING, 0));
+  }
+  __syncthreads();
+  if (tid == 0) {
+    for (int i = 1; i < WARPS; ++i) mx = max(mx, s_red[i]);
+    s_max = mx;
+  }
+  cluster_sync_all();  // 1: every CTA's maximum
+  mx = __reduce_max_sync(0xffffffffu, (uint32_t)lane < G ? dsm_u32(dsm_addr(&s_max, lane)) : 0u);
+  const bool wrong = mx == 0u || mx == ~0u;  // (the same in the whole cluster)
+  if (!wrong) {
+    int e2;
+    (void)frexpf(__uint_as_float(mx), &e2);
+#pragma unroll
+    for (int k = 0; k < RES_K; ++k) s_q[tid + k * BLOCK] = quant_weight(v[k], kshift - e2);
+  }
+  __syncthreads();
+  uint64_t run[RES_K], acc = 0;  // thread t: particles 8 t .. 8 t + 7
+#pragma unroll
+  for (int e = 0; e < RES_K; ++e) {
+    acc += wrong ? 0ull : s_q[RES_K * tid + e];
+    run[e] = acc;
+  }
+  uint64_t tot, stot = 0, sexcl = 0;
+  const uint64_t qexcl = small_scan(acc, s_warp, &tot);
+  if (pos == SP_MULTI) sexcl = small_scan(er, s_warp2, &stot);
+  if (tid == 0) {
+    s_tot = tot;
+    s_stot = stot;
+  }
+  cluster_sync_all();  // 2: every CTA's sums (and its maximum has been read)
+  if (wrong) {
+    if (rank == 0 && tid == 0) *err = ERR_WEIGHTS;
+    for (uint32_t i = tid; i < cnt; i += BLOCK) anc[lo + i] = lo + i;
+    return;
+  }
+  uint64_t T, A = n, pre, spre = 0;
+  {
+    const uint64_t x = (uint32_t)lane < G ? dsm_u64(dsm_addr(&s_tot, lane)) : 0ull;
+    const uint64_t in = warp_incl_scan(x, lane);
+    T = __shfl_sync(0xffffffffu, in, 31);
+    pre = __shfl_sync(0xffffffffu, in - x, rank);
+    if (warp == 0 && (uint32_t)lane < G) s_cum[lane] = in;
+  }
+  const bool multi = pos == SP_MULTI;
+  if (multi) {
+    const uint64_t x = (uint32_t)lane < G ? dsm_u64(dsm_addr(&s_stot, lane)) : 0ull;
+    const uint64_t in = warp_incl_scan(x, lane);
+    A = __shfl_sync(0xffffffffu, in, 31) + s_En;
+    spre = __shfl_sync(0xffffffffu, in - x, rank);
+  }
+  uint64_t r = 0;
+  if (pos == SP_SYS) {
+    const U4 d = draw(seed, filter, t, 0, P_SYS_OFFSET, 0);
+    r = __umul64hi(((uint64_t)d.b << 32) | d.a, T);
+  }
+#pragma unroll
+  for (int e = 0; e < RES_K; ++e) {
+    s_q[RES_K * tid + e] = pre + qexcl + run[e];
+    if (multi) s_s[RES_K * tid + e] = spre + sexcl + Es[e];
+  }
+  cluster_sync_all();  // 3: every CTA's CDF
+  auto above = [&](uint64_t q, const U128& kb) {  // Q A > B
+    return lt128(kb, multi ? mul64(q, A) : mul64x32(q, n));
+  };
+  U128 kb[RES_K];
+#pragma unroll
+  for (int k = 0; k < RES_K; ++k) {
+    const uint32_t i = tid + k * BLOCK, j = lo + i;
+    kb[k] = U128{0, 0};
+    if (i < cnt) {
+      if (pos == SP_SYS) kb[k] = add128(mul64x32(T, j), r);
+      else if (pos == SP_STRAT) kb[k] = add128(mul64x32(T, j), strat_offset(T, seed, filter, t, j));
+      else kb[k] = mul64(s_s[i], T);
+    }
+  }
+  uint32_t an[RES_K];
+  if (m <= BLOCK) cluster_search<1>(s_q, s_cum, G, m, n, kb, above, an);
+  else if (m <= 4 * BLOCK) cluster_search<4>(s_q, s_cum, G, m, n, kb, above, an);
+  else cluster_search<RES_K>(s_q, s_cum, G, m, n, kb, above, an);
+#pragma unroll
+  for (int k = 0; k < RES_K; ++k) {
+    const uint32_t i = tid + k * BLOCK;
+    if (i < cnt) anc[lo + i] = an[k];
+  }
+  cluster_sync_all();  // 4: no CTA leaves while others search its part
 }
 
 }  // namespace pfk
