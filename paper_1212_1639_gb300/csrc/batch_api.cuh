@@ -44,6 +44,9 @@ struct pf_batch {
   cudaEvent_t list_ev[kRing] = {};
   uint32_t ring = 0;
   double* est_dev = nullptr;
+  double* est_part = nullptr;        // k_batch_estimate: sums per unit, and finished
+  uint32_t* est_done = nullptr;      // units per slot
+  unsigned sms = 1;
   double* est_pin = nullptr;
   // admission lists (slot + record per admitted filter), a ring of pinned
   // staging buffers so that admitting never waits for cycles in flight
@@ -128,6 +131,8 @@ BatchArgs<R> batch_args(pf_batch* b) {
   a.count = nullptr;
   a.ctr = b->ctr;
   a.est = b->est_dev;
+  a.est_part = b->est_part;
+  a.est_done = b->est_done;
   a.inits = nullptr;
   a.commit = 1;
   return a;
@@ -176,6 +181,7 @@ pf_status batch_shapes(pf_batch* b) {
   CK(cudaGetDevice(&dev));
   CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   if (sms < 1) return set_err(PF_ERR_CUDA, "no multiprocessors");
+  b->sms = (unsigned)sms;
   b->shapes.clear();
   for (int nt : {256, 512}) {
     const unsigned g = resident_grid(b, nt, 1, sms);
@@ -201,6 +207,20 @@ uint32_t big_items(const pf_batch* b, const BatchItem* items, uint32_t cnt) {
   uint32_t k = 0;
   while (k < cnt && b->Fh[items[k].slot].n >= b->big_min) ++k;
   return k;
+}
+
+// Number k_batch_estimate's units of a list (item i's first unit in its pad);
+// returns the grid of its launch.
+unsigned stage_units(const pf_batch* b, char* list, uint32_t cnt) {
+  BatchItem* items = (BatchItem*)(list + 16);
+  uint64_t u = 0;
+  for (uint32_t i = 0; i < cnt; ++i) {
+    items[i].pad = (uint32_t)u;
+    const BatchFilter& f = b->Fh[items[i].slot];
+    u += f.ess_frac > 0.0 ? 1 : cdiv(f.n, (uint64_t)BLOCK * EST_PER_THREAD);
+  }
+  ((uint32_t*)list)[2] = (uint32_t)u;
+  return (unsigned)std::min<uint64_t>(u, 4ull * b->sms);
 }
 
 pf_status check_batch(pf_batch* b) {
@@ -483,6 +503,9 @@ pf_status pf_batch_create(const pf_config* cfgs, uint32_t n, const pf_batch_opts
   if ((st = batch_alloc(b, (size_t)maxf * sizeof(BatchFilter), (void**)&b->F)) != PF_OK) return bail(st);
   if ((st = batch_alloc(b, 256, (void**)&b->ctr)) != PF_OK) return bail(st);
   if ((st = batch_alloc(b, (size_t)maxf * BATCH_EST_ROW * 8, (void**)&b->est_dev)) != PF_OK) return bail(st);
+  const uint64_t units = pool / ((uint64_t)BLOCK * EST_PER_THREAD) + maxf;
+  if ((st = batch_alloc(b, (size_t)units * 6 * 8, (void**)&b->est_part)) != PF_OK) return bail(st);
+  if ((st = batch_alloc(b, (size_t)maxf * 4, (void**)&b->est_done)) != PF_OK) return bail(st);
   for (int r = 0; r <= pf_batch::kRing; ++r) {
     if ((st = batch_alloc(b, list_bytes(maxf), (void**)&b->list_dev[r])) != PF_OK) return bail(st);
     if (cudaHostAlloc((void**)&b->list_pin[r], list_bytes(maxf), cudaHostAllocDefault) != cudaSuccess) {
@@ -508,6 +531,7 @@ pf_status pf_batch_create(const pf_config* cfgs, uint32_t n, const pf_batch_opts
       return bail(set_err(PF_ERR_CUDA, "cudaEventCreate failed"));
   }
   if (cudaMemsetAsync(b->ctr, 0, 256, b->stream) != cudaSuccess ||
+      cudaMemsetAsync(b->est_done, 0, (size_t)maxf * 4, b->stream) != cudaSuccess ||
       cudaMemsetAsync(b->F, 0, (size_t)maxf * sizeof(BatchFilter), b->stream) != cudaSuccess)
     return bail(set_err(PF_ERR_CUDA, "batch memset failed"));
   b->Fh.assign(maxf, BatchFilter());
@@ -726,9 +750,9 @@ pf_status pf_batch_estimate(pf_batch* b, const uint8_t* mask, pf_estimates* out)
   }
   if (cnt == 0) return pf_batch_sync(b);
   *(uint32_t*)lp = cnt;
+  const unsigned grid = stage_units(b, lp, cnt);
   CK(cudaMemcpyAsync(b->list_dev[pf_batch::kRing], lp, 16 + (size_t)cnt * sizeof(BatchItem),
                      cudaMemcpyHostToDevice, b->stream));
-  const unsigned grid = (unsigned)std::min<uint64_t>(cnt, b->grid);
   cudaError_t e;
   if (b->fp64) {
     BatchArgs<double> a = batch_args<double>(b);

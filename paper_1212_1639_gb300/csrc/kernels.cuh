@@ -1724,12 +1724,10 @@ __device__ __forceinline__ void est_block(const StateV<R>& st, uint64_t n, uint3
   __syncthreads();  // (s_sum is reused; the sums are visible to the block)
 }
 
-// The block sums folded and the summaries written and published: thread i sums
-// blocks i, i + BLOCK, ... (a fixed assignment), then a shuffle tree per warp
-// and the warps in order.
-template <class R>
-__device__ __forceinline__ void est_fold(const FilterArgs<R>& a, uint32_t t, uint32_t nblk, R c0, R c1,
-                                         R c2, double (*s_sum)[WARPS], double* s_tot) {
+// The sums of nblk blocks folded into s_tot: thread i sums blocks i, i + BLOCK,
+// ... (a fixed assignment), then a shuffle tree per warp and the warps in order.
+__device__ __forceinline__ void est_fold_sums(const double* part_est, uint32_t nblk,
+                                              double (*s_sum)[WARPS], double* s_tot) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   // (a warp without a block adds zeros, which change no sum: it is left out)
   const int nw = nblk >= BLOCK ? WARPS : (int)((nblk + 31) / 32);
@@ -1737,7 +1735,7 @@ __device__ __forceinline__ void est_fold(const FilterArgs<R>& a, uint32_t t, uin
     double v[6] = {0, 0, 0, 0, 0, 0};
     for (uint32_t b = threadIdx.x; b < nblk; b += BLOCK) {
 #pragma unroll
-      for (int q = 0; q < 6; ++q) v[q] += __ldcg(a.part_est + (uint64_t)b * 6 + q);
+      for (int q = 0; q < 6; ++q) v[q] += __ldcg(part_est + (uint64_t)b * 6 + q);
     }
     if (nblk > 1) {
 #pragma unroll
@@ -1759,6 +1757,13 @@ __device__ __forceinline__ void est_fold(const FilterArgs<R>& a, uint32_t t, uin
     s_tot[threadIdx.x] = v;
   }
   __syncthreads();
+}
+
+// The fold, and the summaries written and published.
+template <class R>
+__device__ __forceinline__ void est_fold(const FilterArgs<R>& a, uint32_t t, uint32_t nblk, R c0, R c1,
+                                         R c2, double (*s_sum)[WARPS], double* s_tot) {
+  est_fold_sums(a.part_est, nblk, s_sum, s_tot);
   if (threadIdx.x == 0) {
     const double cs[3] = {(double)c0, (double)c1, (double)c2};
     a.ctl->est[0] = (double)t;

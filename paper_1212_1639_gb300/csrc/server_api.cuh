@@ -212,12 +212,12 @@ pf_status srv_launch(pf_server* s, uint32_t r, const std::vector<SrvItem>& items
   const uint32_t cnt = (uint32_t)items.size();
   ((uint32_t*)b->list_pin[r])[0] = cnt;
   ((uint32_t*)b->list_pin[r])[1] = big_items(b, li, cnt);
+  const unsigned grid = stage_units(b, b->list_pin[r], cnt);
   CK(cudaMemcpyAsync(b->list_dev[r], b->list_pin[r], 16 + (size_t)cnt * sizeof(BatchItem),
                      cudaMemcpyHostToDevice, b->stream));
   CK(cudaEventRecord(b->list_ev[r], b->stream));
   CK(cudaGraphLaunch(b->exec[r], b->stream));
   b->cycles++;
-  const unsigned grid = (unsigned)std::min<uint64_t>(cnt, b->grid);
   if (b->fp64) {
     BatchArgs<double> a = batch_args<double>(b);
     set_list(a, b->list_dev[r]);
