@@ -103,6 +103,7 @@ struct pf_filter {
   int scheme = 0;
   unsigned prop_grid = 0;  // persistent propagate grid
   unsigned exp_grid = 0;   // binary64: grid of k_exp
+  unsigned boot_grid = 0;  // grid of the bootstrap filter's kernels
   bool small = false;      // whole cycles by one cluster (k_small)
   uint64_t w_cap = 1;      // resident CTAs of the weights kernel
   unsigned prop_grid_fuse = 0;  // the same for the propagation that also weighs
@@ -394,7 +395,7 @@ pf_status enqueue_cycle(pf_filter* f, KTimer* tm = nullptr, const double* y_src 
     CK(cudaEventRecord(f->ev_join, f->side));
   }
   if (f->bootstrap) {  // Algorithm "Particle Filtering": propagate blind, then weigh
-    k_boot_pw<R><<<(unsigned)cdiv(n, BLOCK), BLOCK, 0, s>>>(a);
+    k_boot_pw<R><<<f->boot_grid, BLOCK, 0, s>>>(a);
     mark(tm, "propagate_weights", s);
   } else if (form_weighs(form)) {
     const unsigned wg = weights_grid<R>(n, f->w_cap);
@@ -422,7 +423,7 @@ pf_status enqueue_cycle(pf_filter* f, KTimer* tm = nullptr, const double* y_src 
   // binary32: slots handed out by ticket when each warp has many 64-slot units
   const bool dyn = (n + 63) / 64 >= (uint64_t)PROP_DYN * pg * WARPS;
   if (f->bootstrap) {
-    k_boot_gather<R><<<(unsigned)cdiv(n, BLOCK), BLOCK, 0, s>>>(a);
+    k_boot_gather<R><<<f->boot_grid, BLOCK, 0, s>>>(a);
     mark(tm, "gather", s);
   } else if (f->ess) {  // adaptive resampling (never fused)
     if constexpr (sizeof(R) == 4) {
@@ -583,6 +584,7 @@ pf_status launch_small(pf_filter* f, const double* y_dev, const double* y, uint3
   sa.pos = is_multinomial(f->scheme) ? SP_MULTI : f->scheme == PF_STRATIFIED ? SP_STRAT : SP_SYS;
   sa.learn = f->learn;
   sa.ess = f->ess;
+  sa.boot = f->bootstrap;
   sa.est = est && !f->ess;
   sa.m = (uint32_t)(cdiv(cdiv(f->n, SMALL_GMAX), 32) * 32);
   sa.steps = steps;
@@ -812,6 +814,8 @@ pf_status pf_create(const pf_config* cfg, pf_filter** out) {
     const uint64_t want = cdiv(n, f->fp64 ? 32ull : 2ull * BLOCK),
                    cap = (uint64_t)per_sm * (uint64_t)sms;
     f->prop_grid = (unsigned)(want < cap ? want : cap);
+    const uint64_t bw = cdiv(n, f->fp64 ? 32 : BLOCK);
+    f->boot_grid = (unsigned)(bw < 8ull * sms ? bw : 8ull * sms);
     f->exp_grid = (unsigned)(want < 8ull * sms ? want : 8ull * sms);
     int per_sm_f = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_f, prop_fuse_fn(f), BLOCK, 0);
@@ -824,7 +828,7 @@ pf_status pf_create(const pf_config* cfg, pf_filter** out) {
     f->w_cap = (uint64_t)per_sm_w * (uint64_t)sms;
     f->prop_grid_fuse = (unsigned)(want < cap_f ? want : cap_f);
   }
-  f->small = !f->bootstrap && n <= (f->fp64 ? SMALL_N64 : SMALL_N32) &&
+  f->small = n <= (f->fp64 ? SMALL_N64 : SMALL_N32) &&
              (f->fp64 ? small_fits<double>() : small_fits<float>());
   if (!f->small && (st = build_graph(f, CF_PLAIN)) != PF_OK) return bail(st);
   *out = f;

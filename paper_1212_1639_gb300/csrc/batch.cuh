@@ -324,9 +324,20 @@ __device__ __forceinline__ void batch_filter(const BatchArgs<R>& a, const BatchI
             if (ess) lam4[e] = a.lam[off + i + e];
           }
         }
+        if constexpr (sizeof(R) == 4) {
+#pragma unroll
+          for (int e = 0; e < 4; e += 2) {
+            const float2 l = log_pred2(make_float2(xv[e], xv[e + 1]), make_float2(sv[e], sv[e + 1]),
+                                       make_float2(tv[e], tv[e + 1]), yr);
+            lv[e] = l.x;
+            lv[e + 1] = l.y;
+          }
+        } else {
+#pragma unroll
+          for (int e = 0; e < 4; ++e) lv[e] = log_pred<R>(xv[e], sv[e], tv[e], yr);
+        }
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-          lv[e] = log_pred<R>(xv[e], sv[e], tv[e], yr);
           if (ess) lv[e] = lam4[e] + lv[e];  // adaptive filters: L = lambda + l
           fail |= !(lv[e] < (R)INFINITY);  // NaN or +inf
           mx = fmax(mx, lv[e]);
@@ -900,6 +911,7 @@ __device__ __forceinline__ void batch_filter(const BatchArgs<R>& a, const BatchI
     // round-robin over the group), the two slots sharing draw B (reading 19)
     // and each paired FMUL2 / FFMA2: the operations of the single-filter
     // paired propagation, lane by lane the scalar ones, so the same bits
+    const bool wide = ig_wide(ds, dt);
     const uint64_t np = (n + 1) / 2, ppstride = (uint64_t)G * NT;
     // the ancestors of a pair (clamped into range), loaded a pass ahead
     auto anc_of = [&](uint64_t jj) -> uint32_t {
@@ -923,11 +935,10 @@ __device__ __forceinline__ void batch_filter(const BatchArgs<R>& a, const BatchI
         const float2 ta = make_float2(c0.t2, c1.t2);
         // V and mu share one correctly rounded reciprocal of s = sigma^2 + tau^2
         const float2 sp = addp(sa, ta);
-        const float2 ri = make_float2(__frcp_rn(sp.x), __frcp_rn(sp.y));
-        const float2 V = mul2(mul2(sa, ta), ri);
+        float2 ri, sv;
+        state_scale2(sa, ta, sp, &ri, &sv);
         const float2 nn = fma2(xa, sa, mul2(splat2(yr), ta));
         const float2 mu = mul2(nn, ri);
-        const float2 sv = make_float2(sqrtf(V.x), sqrtf(V.y));
         float2 Z;
         theta_draws2(sm.rk, fid, t, (uint32_t)kp, &Z, &Zs, &Us, &Zt, &Ut);
         const float2 xj = fma2(sv, Z, mu);
@@ -978,7 +989,8 @@ __device__ __forceinline__ void batch_filter(const BatchArgs<R>& a, const BatchI
                                   splat2(0x1p-32f),
                                   make_float2(__uint2float_rn((uint32_t)(bt0 >> 32)),
                                               __uint2float_rn((uint32_t)(bt1 >> 32))));
-          const float q0 = bsf.x / Gs.x, r0 = btf.x / Gt.x, q1 = bsf.y / Gs.y, r1 = btf.y / Gt.y;
+          const float2 qs = ig2(bsf, Gs, wide), qt = ig2(btf, Gt, wide);
+          const float q0 = qs.x, r0 = qt.x, q1 = qs.y, r1 = qt.y;
           ds0 = !as0; dt0 = !at0; ds1 = v1 && !as1; dt1 = v1 && !at1;
           if (v1 && as0 && as1) {
             *reinterpret_cast<float2*>(dst.s2 + d) = make_float2(q0, q1);

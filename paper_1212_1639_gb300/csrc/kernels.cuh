@@ -294,6 +294,18 @@ __device__ __forceinline__ R log_pred(R x, R s2, R t2, R y) {
   return (R)-0.5 * sum;
 }
 
+// log_pred on two particles with paired operations; per lane the same IEEE
+// operations in the same order, so the same bits.
+__device__ __forceinline__ float2 log_pred2(float2 x, float2 s2, float2 t2, float yn) {
+  const float2 s = add2(s2, t2);
+  const float2 dx = sub2(splat2(yn), x);
+  const float2 q = mul2(dx, dx);
+  const float2 lg = det_log2(s);
+  const float2 r = pair_safe(s, q) ? div_rn2(q, s) : make_float2(q.x / s.x, q.y / s.y);
+  const float2 sum = add2(lg, r);
+  return mul2(splat2(-0.5f), sum);
+}
+
 // Running maximum of log-likelihoods and whether one was NaN or +inf (such a
 // value is left out of the maximum; the cycle fails).  Binary64 keeps the
 // order-preserving signed integer of the value, so that neither the comparison
@@ -414,8 +426,17 @@ __global__ void __launch_bounds__(BLOCK, W_CTAS_PER_SM) k_weights(FilterArgs<R> 
         VW::get(*reinterpret_cast<const V*>(a.lam + i0), lm);
         VW::get(*reinterpret_cast<const V*>(a.lam + i1), lm + NV);
       }
+      if constexpr (sizeof(R) == 4) {
 #pragma unroll
-      for (int e = 0; e < 2 * NV; ++e) lv[e] = weigh(xv[e], sv[e], tv[e], ESS ? lm[e] : (R)0);
+        for (int e = 0; e < 2 * NV; e += 2) {
+          const float2 l = log_pred2(make_float2(xv[e], xv[e + 1]), make_float2(sv[e], sv[e + 1]),
+                                     make_float2(tv[e], tv[e + 1]), yr);
+          lv[e] = ESS ? lm[e] + l.x : l.x;
+          lv[e + 1] = ESS ? lm[e + 1] + l.y : l.y;
+          top.take(lv[e]);
+          top.take(lv[e + 1]);
+        }
+      }
       *reinterpret_cast<V*>(a.ell + i0) = VW::make(lv);
       *reinterpret_cast<V*>(a.ell + i1) = VW::make(lv + NV);
     } else {
@@ -487,22 +508,20 @@ __global__ void __launch_bounds__(BLOCK) k_boot_pw(FilterArgs<R> a) {
     c->y = y;
     c->yf = (float)y;
   }
-  R mx = (R)-INFINITY;
-  bool bad = false;
-  const uint64_t i = (uint64_t)blockIdx.x * BLOCK + threadIdx.x;
-  if (i < a.n) {
+  MaxL<R> top;
+  const uint64_t stride = (uint64_t)gridDim.x * BLOCK;
+  for (uint64_t i = sizeof(R) == 8 ? spread_slot() : (uint64_t)blockIdx.x * BLOCK + threadIdx.x; i < a.n; i += stride) {
     const R Z = bm_normal(draw(a.seed, a.filter, t, (uint32_t)i, P_BOOT_STATE, 0), (R)0);
     const R sv = sqrt_rn(st.t2[i]);
     const R xz = sv * Z;
     const R xp = st.x[i] + xz;
     st.x[i] = xp;
     const R l = log_pred<R>(xp, st.s2[i], (R)0, yr);
-    bad = !(l < (R)INFINITY);  // NaN or +inf
-    mx = l;
+    top.take(l);
     a.ell[i] = l;
   }
-  if (bad) atomicOr(&c->err, ERR_NUMERIC);
-  mx = block_max<R>(mx, s_red);
+  if (top.bad) atomicOr(&c->err, ERR_NUMERIC);
+  const R mx = block_max<R>(top.value(), s_red);
   if (threadIdx.x == 0 && mx > (R)-INFINITY) atomicMax(&c->maxenc, enc_max(mx));
 }
 
@@ -1103,6 +1122,30 @@ __device__ __forceinline__ void wq_drain(Item* q, uint32_t& qn, uint32_t lo, int
   }
 }
 
+// The propagation's shared reciprocal 1 / s of s = sigma^2 + tau^2 and
+// sqrt(V), V = (sigma^2 tau^2) / s, of a slot pair.
+__device__ __forceinline__ void state_scale2(float2 sa, float2 ta, float2 s, float2* ri, float2* sv) {
+  const float2 p = mul2(sa, ta);
+  if (pair_safe(sa, ta)) {  // then s and V lie within [2^-81, 2^41] too
+    *ri = rcp_rn2(s);
+    *sv = sqrt_rn2(mul2(p, *ri));
+  } else {
+    *ri = make_float2(__frcp_rn(s.x), __frcp_rn(s.y));
+    const float2 V = mul2(p, *ri);
+    *sv = make_float2(sqrtf(V.x), sqrtf(V.y));
+  }
+}
+// The inverse-gamma quotients b / G of a slot pair.  b is 0 or in [2^-32, 2^32);
+// an accepted draw has G = d v^3 with v above 0.04 (the squeeze bounds |Z|) and
+// below 4, so for shapes below 2^60 both operands and the quotient are far from
+// the ends of the range (the quotient of a draw that missed the squeeze is not
+// used).  wide: a larger shape (the same in every thread).
+__device__ __forceinline__ bool ig_wide(float ds, float dt) { return !(ds < 0x1p60f && dt < 0x1p60f); }
+__device__ __forceinline__ float2 ig2(float2 b, float2 G, bool wide) {
+  if (wide) return make_float2(b.x / G.x, b.y / G.y);
+  return div_rn2(b, G);
+}
+
 // The next cycle's weight of one slot: l = log p(y_{t+2} | x, sigma^2, tau^2),
 // the weights kernel's arithmetic; its maximum and finiteness are tracked.
 template <class R>
@@ -1112,18 +1155,6 @@ __device__ __forceinline__ void weigh_next(R* ell, uint64_t j, R x, R s2, R t2, 
   ell[j] = l;
   bad |= !(l < (R)INFINITY);
   mx = fmax(mx, l);
-}
-
-// log_pred on two slots with paired operations; per lane the same IEEE
-// operations in the same order, so the same bits.
-__device__ __forceinline__ float2 log_pred2(float2 x, float2 s2, float2 t2, float yn) {
-  const float2 s = add2(s2, t2);
-  const float2 dx = sub2(splat2(yn), x);
-  const float2 q = mul2(dx, dx);
-  const float2 lg = det_log2(s);
-  const float2 r = make_float2(q.x / s.x, q.y / s.y);
-  const float2 sum = add2(lg, r);
-  return mul2(splat2(-0.5f), sum);
 }
 
 // Store a next-cycle weight computed elsewhere and track it.
@@ -1345,6 +1376,7 @@ __global__ void __launch_bounds__(BLOCK, 3) k_propagate2(FilterArgs<float> a) {
   const StateV<float> dst = (t & 1) ? a.st[0] : a.st[1];
   const float yr = c->yf, ds = c->mtf[0], cs = c->mtf[1], dt = c->mtf[2], ct = c->mtf[3];
   const float ks = c->mtf[4], kt = c->mtf[5];
+  const bool wide = ig_wide(ds, dt);
   const int lane = threadIdx.x & 31;
   Item* const wq = s_q[threadIdx.x >> 5];
   uint32_t qn = 0;  // warp-uniform
@@ -1446,11 +1478,10 @@ __global__ void __launch_bounds__(BLOCK, 3) k_propagate2(FilterArgs<float> a) {
       const float2 ta = make_float2(c0.t2, c1.t2);
       // V and mu share one correctly rounded reciprocal of s = sigma^2 + tau^2
       const float2 sm = addp(sa, ta);
-      const float2 ri = make_float2(__frcp_rn(sm.x), __frcp_rn(sm.y));
-      const float2 V = mul2(mul2(sa, ta), ri);
+      float2 ri, sv;
+      state_scale2(sa, ta, sm, &ri, &sv);
       const float2 nn = fma2(xa, sa, mul2(splat2(yr), ta));
       const float2 mu = mul2(nn, ri);
-      const float2 sv = make_float2(sqrtf(V.x), sqrtf(V.y));
       float2 Z, Zs, Us, Zt, Ut;
       theta_draws2(a.rk, a.filter, t, (uint32_t)(j0 >> 1), &Z, &Zs, &Us, &Zt, &Ut);
       const float2 xj = fma2(sv, Z, mu);
@@ -1507,7 +1538,8 @@ __global__ void __launch_bounds__(BLOCK, 3) k_propagate2(FilterArgs<float> a) {
                                 splat2(0x1p-32f),
                                 make_float2(__uint2float_rn((uint32_t)(bt0 >> 32)),
                                             __uint2float_rn((uint32_t)(bt1 >> 32))));
-        const float q0 = bsf.x / Gs.x, r0 = btf.x / Gt.x, q1 = bsf.y / Gs.y, r1 = btf.y / Gt.y;
+        const float2 qs = ig2(bsf, Gs, wide), qt = ig2(btf, Gt, wide);
+        const float q0 = qs.x, r0 = qt.x, q1 = qs.y, r1 = qt.y;
         ds0 = v0 && !as0; dt0 = v0 && !at0; ds1 = v1 && !as1; dt1 = v1 && !at1;
         if (v1 && as0 && as1) {
           *reinterpret_cast<float2*>(dst.s2 + j0) = make_float2(q0, q1);
@@ -1593,8 +1625,11 @@ __global__ void __launch_bounds__(BLOCK) k_boot_gather(FilterArgs<R> a) {
   const StateV<R> src = (t & 1) ? a.st[1] : a.st[0];
   const StateV<R> dst = (t & 1) ? a.st[0] : a.st[1];
   const uint64_t n = a.n;
-  const uint64_t j = (uint64_t)blockIdx.x * BLOCK + threadIdx.x;
-  if (j < n) {
+  // (grid-stride and one completion count per CTA: a count per warp of a grid of
+  // all slots, 32,768 atomics on one word at N = 2^20, held the kernel at 37 us)
+  const uint64_t stride = (uint64_t)gridDim.x * BLOCK;
+#pragma unroll 2
+  for (uint64_t j = (uint64_t)blockIdx.x * BLOCK + threadIdx.x; j < n; j += stride) {
     uint32_t an = a.anc[j];
     an = an < n ? an : (uint32_t)(n - 1);
     dst.x[j] = src.x[an];
@@ -1603,9 +1638,10 @@ __global__ void __launch_bounds__(BLOCK) k_boot_gather(FilterArgs<R> a) {
     dst.bs[j] = src.bs[an];
     dst.bt[j] = src.bt[an];
   }
-  const int lane = threadIdx.x & 31;
+  __syncthreads();  // every warp has read t
+  if (threadIdx.x >= 32) return;
   bool last = false;
-  if (lane == 0) last = atomicAdd(&a.ctl->done_prop, 1u) == gridDim.x * WARPS - 1;
+  if (threadIdx.x == 0) last = atomicAdd(&a.ctl->done_prop, 1u) == gridDim.x - 1;
   last = __shfl_sync(0xffffffffu, last, 0);
   if (last) fold_cycle_warp<R>(a, t);
 }

@@ -28,7 +28,8 @@ enum SmallPos : int { SP_SYS = 0, SP_STRAT = 1, SP_MULTI = 2 };
 
 struct SmallArgs {
   int pos;                 // SmallPos (the cut-point schemes give the same ancestors)
-  int learn, ess, est;     // est: the summaries after the last cycle
+  int learn, ess, boot;    // boot: Algorithm "Particle Filtering"
+  int est;                 // the summaries after the last cycle
   uint32_t m;              // particles per CTA, a multiple of 32
   uint32_t steps;
   double ess_frac;
@@ -189,7 +190,15 @@ __global__ void __launch_bounds__(BLOCK) k_small(FilterArgs<R> a, SmallArgs sa) 
       l[k] = (R)-INFINITY;
       if (i < cnt) {
         const uint32_t g = lo + i;
-        l[k] = log_pred<R>(__ldcg(src.x + g), __ldcg(src.s2 + g), __ldcg(src.t2 + g), yr);
+        const R s2 = __ldcg(src.s2 + g), t2 = __ldcg(src.t2 + g);
+        R x = __ldcg(src.x + g);
+        if (sa.boot) {  // propagate blind, in place (k_boot_pw)
+          const R Z = bm_normal(draw(a.seed, a.filter, t, g, P_BOOT_STATE, 0), (R)0);
+          const R xz = sqrt_rn(t2) * Z;
+          x = x + xz;
+          src.x[g] = x;
+        }
+        l[k] = log_pred<R>(x, s2, sa.boot ? (R)0 : t2, yr);
         if (ess) l[k] = a.lam[g] + l[k];
         top.take(l[k]);
       }
@@ -422,6 +431,14 @@ __global__ void __launch_bounds__(BLOCK) k_small(FilterArgs<R> a, SmallArgs sa) 
         for (int q = 1; q < SMALL_K; ++q)
           if (q == k) cur = rec[q];
         const R xa = cur.x, s2 = cur.s2, t2 = cur.t2;
+        if (sa.boot) {  // Step 3: the ancestor as it is
+          dst.x[j] = xa;
+          dst.s2[j] = s2;
+          dst.t2[j] = t2;
+          dst.bs[j] = cur.bs;
+          dst.bt[j] = cur.bt;
+          continue;
+        }
         // V and mu share one correctly rounded reciprocal of s
         const R s = s2 + t2;
         const R ri = div_rn((R)1, s);

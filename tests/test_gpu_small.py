@@ -64,3 +64,16 @@ def test_small_blocks_and_forms(pf, orc, kw):
         o.step(v)
     _same(g, o, "fp32")
     assert e == g.estimate()
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+@pytest.mark.parametrize("n", [1, 300, 4096, 10_000])
+def test_small_and_general_bootstrap(pf, orc, n, prec):
+    _, y = synth.local_level_series(8, 7)
+    kw = dict(seed=n, known_variances=True, sigma2=0.8, tau2=0.3)
+    g = pf.Filter(n, scheme="stratified", precision=prec, algorithm="bootstrap", **kw)
+    o = orc.Filter(orc.make_config(n, scheme=pf.SCHEMES["stratified"], precision=int(prec == "fp64"), algorithm=1, **kw))
+    g.run(y)
+    for v in y:
+        o.step(v)
+    _same(g, o, prec)
