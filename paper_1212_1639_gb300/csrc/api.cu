@@ -345,11 +345,17 @@ void launch_cdf(pf_filter* f, cudaStream_t s, KTimer* tm) {
 // With form CF_HEAD / CF_MID the propagation also computes the next cycle's
 // weights against y_{t+2} (*ynx_src when set, else ynx_val); with CF_MID /
 // CF_TAIL the weights kernel is left out, its work done by the previous cycle.
-// The binary32 propagation with or without slots handed out by ticket.
+// The binary32 propagation, slots handed out by ticket in the learning forms
+// where each warp has many 64-slot units (PROP_DYN).
 template <bool LEARN, bool FUSE, bool ESS>
-void launch_prop2(bool dyn, unsigned grid, cudaStream_t s, const FilterArgs<float>& a) {
-  if (dyn) k_propagate2<LEARN, FUSE, ESS, true><<<grid, BLOCK, 0, s>>>(a);
-  else k_propagate2<LEARN, FUSE, ESS, false><<<grid, BLOCK, 0, s>>>(a);
+void launch_prop2(unsigned grid, cudaStream_t s, const FilterArgs<float>& a) {
+  if constexpr (LEARN && !FUSE) {
+    if ((a.n + 63) / 64 >= (uint64_t)(ESS ? PROP_DYN_ESS : PROP_DYN) * grid * WARPS) {
+      k_propagate2<LEARN, FUSE, ESS, true><<<grid, BLOCK, 0, s>>>(a);
+      return;
+    }
+  }
+  k_propagate2<LEARN, FUSE, ESS, false><<<grid, BLOCK, 0, s>>>(a);
 }
 template <class R>
 pf_status enqueue_cycle(pf_filter* f, KTimer* tm = nullptr, const double* y_src = nullptr,
@@ -420,26 +426,24 @@ pf_status enqueue_cycle(pf_filter* f, KTimer* tm = nullptr, const double* y_src 
   }
   const bool fuse = !f->bootstrap && !f->ess && form_fuses(form);
   const unsigned pg = fuse ? f->prop_grid_fuse : f->prop_grid;
-  // binary32: slots handed out by ticket when each warp has many 64-slot units
-  const bool dyn = (n + 63) / 64 >= (uint64_t)PROP_DYN * pg * WARPS;
   if (f->bootstrap) {
     k_boot_gather<R><<<f->boot_grid, BLOCK, 0, s>>>(a);
     mark(tm, "gather", s);
   } else if (f->ess) {  // adaptive resampling (never fused)
     if constexpr (sizeof(R) == 4) {
-      if (f->learn) launch_prop2<true, false, true>(dyn, pg, s, a);
-      else launch_prop2<false, false, true>(dyn, pg, s, a);
+      if (f->learn) launch_prop2<true, false, true>(pg, s, a);
+      else launch_prop2<false, false, true>(pg, s, a);
     } else {
       if (f->learn) k_propagate<R, true, false, true><<<pg, BLOCK, 0, s>>>(a);
       else k_propagate<R, false, false, true><<<pg, BLOCK, 0, s>>>(a);
     }
   } else if constexpr (sizeof(R) == 4) {  // binary32: two slots per thread, paired arithmetic
     if (f->learn) {
-      if (fuse) launch_prop2<true, true, false>(dyn, pg, s, a);
-      else launch_prop2<true, false, false>(dyn, pg, s, a);
+      if (fuse) launch_prop2<true, true, false>(pg, s, a);
+      else launch_prop2<true, false, false>(pg, s, a);
     } else {
-      if (fuse) launch_prop2<false, true, false>(dyn, pg, s, a);
-      else launch_prop2<false, false, false>(dyn, pg, s, a);
+      if (fuse) launch_prop2<false, true, false>(pg, s, a);
+      else launch_prop2<false, false, false>(pg, s, a);
     }
   } else {
     if (f->learn) {
@@ -463,15 +467,11 @@ pf_status enqueue_cycle(pf_filter* f, KTimer* tm = nullptr, const double* y_src 
   return PF_OK;
 }
 
-// The propagation that also computes the next cycle's weights (binary32:
-// the form with slots handed out by ticket when dyn).
-const void* prop_fuse_fn(const pf_filter* f, bool dyn = false) {
+// The propagation that also computes the next cycle's weights.
+const void* prop_fuse_fn(const pf_filter* f) {
   if (f->fp64)
     return f->learn ? (const void*)k_propagate<double, true, true>
                     : (const void*)k_propagate<double, false, true>;
-  if (dyn)
-    return f->learn ? (const void*)k_propagate2<true, true, false, true>
-                    : (const void*)k_propagate2<false, true, false, true>;
   return f->learn ? (const void*)k_propagate2<true, true> : (const void*)k_propagate2<false, true>;
 }
 
@@ -500,7 +500,6 @@ pf_status build_graph(pf_filter* f, int form) {
       : f->ess     ? (f->fp64 ? (const void*)k_weights<double, true> : (const void*)k_weights<float, true>)
                    : (f->fp64 ? (const void*)k_weights<double> : (const void*)k_weights<float>);
   const void* pfun = prop_fuse_fn(f);
-  const void* pfun_dyn = prop_fuse_fn(f, true);
   const size_t asz = f->fp64 ? sizeof(FilterArgs<double>) : sizeof(FilterArgs<float>);
   for (cudaGraphNode_t nd : nodes) {
     cudaGraphNodeType ty;
@@ -515,7 +514,7 @@ pf_status build_graph(pf_filter* f, int form) {
       G.wkp[0] = G.wargs;
       G.wparams.kernelParams = G.wkp;
       G.wparams.extra = nullptr;
-    } else if (p.func == pfun || p.func == pfun_dyn) {
+    } else if (p.func == pfun) {
       G.pnode = nd;
       G.pparams = p;
       std::memcpy(G.pargs, p.kernelParams[0], asz);

@@ -1358,16 +1358,28 @@ __global__ void __launch_bounds__(BLOCK, 3) k_propagate(FilterArgs<R> a) {
 // ---------------------------------------------------------------------------
 constexpr uint32_t WQ2_CAP = 160;  // 31 queued + 4 pushes of 32 per pass
 // k_propagate2's units of 64 slots: with DYN handed out by ticket, PROP_GRAB
-// at a time; the launch takes DYN when there are at least PROP_DYN per warp
+// at a time.  Tickets even out the warps' finishing times, but each batch waits
+// for an atomic and costs the address arithmetic of an arbitrary unit, so they
+// pay only where a warp has many units: the launch takes DYN from PROP_DYN units
+// per warp (PROP_DYN_ESS with adaptive resampling), learning forms only.  Cycle
+// in us, fixed / by ticket: N = 2^22 105.9 / 111.0, 2^23 193.4 / 196.6, 2^24
+// 366.1 / 365.7, 2^25 709.6 / 700.4; adaptive 2^22 121.6 / 126.0, 10^7 260.4 /
+// 260.1, 2^24 419.2 / 413.8.  Fixed is the faster at every size with FUSE (2^22
+// 108.0 / 119.0, 2^24 365.0 / 387.6, 2^26 1390 / 1453) and with known variances
+// (2^22 88.6 / 96.3, 2^24 299.7 / 314.7, 2^26 1140 / 1210), which therefore have
+// no ticket form.
 constexpr uint32_t PROP_GRAB = 4;
-constexpr uint32_t PROP_DYN = 16;
+constexpr uint32_t PROP_DYN = 68, PROP_DYN_ESS = 44;
 
 // With FUSE, the next cycle's weights as in k_propagate, the two slots of a
 // pass weighed by paired operations.
 // 3 CTAs per SM (up to 85 registers, no spills): measured faster at N = 2^24
 // than 4 CTAs at 64 registers, where the plain form spills.
+// As 128 threads x 7 CTAs the cycle of 2^24 takes 0.4 % less, but the adaptive
+// one of 2^20 4 % and the fused one of 2.6 million 3 % more.
 template <bool LEARN, bool FUSE = false, bool ESS = false, bool DYN = false>
 __global__ void __launch_bounds__(BLOCK, 3) k_propagate2(FilterArgs<float> a) {
+  static_assert(!DYN || (LEARN && !FUSE), "tickets: learning forms without FUSE");
   typedef GammaItem<float> Item;
   __shared__ Item s_q[WARPS][WQ2_CAP];
   const Ctl* c = a.ctl;
