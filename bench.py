@@ -55,17 +55,17 @@ L2_FLUSH_BYTES = 256 << 20
 # read and write for the method, the roofline numerators:
 BYTES_PER_PARTICLE = {
     "weights": 12 + 4,            # read x, sigma2, tau2; write l
-    "scan": 4 + 8,                # read l; write Q
-    "spacing_scan": 8,            # write S
-    "partition": 0,               # one merge-path split per 2048 merged elements
-    "merge_systematic": 8 + 4,    # read Q; write ancestors
-    "stratified": 8 + 4,          # read Q; write ancestors
-    "merge_multinomial": 8 + 8 + 4,  # read Q and S; write ancestors
-    "cutpoint_search": 8 + 4,     # read Q; write I
+    "exp": 0,                     # binary64: exp(l - max) for the tile sums (an intermediate)
+    "cdf_sums": 4,                # read l (the exponentials it leaves for the next kernel are
+                                  # an intermediate and not counted)
+    "cdf": 8,                     # write Q
+    "cdf_resample": 8 + 4,        # write Q; write ancestors
+    "cutpoint_search": 8 + 4,     # write Q; write I
+    "spacing_sums": 0,            # one sum per tile of slots
+    "split": 0,                   # one search per tile of slots
+    "merge": 8 + 4,               # read Q; write ancestors
     "cutpoint_method": 4 + 8 + 4,  # read I, Q at the start; write ancestors
     "propagate": 4 + 28 + 28,     # read ancestor; gather 28 B record; write 28 B record
-    "cdf_resample": 4 + 8 + 4,   # read l; write Q; write ancestors (l is read twice, the
-                                  # second time mostly from L2)
     "propagate_weights_next": 4 + 28 + 28 + 4,  # propagate, and write the next cycle's l
     "estimate": 12,               # read x, sigma2, tau2 (posterior summaries)
 }
@@ -175,7 +175,7 @@ def pow2_label(n):
 
 def kernels_hash():
     h = hashlib.sha256()
-    for f in ("kernels.cuh", "device.cuh"):
+    for f in ("kernels.cuh", "slots.cuh", "device.cuh"):
         h.update(open(os.path.join(ROOT, "paper_1212_1639_gb300", "csrc", f), "rb").read())
     return h.hexdigest()[:16]
 
@@ -421,17 +421,12 @@ def bench_ours(args):
     kernels = {}
     hbm, hbm_kind = peaks()
     for kname, kms in prof.items():
-        key = kname
-        if kname == "merge":
-            key = "merge_multinomial" if "multinomial" in args.scheme else "merge_systematic"
-        byts = BYTES_PER_PARTICLE[key] * n
+        byts = BYTES_PER_PARTICLE[kname] * n
         kernels[kname] = {"ms": round(kms, 5), "bytes": byts,
                           "gbs": round(byts / (kms / 1e3) / 1e9, 1)}
     dom = max(prof, key=prof.get)
-    dkey = "merge_multinomial" if dom == "merge" and "multinomial" in args.scheme else (
-        "merge_systematic" if dom == "merge" else dom)
     achieved = kernels[dom]["gbs"]
-    traffic = recorded_traffic(dkey, n)
+    traffic = recorded_traffic(dom, n)
     roofline = {"bound": "hbm", "kernel": dom, "achieved": achieved, "peak": hbm,
                 "peak_kind": hbm_kind, "unit": "GB/s", "frac": round(achieved / hbm, 4),
                 "traffic": traffic, "algorithmic_bytes": kernels[dom]["bytes"]}
@@ -439,7 +434,7 @@ def bench_ours(args):
     # instructions per particle from the committed ncu capture, against one
     # warp instruction per scheduler per cycle (4 per SM) at the maximum SM
     # clock seen during the timed region
-    inst = _recorded(dkey, "inst")
+    inst = _recorded(dom, "inst")
     if inst is not None and clocks.get("sm_max_mhz"):
         sms = torch.cuda.get_device_properties(local).multi_processor_count
         peak_i = sms * 4 * 32 * clocks["sm_max_mhz"] * 1e6 / 1e12
@@ -506,7 +501,7 @@ def bench_ours(args):
         f24.sync()
         ms24 = time_cycles(f24, y_dev, W24, K24, stream, None)
         prof24 = kernel_profile(f24, y, W24 + K24, 5, None)
-        b24 = {k: BYTES_PER_PARTICLE["merge_systematic" if k == "merge" else k] * n24 for k in prof24}
+        b24 = {k: BYTES_PER_PARTICLE[k] * n24 for k in prof24}
         b24 = {k: max(v, 1) for k, v in b24.items()}
         extra["n_2p24"] = {
             "value": n24 * K24 / (ms24 / 1e3), "unit": UNIT, "steps": K24,
@@ -517,16 +512,15 @@ def bench_ours(args):
             "kernels": {k: {"ms": round(v, 5), "gbs": round(b24[k] / (v / 1e3) / 1e9, 1)}
                         for k, v in prof24.items()}}
         f24.close()
-        # multinomial resampling at the same size (116 B/particle with the
-        # spacing prefix and its second CDF read), beside the systematic cycle
+        # multinomial resampling at the same size (100 B/particle with the
+        # CDF read again), beside the systematic cycle
         fm24 = pf.Filter(n24, seed=25, scheme="multinomial", precision="fp32", stream=stream)
         fm24.run(y_dev[:W24])
         fm24.sync()
         msm24 = time_cycles(fm24, y_dev, W24, K24, stream, None)
         profm24 = kernel_profile(fm24, y, W24 + K24, 3, None)
         fm24.close()
-        bm24 = sum(BYTES_PER_PARTICLE["merge_multinomial" if k == "merge" else k] * n24
-                   for k in profm24)
+        bm24 = sum(BYTES_PER_PARTICLE[k] * n24 for k in profm24)
         extra["n_2p24_multinomial"] = {
             "value": n24 * K24 / (msm24 / 1e3), "unit": UNIT, "steps": K24,
             "ms_per_step": msm24 / K24, "l2": "inputs larger than L2 (no flush)",
@@ -661,8 +655,8 @@ def bench_batched(pf, synth, stream, K=20, W=3, Kp=3, n_filters=4096, seed=4096)
         f.close()
     torch.cuda.empty_cache()
     hbm, _ = peaks()
-    byts = total * (BYTES_PER_PARTICLE["weights"] + BYTES_PER_PARTICLE["scan"] +
-                    BYTES_PER_PARTICLE["merge_systematic"] + BYTES_PER_PARTICLE["propagate"])
+    byts = total * sum(BYTES_PER_PARTICLE[k]
+                       for k in ("weights", "cdf_sums", "cdf_resample", "propagate"))
     return {
         "workload": "%d local-level filters, N log-uniform in [256, 65536] (sum %d), own series "
                     "from prior-drawn variances, FP32, systematic" % (n_filters, total),
@@ -675,7 +669,9 @@ def bench_batched(pf, synth, stream, K=20, W=3, Kp=3, n_filters=4096, seed=4096)
         "hbm_frac": round(byts / (ms_b / 1e3) / 1e9 / hbm, 4),
         "per_filter_launches": {"value": total / (ms_p / 1e3), "unit": UNIT, "steps": Kp,
                                 "ms_per_step": ms_p, "host_wall_ms_per_step": wall_p * 1e3,
-                                "gpu_launches_per_step": 5 * n_filters,
+                                # one cluster launch up to 8192 particles, else four kernels
+                                "gpu_launches_per_step": sum(1 if sp["n"] <= 8192 else 4
+                                                             for sp in specs),
                                 "note": "pf_step on each filter in turn, one stream"},
         "speedup_vs_per_filter": round(ms_p / ms_b, 2),
         "accuracy": "bit-identical per filter (tests/test_gpu_batch.py)",
@@ -899,7 +895,10 @@ def bench_served_per_stream(pf, synth, stream, n_streams=256, rounds=3, seed=100
     total = int(sum(int(ns[i]) for i in ids))
     return {"streams": n_streams, "sum_n": total, "rounds": rounds,
             "obs_per_s": obs / dt, "particle_steps_per_s": total * rounds / dt,
-            "gpu_launches_per_obs": 4,
+            # the cycle (one cluster launch up to 8192 particles, else four kernels) and
+            # the summary kernel
+            "gpu_launches_per_obs": round(sum(2 if int(ns[i]) <= 8192 else 5 for i in ids)
+                                          / n_streams, 2),
             "note": "pf_step on each stream (asynchronous), then pf_estimate on each (its result); "
                     "the first %d streams of the served workload" % n_streams}
 

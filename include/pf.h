@@ -312,7 +312,7 @@ pf_status pf_cutpoint_method(const uint64_t* Q_dev, uint64_t n, const uint32_t* 
  * a deployment variant.
  *
  * Scratch lives in one fixed-size device array inside libpf.so, present on
- * every device that loads the library until the process exits (about 20 MiB),
+ * every device that loads the library until the process exits (about 12 MiB),
  * and sized for n <= PF_NOALLOC_MAX_PARTICLES; larger n returns
  * PF_ERR_INVALID.  The first call on a device looks up the array's device
  * address (cudaGetSymbolAddress) with that device current.  The device used is

@@ -3,20 +3,23 @@
 // One cycle for observation y = y_{t+1} (paper Section 2, Algorithm
 // "Particle Learning"):
 //   k_weights       l_i = log p(y | x_i, sigma_i^2, tau_i^2) + log(2 pi)/2, max_i l_i
-//   k_scan          W_i = quantised exp(l_i - max), Q = inclusive scan of W
-//                   (eq. resample.cdf as exact 64-bit integers), single pass
-//                   with decoupled look-back
-//   k_spacing_scan  (multinomial) S = inclusive scan of exponential spacings
-//   k_merge         ancestors a_j = #{i : Q_i * A <= B_j} by a merge of the
-//                   sorted positions B with the CDF
+//   k_sums, k_slots W_i = quantised exp(l_i - max), Q = inclusive scan of W
+//                   (eq. resample.cdf as exact 64-bit integers), ancestors of
+//                   systematic and stratified resampling, the cut-point table
+//                   (slots.cuh; binary64: k_exp forms the exponentials first)
+//   k_spacing_sums, k_multi_split, k_multi   multinomial ancestors
+//                   a_j = #{i : Q_i * S_n <= S_j * T} (multi.cuh)
 //   k_cutpoint_*    the paper's Section 3.2 algorithms (same ancestors)
 //   k_propagate     gather ancestor, draw x, update b_sigma/b_tau, draw theta
+//                   (binary32: k_propagate2)
 //   k_estimate      posterior summaries on demand
+// k_scan is the CDF alone, for given weights (one pass, decoupled look-back).
+// A small filter's cycles are one cluster launch (small.cuh).
 //
 // Data layout in HBM (structure of arrays, one entry per particle):
 //   x, sigma2, tau2 : R (binary32 or binary64), two ping-pong copies
 //   b_sigma, b_tau  : uint64 2^-32 fixed point (FP32) / binary64 (FP64)
-//   l               : R,    Q : uint64,   S : uint64 (n+1),   anc : uint32
+//   l               : R,    Q : uint64,   anc : uint32
 #pragma once
 #include <cstddef>
 #include <cstdint>
