@@ -481,9 +481,11 @@ __global__ void __launch_bounds__(BLOCK) k_small(FilterArgs<R> a, SmallArgs sa) 
         if (i < cnt) a.lam[lo + i] = rs ? (R)0 : l[k] - mx;
       }
     }
+    // a failure goes to the error word before the last barrier, which orders it
+    // before rank 0 publishes that word with the summaries
+    if (step + 1 == sa.steps && __syncthreads_or(fail) && tid == 0) atomicOr(&c->err, ERR_NUMERIC);
     cluster_sync_all();  // 4: the new state, before the next cycle reads it
   }
-  if (__syncthreads_or(fail) && tid == 0) atomicOr(&c->err, ERR_NUMERIC);
   const uint32_t t1 = t0 + sa.steps;
   if (rank == 0 && tid == 0) {
     c->t = t1;
