@@ -1887,6 +1887,7 @@ __global__ void __launch_bounds__(BLOCK) k_estimate_w(FilterArgs<R> a) {
     for (int w = 0; w < WARPS; ++w) v += s_sum[threadIdx.x][w];
     a.part_est[(uint64_t)blockIdx.x * 7 + threadIdx.x] = v;
   }
+  __syncthreads();  // all seven sums, before the count that announces them
   if (threadIdx.x == 0) {
     __threadfence();
     s_last = atomicAdd(&a.ctl->done_est, 1u) == gridDim.x - 1;
