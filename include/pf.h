@@ -94,7 +94,9 @@ typedef enum {
 typedef enum { PF_FP32 = 0, PF_FP64 = 1 } pf_precision;
 
 /* Optional device allocator (e.g. a caching allocator).  alloc returns NULL on
- * failure.  stream is the handle's cudaStream_t. */
+ * failure, else an address that is a multiple of 16; where it is not one of 32
+ * the library frees the block and asks once more, for a larger one.  stream is
+ * the handle's cudaStream_t. */
 typedef void* (*pf_alloc_fn)(size_t bytes, void* stream, void* ctx);
 typedef void (*pf_free_fn)(void* ptr, void* stream, void* ctx);
 

@@ -1,9 +1,9 @@
 /*
- * pf_diag.h -- diagnostic entry points of libpf.so for failure-detection
- * tests.  They are not part of the particle-learning method: the paper has
- * no counterpart.  They exercise the library's failure handling without
- * faulting or hanging a GPU, by making one of its bounded device waits run
- * out on purpose.
+ * pf_diag.h -- diagnostic entry points of libpf.so for tests of what a
+ * filter's results do not show.  They are not part of the particle-learning
+ * method: the paper has no counterpart.  The failure handling is exercised
+ * without faulting or hanging a GPU, by making one of the library's bounded
+ * device waits run out on purpose.
  */
 #ifndef PF_DIAG_H
 #define PF_DIAG_H
@@ -31,6 +31,12 @@ extern "C" {
  * n in [1, 2^26], spin_limit >= 1); synchronises `stream`. */
 pf_status pf_diag_cdf_wait(const float* w_dev, uint64_t n, uint32_t withhold_tile,
                            uint32_t spin_limit, uint64_t* Q_dev, void* stream);
+
+/* How a handle takes one block of device memory from its allocator callbacks,
+ * on the host alone (the addresses are not used): *raw is what free must get
+ * back, *start the block's first byte, at a multiple of 32. */
+pf_status pf_diag_block(pf_alloc_fn alloc, pf_free_fn free, void* ctx, size_t bytes, void** raw,
+                        void** start);
 
 #ifdef __cplusplus
 }

@@ -145,24 +145,46 @@ struct pf_filter {
 
 namespace {
 
-pf_status dev_alloc(pf_filter* f, size_t bytes, void** out) {
+// Device memory of a handle, from its allocator callbacks or cudaMallocAsync.
+// The kernels load and store up to 32 bytes at a time, and a callback's block
+// may start at any multiple of 16: one that does not start at a multiple of 32
+// goes back, and a larger block is used from its first such address.  *raw is
+// the pointer to free.
+constexpr size_t DEV_ALIGN = 32, DEV_ALIGN_MIN = 16;
+pf_status device_block(pf_alloc_fn alloc, pf_free_fn free, void* ctx, cudaStream_t stream, size_t bytes,
+                       void** raw, void** out) {
   bytes = (bytes + 255) & ~size_t(255);
   void* p = nullptr;
-  if (f->cfg.alloc) {
-    p = f->cfg.alloc(bytes, f->stream, f->cfg.alloc_ctx);
+  if (alloc) {
+    p = alloc(bytes, stream, ctx);
+    if (p && ((uintptr_t)p & (DEV_ALIGN - 1)) == DEV_ALIGN_MIN) {
+      free(p, stream, ctx);
+      bytes += 256;
+      p = alloc(bytes, stream, ctx);
+    }
     if (!p) return set_err(PF_ERR_OOM, "allocator callback returned NULL for %zu bytes", bytes);
+    if (((uintptr_t)p & (DEV_ALIGN_MIN - 1)) != 0) {
+      free(p, stream, ctx);
+      return set_err(PF_ERR_INVALID, "allocator returned a pointer not 16-byte aligned");
+    }
   } else {
-    cudaError_t e = cudaMallocAsync(&p, bytes, f->stream);
+    cudaError_t e = cudaMallocAsync(&p, bytes, stream);
     if (e != cudaSuccess) {
       cudaGetLastError();
       return set_err(e == cudaErrorMemoryAllocation ? PF_ERR_OOM : PF_ERR_CUDA,
                      "cudaMallocAsync(%zu): %s", bytes, cudaGetErrorString(e));
     }
   }
-  if (((uintptr_t)p & 15) != 0) return set_err(PF_ERR_INVALID, "allocator returned a pointer not 16-byte aligned");
-  f->allocs.push_back(p);
-  *out = p;
+  *raw = p;
+  *out = (void*)(((uintptr_t)p + DEV_ALIGN - 1) & ~(uintptr_t)(DEV_ALIGN - 1));
   return PF_OK;
+}
+
+pf_status dev_alloc(pf_filter* f, size_t bytes, void** out) {
+  void* raw = nullptr;
+  pf_status st = device_block(f->cfg.alloc, f->cfg.free, f->cfg.alloc_ctx, f->stream, bytes, &raw, out);
+  if (st == PF_OK) f->allocs.push_back(raw);
+  return st;
 }
 
 void free_all(pf_filter* f) {
@@ -1563,6 +1585,12 @@ pf_status pf_diag_cdf_wait(const float* w_dev, uint64_t n, uint32_t withhold_til
   dg.spin_limit = spin_limit;
   dg.withhold = withhold_tile;
   return resample_common(w_dev, n, 0, 0, 0, PF_SYSTEMATIC, nullptr, Q_dev, stream, dg);
+}
+
+pf_status pf_diag_block(pf_alloc_fn alloc, pf_free_fn free, void* ctx, size_t bytes, void** raw,
+                        void** start) {
+  if (!alloc || !free || !raw || !start) return set_err(PF_ERR_INVALID, "NULL pointer");
+  return device_block(alloc, free, ctx, nullptr, bytes, raw, start);
 }
 
 pf_status pf_cutpoint_search(const uint64_t* Q_dev, uint64_t n, uint32_t* I_dev, void* stream) {

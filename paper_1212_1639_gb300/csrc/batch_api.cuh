@@ -84,23 +84,10 @@ constexpr uint64_t kPoolAlign = 32;  // particles: 128-byte aligned filter range
 size_t list_bytes(uint32_t max_filters) { return 16 + (size_t)max_filters * sizeof(BatchItem); }
 
 pf_status batch_alloc(pf_batch* b, size_t bytes, void** out) {
-  bytes = (bytes + 255) & ~size_t(255);
-  void* p = nullptr;
-  if (b->alloc) {
-    p = b->alloc(bytes, b->stream, b->alloc_ctx);
-    if (!p) return set_err(PF_ERR_OOM, "allocator callback returned NULL for %zu bytes", bytes);
-  } else {
-    cudaError_t e = cudaMallocAsync(&p, bytes, b->stream);
-    if (e != cudaSuccess) {
-      cudaGetLastError();
-      return set_err(e == cudaErrorMemoryAllocation ? PF_ERR_OOM : PF_ERR_CUDA,
-                     "cudaMallocAsync(%zu): %s", bytes, cudaGetErrorString(e));
-    }
-  }
-  if (((uintptr_t)p & 15) != 0) return set_err(PF_ERR_INVALID, "allocator returned a pointer not 16-byte aligned");
-  b->allocs.push_back(p);
-  *out = p;
-  return PF_OK;
+  void* raw = nullptr;
+  pf_status st = device_block(b->alloc, b->free, b->alloc_ctx, b->stream, bytes, &raw, out);
+  if (st == PF_OK) b->allocs.push_back(raw);
+  return st;
 }
 
 uint64_t batch_bytes_per_particle(bool fp64, bool multi, bool adaptive) {

@@ -137,6 +137,7 @@ _SIGS = {
     "pf_resample_noalloc": [_V, C.c_uint64, C.c_uint64, C.c_uint32, C.c_uint32, C.c_int32, _V,
                             _V],
     "pf_cdf": [_V, C.c_uint64, _V, _V],
+    "pf_diag_block": [ALLOC_FN, FREE_FN, _V, C.c_size_t, C.POINTER(_V), C.POINTER(_V)],
     "pf_diag_cdf_wait": [_V, C.c_uint64, C.c_uint32, C.c_uint32, _V, _V],
     "pf_cutpoint_search": [_V, C.c_uint64, _V, _V],
     "pf_cutpoint_method": [_V, C.c_uint64, _V, _V, C.c_uint64, _V, _V],
