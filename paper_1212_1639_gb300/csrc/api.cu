@@ -338,9 +338,10 @@ void launch_cdf(pf_filter* f, cudaStream_t s, KTimer* tm) {
   a.src_vec = a.anc_vec = 1;
   const unsigned sg = sums_grid(f->n);
   const int pos = slot_pos(f->scheme);
-  if (pos != SLOTS_NONE && !f->fp64) a.heavy = (char*)f->pre + pre_bytes(f->n);
+  if (pos != SLOTS_NONE) a.heavy = (char*)f->pre + pre_bytes(f->n);
   if constexpr (sizeof(R) == 8) {
     a.src = f->Q;
+    a.l = (const double*)f->ell;
     a.part_blk = f->part;
     if (f->ess) k_sums<SRC_E64, true><<<sg, BLOCK, 0, s>>>(a);
     else k_sums<SRC_E64, false><<<sg, BLOCK, 0, s>>>(a);

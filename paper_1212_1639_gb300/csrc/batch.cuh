@@ -256,6 +256,77 @@ static __device__ __noinline__ uint32_t sys_first_exact(uint64_t q, uint64_t n, 
   return (uint32_t)sys_first_slot(q, n, r, make_sysdiv(T));
 }
 
+// Clipped marking out of line (few warps need it): 4096 filters per cycle 1184 ->
+// 1167 us with the registers that this leaves the tiles' loop.
+template <uint32_t WIN>
+static __device__ __noinline__ void mark_out(uint16_t* win, uint32_t (*runs)[3], uint32_t* nruns, uint32_t wb, uint32_t j,
+                                             uint32_t mk0, uint32_t r0, uint32_t r1, uint32_t r2, uint32_t r3,
+                                             uint32_t r4, uint32_t r5, uint32_t r6, uint32_t r7) {
+  const uint32_t Rs[SLOT_PER] = {r0, r1, r2, r3, r4, r5, r6, r7};
+  win_mark_clipped<WIN>(win, runs, nruns, wb, j, Rs, mk0);
+}
+
+// The slots from wb on of a tile with more than its first window holds (S0: its
+// first slot), window after window, from the CDF values that its CTA has stored;
+// the slots of a particle that owns many of them go out straight.  Out of line:
+// few tiles come here, and its registers are not the others'.  Cycle of one
+// filter of 131,072 particles on a cluster of eight, all its mass on one
+// particle: 147 us with every window of 4096 slots built and read, 119 so (one
+// thread's walk over the CDF, before: 129).
+template <class R, int NT>
+static __device__ __noinline__ void batch_windows(BatchSmem<R, NT>& sm, const uint64_t* Q, uint32_t* anc, uint64_t tb,
+                                                  uint64_t n, uint32_t S0, uint64_t r, uint64_t T, uint32_t wb) {
+  constexpr uint32_t WIN = 2 * NT * SLOT_PER;
+  const uint64_t base = tb + (uint64_t)threadIdx.x * SLOT_PER;
+  const uint32_t S1 = sm.wend, mk0 = threadIdx.x * SLOT_PER + 1u;
+  const int z = sm.z;
+  SlotMap map;
+  map.rho = sm.rho;
+  map.r32 = sm.r32;
+  auto below = [&](uint64_t q) -> uint32_t {
+    uint32_t close = ~0u;
+    const uint32_t v = slot_below<SLOTS_SYS>(q << z, map, &close);
+    return close < 8u ? sys_first_exact(q, n, r, T) : v;
+  };
+  uint32_t Rs[SLOT_PER];
+  const uint32_t j = threadIdx.x == 0 ? S0 : below(base <= n ? Q[base - 1] : T);
+#pragma unroll
+  for (int e = 0; e < SLOT_PER; ++e) Rs[e] = base + e < n ? below(Q[base + e]) : S1;
+  while (true) {
+    if (threadIdx.x == 0) sm.nruns = 0;
+#pragma unroll
+    for (uint32_t i = 0; i < WIN; i += 8 * NT)
+      *reinterpret_cast<uint4*>(sm.win + i + 8 * threadIdx.x) = make_uint4(0u, 0u, 0u, 0u);
+    if (j <= wb && wb < Rs[SLOT_PER - 1]) {  // one thread: the particle that owns slot wb
+      uint32_t own = (uint32_t)base, end = Rs[0];
+#pragma unroll
+      for (int e = 1; e < SLOT_PER; ++e)
+        if (Rs[e - 1] <= wb) {
+          own = (uint32_t)base + e;
+          end = Rs[e];
+        }
+      sm.roff = (uint64_t)end << 32 | own;
+    }
+    __syncthreads();
+    const uint32_t o = (uint32_t)sm.roff, end = (uint32_t)(sm.roff >> 32), full = end & ~3u;
+    if (end - wb > WIN / 4) {
+      for (uint32_t x = wb + 4u * threadIdx.x; x < full; x += 4u * NT)
+        *reinterpret_cast<uint4*>(anc + x) = make_uint4(o, o, o, o);
+      if (threadIdx.x < end - full) anc[full + threadIdx.x] = o;
+      if (end == S1) break;
+      wb = full;  // (slots [full, end) are stored again, alike)
+    }
+    win_mark_clipped<WIN>(sm.win, sm.run, &sm.nruns, wb, j, Rs, mk0);
+    __syncthreads();
+    win_runs<NT>(sm.win, sm.run, &sm.nruns);
+    win_store<NT>(sm.win, anc, wb, wb, min(S1, wb + WIN), (uint32_t)tb, true);
+    wb += WIN;
+    if (S1 <= wb) break;
+    __syncthreads();  // the window has been read
+  }
+  __syncthreads();
+}
+
 // One cycle of one filter by a group of G CTAs (G = 1: one CTA; G > 1: the
 // CTAs of a cluster, this one being `rank`).  The particles are cut into
 // passes of NT / 256 scan tiles; round j gives pass j G + rank to this CTA.
@@ -622,7 +693,10 @@ __device__ __forceinline__ void batch_filter(const BatchArgs<R>& a, const BatchI
         sm.z = z - zs;
         sm.rho = div_2by1(n << (32 + zs), 0, T << z);
       }
-      if (threadIdx.x == 32) sm.r32 = div_2by1((r << z) >> 32, (r << z) << 32, T << z);
+      if (threadIdx.x == 32) {
+        if constexpr (G > 1) sm.rsum = r;
+        sm.r32 = div_2by1((r << z) >> 32, (r << z) << 32, T << z);
+      }
     }
     __syncthreads();
     SlotMap map;
@@ -630,6 +704,11 @@ __device__ __forceinline__ void batch_filter(const BatchArgs<R>& a, const BatchI
     map.r32 = sm.r32;
     const int z = sm.z;
     const bool go = resamp && T > 0;
+    // (the offset is read back with clusters: two registers fewer there)
+    auto offset = [&]() -> uint64_t {
+      if constexpr (G > 1) return sm.rsum;
+      else return r;
+    };
     auto clear = [&]() {
       if (threadIdx.x == 0) sm.nruns = 0;
 #pragma unroll
@@ -660,7 +739,8 @@ __device__ __forceinline__ void batch_filter(const BatchArgs<R>& a, const BatchI
         woff += __shfl_xor_sync(0xffffffffu, woff, o);
         tot += __shfl_xor_sync(0xffffffffu, tot, o);
       }
-      uint64_t q0 = carry + woff + incl - acc;
+      uint64_t p0 = carry, q0 = carry + woff + incl - acc;
+      carry += tot;
       if (base + SLOT_PER <= n) {
         st4(a.Q + off + base, q0 + run[0], q0 + run[1], q0 + run[2], q0 + run[3]);
         st4(a.Q + off + base + 4, q0 + run[4], q0 + run[5], q0 + run[6], q0 + run[7]);
@@ -670,7 +750,6 @@ __device__ __forceinline__ void batch_filter(const BatchArgs<R>& a, const BatchI
           if (base + e < n) a.Q[off + base + e] = q0 + run[e];
       }
       if (go) {
-        uint64_t p0 = carry;
         if (z) {  // (rare, and the same in every thread)
           p0 <<= z;
           q0 <<= z;
@@ -679,85 +758,34 @@ __device__ __forceinline__ void batch_filter(const BatchArgs<R>& a, const BatchI
         }
         uint32_t close = ~0u, close0 = ~0u;
         uint32_t S0 = slot_below<SLOTS_SYS>(p0, map, &close0);
-        if (close0 < 8u) S0 = sys_first_exact(carry, n, r, T);
+        if (close0 < 8u) S0 = sys_first_exact(p0 >> z, n, offset(), T);
         uint32_t Rs[SLOT_PER];
         uint32_t j = slot_below<SLOTS_SYS>(q0, map, &close);
 #pragma unroll
         for (int e = 0; e < SLOT_PER; ++e) Rs[e] = slot_below<SLOTS_SYS>(q0 + run[e], map, &close);
         if (close < 8u) {
-          j = sys_first_exact(q0 >> z, n, r, T);
-          for (int e = 0; e < SLOT_PER; ++e) Rs[e] = sys_first_exact((q0 + run[e]) >> z, n, r, T);
+          j = sys_first_exact(q0 >> z, n, offset(), T);
+          for (int e = 0; e < SLOT_PER; ++e) Rs[e] = sys_first_exact((q0 + run[e]) >> z, n, offset(), T);
         }
         if (threadIdx.x == NT - 1) sm.wend = Rs[SLOT_PER - 1];
         const uint32_t mk0 = threadIdx.x * SLOT_PER + 1u;
         uint32_t most = Rs[0] - j;
 #pragma unroll
         for (int e = 1; e < SLOT_PER; ++e) most = max(most, Rs[e] - Rs[e - 1]);
-        for (uint32_t wb = S0 & ~3u;;) {  // the tile's windows (one, but for heavy particles)
-          if (!__any_sync(0xffffffffu, most > 5u || j < wb || Rs[SLOT_PER - 1] - wb > WIN)) {
-            uint32_t x = j - wb;
-#pragma unroll
-            for (int e = 0; e < SLOT_PER; ++e) {
-              const uint32_t xe = Rs[e] - wb, g = (x + 4u) & ~3u;
-              if (xe > x) sm.win[win_entry(x)] = (uint16_t)(mk0 + e);
-              if (xe > g) sm.win[win_entry(g)] = (uint16_t)(mk0 + e);
-              x = xe;
-            }
-          } else {
-            uint32_t x = j < wb ? 0u : min(j - wb, WIN);
-#pragma unroll
-            for (int e = 0; e < SLOT_PER; ++e) {
-              const uint32_t xe = Rs[e] < wb ? 0u : min(Rs[e] - wb, WIN), g = (x + 4u) & ~3u;
-              const uint16_t mk = (uint16_t)(mk0 + e);
-              if (xe > x) sm.win[win_entry(x)] = mk;
-              if (xe > g) sm.win[win_entry(g)] = mk;
-              if (xe > g + 4u) mark_rest(g + 4u, xe, mk, sm.win, sm.run, &sm.nruns);
-              x = xe;
-            }
-          }
-          __syncthreads();
-          const uint32_t nr = sm.nruns < BB_MAX_RUNS ? sm.nruns : BB_MAX_RUNS;
-          if (nr) {
-            for (uint32_t q = 0; q < nr; ++q) {
-              const uint32_t en = sm.run[q][1];
-              for (uint32_t x = sm.run[q][0] + 4u * threadIdx.x; x < en; x += 4u * NT)
-                sm.win[win_entry(x)] = (uint16_t)sm.run[q][2];
-            }
-            __syncthreads();
-          }
-          const uint32_t S1 = sm.wend;
-          const uint32_t ws = max(S0, wb), we = min(S1, wb + WIN);
-          const uint32_t tb32 = (uint32_t)tb - 1u;
-          const uint32_t ng = we > ws ? (we - wb + 3u) >> 2 : 0u;
-          uint32_t* const anc = a.anc + off;  // (off is a multiple of 32)
-          for (uint32_t g = threadIdx.x; g < ng; g += NT) {
-            const uint32_t x0 = g << 2;
-            const uint32_t sw = ((x0 >> 6) & 7u) << 1;
-            const uint2 w = *reinterpret_cast<const uint2*>(sm.win + (x0 ^ (sw & 12u)));
-            const uint32_t lo = (sw & 2u) ? w.y : w.x, hi = (sw & 2u) ? w.x : w.y;
-            const uint32_t slot = wb + x0;
-            const uint32_t e0 = lo & 0xffffu, e1 = max(e0, lo >> 16);
-            const uint32_t e2 = max(e1, hi & 0xffffu), e3 = max(e2, hi >> 16);
-            const uint4 o4 = make_uint4(tb32 + e0, tb32 + e1, tb32 + e2, tb32 + e3);
-            if (slot >= ws && slot + 4u <= we) {
-              *reinterpret_cast<uint4*>(anc + slot) = o4;
-            } else {
-              if (slot >= ws && slot < we) anc[slot] = o4.x;
-              if (slot + 1u >= ws && slot + 1u < we) anc[slot + 1u] = o4.y;
-              if (slot + 2u >= ws && slot + 2u < we) anc[slot + 2u] = o4.z;
-              if (slot + 3u >= ws && slot + 3u < we) anc[slot + 3u] = o4.w;
-            }
-          }
-          __syncthreads();  // the window has been read
-          wb += WIN;
-          if (S1 <= wb) break;
-          clear();
-          __syncthreads();
-        }
+        const uint32_t wb = S0 & ~3u;
+        if (!__any_sync(0xffffffffu, most > 5u || Rs[SLOT_PER - 1] - wb > WIN))
+          win_mark(sm.win, wb, j, Rs, mk0);
+        else
+          mark_out<WIN>(sm.win, sm.run, &sm.nruns, wb, j, mk0, Rs[0], Rs[1], Rs[2], Rs[3], Rs[4], Rs[5], Rs[6], Rs[7]);
+        __syncthreads();
+        win_runs<NT>(sm.win, sm.run, &sm.nruns);
+        uint32_t* const anc = a.anc + off;  // (off is a multiple of 32)
+        win_store<NT>(sm.win, anc, wb, S0, min(sm.wend, wb + WIN), (uint32_t)tb, true);
+        __syncthreads();  // the window has been read
+        if (sm.wend > wb + WIN) batch_windows<R, NT>(sm, a.Q + off, anc, tb, n, S0, offset(), T, wb + WIN);
       } else {
         __syncthreads();  // sm.warp has been read
       }
-      carry += tot;
     }
   } else {
   // 3. resampling: slot keys B_j against the CDF keys Q_i A (ties go to the

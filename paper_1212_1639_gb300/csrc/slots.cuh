@@ -64,7 +64,8 @@ struct SlotArgs {
   uint64_t seed;
   uint32_t filter;
   double ess_frac;
-  void* heavy;            // heavy list, or NULL (no further windows: NONE and binary64)
+  void* heavy;            // heavy list, or NULL (NONE: no windows)
+  const double* l;        // binary64: the l_i, for the tiles of the heavy list
   uint32_t* host_err;     // mapped host word for pf_resample's errors, or NULL
   int multi;              // multinomial: S_n is known (k_spacing_sums ran before)
   int cut;                // k_slots builds the cut-point table in anc: the slot map with r = 0
@@ -392,16 +393,21 @@ static __device__ __noinline__ void sums_last(const SlotArgs& a, uint64_t* s_tot
   // estimate of a tile's slots is within 32 of them, so a last window may turn
   // out empty.
   const float per_slot = nf / Tf;
-  auto chunks = [&](uint32_t i) -> uint32_t {
-    const uint64_t q0 = a.pre[i], q1 = i + 1 < a.ntiles ? a.pre[i + 1] : T;
-    if (!(q1 - q0 > most)) return 0;
-    return (uint32_t)((__ull2float_rn(q1 - q0) * per_slot + 40.0f) * (1.0f / SLOT_WIN));
+  auto chunks = [&](uint64_t sum) -> uint32_t {
+    return sum > most ? (uint32_t)((__ull2float_rn(sum) * per_slot + 40.0f) * (1.0f / SLOT_WIN)) : 0u;
+  };
+  // each of this thread's heavy tiles, in order (the first sums from registers:
+  // a trip to L2 per tile took 3 us here)
+  auto each = [&](auto f) {
+    if (!heavy) return;
+#pragma unroll
+    for (uint32_t i = 0; i < KEEP; ++i)
+      if (const uint32_t k = chunks(kept[i])) f(t0 + i, k);
+    for (uint32_t i = t0 + KEEP; i < t1; ++i)
+      if (const uint32_t k = chunks((i + 1 < a.ntiles ? a.pre[i + 1] : T) - a.pre[i])) f(i, k);
   };
   uint64_t cnt = 0;  // entries, then chunks
-  for (uint32_t i = t0; i < t1; ++i) {
-    const uint32_t k = chunks(i);
-    cnt += k ? (1ull << 32) + k : 0ull;
-  }
+  each([&](uint32_t, uint32_t k) { cnt += (1ull << 32) + k; });
   const uint64_t ci = warp_incl_scan(cnt, lane);
   if (lane == 31) s_tot[warp] = ci;
   __syncthreads();
@@ -410,12 +416,10 @@ static __device__ __noinline__ void sums_last(const SlotArgs& a, uint64_t* s_tot
     if (w < warp) at += s_tot[w];
     all += s_tot[w];
   }
-  for (uint32_t i = t0; i < t1; ++i) {
-    const uint32_t k = chunks(i);
-    if (!k) continue;
+  each([&](uint32_t i, uint32_t k) {
     reinterpret_cast<uint2*>(a.heavy)[at >> 32] = make_uint2(i, (uint32_t)at);
     at += (1ull << 32) + k;
-  }
+  });
   if (threadIdx.x == 0) {
     c->heavy_count = (uint32_t)(all >> 32);
     c->heavy_chunks = (uint32_t)all;
@@ -530,6 +534,78 @@ static __device__ __noinline__ void mark_rest(uint32_t from, uint32_t to, uint16
   for (uint32_t q = from; q < to; q += 4u) win[win_entry(q)] = mk;
 }
 
+// The slots [j, Rs[0]), [Rs[0], Rs[1]), ... of a thread's particles marked in the
+// window of WIN slots from wb; mk0: the first particle's mark.  When the window
+// holds them all and none has more than five (for a whole warp):
+__device__ __forceinline__ void win_mark(uint16_t* win, uint32_t wb, uint32_t j, const uint32_t* Rs, uint32_t mk0) {
+  uint32_t x = j - wb;
+#pragma unroll
+  for (int e = 0; e < SLOT_PER; ++e) {
+    const uint32_t xe = Rs[e] - wb, g = (x + 4u) & ~3u;
+    if (xe > x) win[win_entry(x)] = (uint16_t)(mk0 + e);
+    if (xe > g) win[win_entry(g)] = (uint16_t)(mk0 + e);
+    x = xe;
+  }
+}
+// else each particle's slots clipped to the window
+template <uint32_t WIN>
+__device__ __forceinline__ void win_mark_clipped(uint16_t* win, uint32_t (*runs)[3], uint32_t* nruns, uint32_t wb,
+                                                 uint32_t j, const uint32_t* Rs, uint32_t mk0) {
+  uint32_t x = j < wb ? 0u : min(j - wb, WIN);
+#pragma unroll
+  for (int e = 0; e < SLOT_PER; ++e) {
+    const uint32_t xe = Rs[e] < wb ? 0u : min(Rs[e] - wb, WIN), g = (x + 4u) & ~3u;
+    const uint16_t mk = (uint16_t)(mk0 + e);
+    if (xe > x) win[win_entry(x)] = mk;
+    if (xe > g) win[win_entry(g)] = mk;
+    if (xe > g + 4u) mark_rest(g + 4u, xe, mk, win, runs, nruns);
+    x = xe;
+  }
+}
+// the runs that marking left, by the whole CTA of NT threads (after a barrier)
+template <int NT>
+__device__ __forceinline__ void win_runs(uint16_t* win, const uint32_t (*runs)[3], const uint32_t* nruns) {
+  const uint32_t nr = *nruns < SLOT_RUNS ? *nruns : SLOT_RUNS;
+  if (!nr) return;
+  for (uint32_t q = 0; q < nr; ++q) {
+    const uint32_t en = runs[q][1];
+    for (uint32_t y = runs[q][0] + 4u * threadIdx.x; y < en; y += 4u * NT) win[win_entry(y)] = (uint16_t)runs[q][2];
+  }
+  __syncthreads();
+}
+// the window's slots [ws, wend), four per 16-byte store where vec (the partial
+// groups at either end slot by slot); tb: the tile's first particle
+template <int NT>
+__device__ __forceinline__ void win_store(const uint16_t* win, uint32_t* anc, uint32_t wb, uint32_t ws, uint32_t wend,
+                                          uint32_t tb, bool vec) {
+  const uint32_t tb32 = tb - 1u;
+  const uint32_t ng = wend > ws ? (wend - wb + 3u) >> 2 : 0u;
+  for (uint32_t g = threadIdx.x; g < ng; g += NT) {
+    const uint32_t x0 = g << 2;
+    const uint32_t sw = ((x0 >> 6) & 7u) << 1;
+    const uint2 w = *reinterpret_cast<const uint2*>(win + (x0 ^ (sw & 12u)));
+    const uint32_t lo = (sw & 2u) ? w.y : w.x, hi = (sw & 2u) ? w.x : w.y;
+    const uint32_t slot = wb + x0;
+    const uint32_t e0 = lo & 0xffffu, e1 = max(e0, lo >> 16);
+    const uint32_t e2 = max(e1, hi & 0xffffu), e3 = max(e2, hi >> 16);
+    const uint4 o4 = make_uint4(tb32 + e0, tb32 + e1, tb32 + e2, tb32 + e3);
+    if (slot >= ws && slot + 4u <= wend && vec) {
+      *reinterpret_cast<uint4*>(anc + slot) = o4;
+    } else {
+      if (slot >= ws && slot < wend) anc[slot] = o4.x;
+      if (slot + 1u >= ws && slot + 1u < wend) anc[slot + 1u] = o4.y;
+      if (slot + 2u >= ws && slot + 2u < wend) anc[slot + 2u] = o4.z;
+      if (slot + 3u >= ws && slot + 3u < wend) anc[slot + 3u] = o4.w;
+    }
+  }
+}
+
+// Binary64: an exponential of a heavy tile, taken again from l by another CTA than
+// the tile's, which may have written Q over k_exp's values already.
+static __device__ __noinline__ double heavy_exp64(const SlotArgs& a, uint64_t i) {
+  return i < a.n ? exp_weight(a.l[i] - dec_d(a.ctl->maxenc)) : 0.0;
+}
+
 // One CTA per tile.  Thread t takes particles [8 t, 8 t + 8) of the tile.  The
 // ancestors of the tile's slots are built in a shared-memory window of one
 // 16-bit entry per slot (at least two slots per particle of the tile), cleared
@@ -543,9 +619,10 @@ static __device__ __noinline__ void mark_rest(uint32_t from, uint32_t to, uint16
 //
 // A tile of more slots than its window leaves the others to the CTAs of the
 // heavy list (k_sums): CTA b < heavy_chunks, after its own tile, rebuilds the
-// heavy tile of chunk b and stores that window (all the mass on one particle of
-// 2^24: 1.1 ms by one CTA).  Binary64 overwrites its source with Q, so there
-// each CTA stores all windows of its own tile.
+// heavy tile of chunk b and stores that window.  With all the mass on one particle
+// of 2^23 the kernel takes 43 us (binary64 55), by one CTA window after window
+// 2.5 ms.  Binary64 overwrites its source with Q, so there the heavy tile is
+// rebuilt from l.
 template <int SRC, int POS>
 __global__ void __launch_bounds__(BLOCK, 4) k_slots(SlotArgs a) {
   typedef typename SrcT<SRC>::R R;
@@ -564,7 +641,16 @@ __global__ void __launch_bounds__(BLOCK, 4) k_slots(SlotArgs a) {
     const uint64_t tbase = (uint64_t)tile * SLOT_TILE;
     const uint64_t base = tbase + (uint64_t)threadIdx.x * SLOT_PER;
     R v[SLOT_PER];
-    load8<SRC>(a, base, v);
+    if constexpr (SRC == SRC_E64) {
+      if (pass == 0) {
+        load8<SRC>(a, base, v);
+      } else {
+#pragma unroll
+        for (int e = 0; e < SLOT_PER; ++e) v[e] = heavy_exp64(a, base + e);
+      }
+    } else {
+      load8<SRC>(a, base, v);
+    }
     uint64_t run[SLOT_PER];
     uint64_t acc = 0;
     quant.exps(v);
@@ -652,73 +738,15 @@ __global__ void __launch_bounds__(BLOCK, 4) k_slots(SlotArgs a) {
 #pragma unroll
     for (int e = 1; e < SLOT_PER; ++e) most = max(most, Rs[e] - Rs[e - 1]);
     // the window's base: slots in aligned groups of four
-    uint32_t wb = (S0 & ~3u) + wsel * SLOT_WIN;
-    while (true) {
-      if (!__any_sync(0xffffffffu, most > 5u || j < wb || Rs[SLOT_PER - 1] - wb > SLOT_WIN)) {
-        uint32_t x = j - wb;
-#pragma unroll
-        for (int e = 0; e < SLOT_PER; ++e) {
-          const uint32_t xe = Rs[e] - wb, g = (x + 4u) & ~3u;
-          if (xe > x) s_win[win_entry(x)] = (uint16_t)(mk0 + e);
-          if (xe > g) s_win[win_entry(g)] = (uint16_t)(mk0 + e);
-          x = xe;
-        }
-      } else {
-        // each particle's slots clipped to the window
-        uint32_t x = j < wb ? 0u : min(j - wb, SLOT_WIN);
-#pragma unroll
-        for (int e = 0; e < SLOT_PER; ++e) {
-          const uint32_t xe = Rs[e] < wb ? 0u : min(Rs[e] - wb, SLOT_WIN), g = (x + 4u) & ~3u;
-          const uint16_t mk = (uint16_t)(mk0 + e);
-          if (xe > x) s_win[win_entry(x)] = mk;
-          if (xe > g) s_win[win_entry(g)] = mk;
-          if (xe > g + 4u) mark_rest(g + 4u, xe, mk, s_win, s_run, &s_nruns);
-          x = xe;
-        }
-      }
-      __syncthreads();
-      // runs, by the whole CTA
-      const uint32_t nr = s_nruns < SLOT_RUNS ? s_nruns : SLOT_RUNS;
-      if (nr) {
-        for (uint32_t q = 0; q < nr; ++q) {
-          const uint32_t en = s_run[q][1];
-          for (uint32_t y = s_run[q][0] + 4u * threadIdx.x; y < en; y += 4u * BLOCK)
-            s_win[win_entry(y)] = (uint16_t)s_run[q][2];
-        }
-        __syncthreads();
-      }
-      // the window's slots [ws, wend), four per 16-byte store (the partial
-      // groups at either end slot by slot)
-      const uint32_t S1 = s_end;
-      const uint32_t ws = max(S0, wb);
-      const uint32_t wend = min(S1, wb + SLOT_WIN);
-      const uint32_t tb32 = (uint32_t)tbase - 1u;
-      const uint32_t ng = wend > ws ? (wend - wb + 3u) >> 2 : 0u;
-      for (uint32_t g = threadIdx.x; g < ng; g += BLOCK) {
-        const uint32_t x0 = g << 2;
-        const uint32_t sw = ((x0 >> 6) & 7u) << 1;
-        const uint2 w = *reinterpret_cast<const uint2*>(s_win + (x0 ^ (sw & 12u)));
-        const uint32_t lo = (sw & 2u) ? w.y : w.x, hi = (sw & 2u) ? w.x : w.y;
-        const uint32_t slot = wb + x0;
-        const uint32_t e0 = lo & 0xffffu, e1 = max(e0, lo >> 16);
-        const uint32_t e2 = max(e1, hi & 0xffffu), e3 = max(e2, hi >> 16);
-        const uint4 o4 = make_uint4(tb32 + e0, tb32 + e1, tb32 + e2, tb32 + e3);
-        if (slot >= ws && slot + 4u <= wend && a.anc_vec) {
-          *reinterpret_cast<uint4*>(a.anc + slot) = o4;
-        } else {
-          if (slot >= ws && slot < wend) a.anc[slot] = o4.x;
-          if (slot + 1u >= ws && slot + 1u < wend) a.anc[slot + 1u] = o4.y;
-          if (slot + 2u >= ws && slot + 2u < wend) a.anc[slot + 2u] = o4.z;
-          if (slot + 3u >= ws && slot + 3u < wend) a.anc[slot + 3u] = o4.w;
-        }
-      }
-      if (SRC != SRC_E64 || S1 <= wb + SLOT_WIN) break;
-      wb += SLOT_WIN;
-      __syncthreads();  // the window has been read
-      clear();
-      __syncthreads();
-    }
-    if (SRC == SRC_E64 || pass == 1 || blockIdx.x >= c->heavy_chunks) return;
+    const uint32_t wb = (S0 & ~3u) + wsel * SLOT_WIN;
+    if (!__any_sync(0xffffffffu, most > 5u || j < wb || Rs[SLOT_PER - 1] - wb > SLOT_WIN))
+      win_mark(s_win, wb, j, Rs, mk0);
+    else
+      win_mark_clipped<SLOT_WIN>(s_win, s_run, &s_nruns, wb, j, Rs, mk0);
+    __syncthreads();
+    win_runs<BLOCK>(s_win, s_run, &s_nruns);
+    win_store<BLOCK>(s_win, a.anc, wb, max(S0, wb), min(s_end, wb + SLOT_WIN), (uint32_t)tbase, a.anc_vec);
+    if (pass == 1 || blockIdx.x >= c->heavy_chunks) return;
     // the heavy tile of chunk blockIdx.x: the last entry whose first chunk is
     // not above it
     const uint2* const list = reinterpret_cast<const uint2*>(a.heavy);
