@@ -287,9 +287,14 @@ pf_status launch_resample(int scheme, const MultiArgs& ma, const uint32_t* I, cu
     k_multi<true><<<ma.ntiles, BLOCK, 0, s>>>(ma);
     mark(tm, "cutpoint_method", s);
   } else {
-    k_multi_split<<<(unsigned)cdiv(ma.ntiles + 1, WARPS), BLOCK, 0, s>>>(ma);
-    mark(tm, "split", s);
-    k_multi<false><<<ma.ntiles, BLOCK, 0, s>>>(ma);
+    MultiArgs mb = ma;
+    if (ma.ntiles <= MULTI_OWN) {
+      mb.splits = nullptr;
+    } else {
+      k_multi_split<<<(unsigned)cdiv(ma.ntiles + 1, WARPS), BLOCK, 0, s>>>(ma);
+      mark(tm, "split", s);
+    }
+    k_multi<false><<<ma.ntiles, BLOCK, 0, s>>>(mb);
     mark(tm, "merge", s);
   }
   CK(cudaGetLastError());

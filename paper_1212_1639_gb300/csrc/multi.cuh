@@ -148,25 +148,32 @@ __device__ __forceinline__ uint64_t warp_last(uint64_t lo, uint64_t hi, F below)
   return lo;
 }
 
-// splits[s] = #{i : Q_i S_n <= S T} for S the spacings before slot tile s, one
-// warp per tile: the CDF tile by its prefix, then the particle in the tile.
+// #{i : Q_i S_n <= S T} for S the spacings before slot tile s, by one warp: the
+// CDF tile by its prefix, then the particle in the tile.  Past the last tile: the
+// first particle whose CDF value is T (no ancestor lies beyond it).
+__device__ __forceinline__ uint32_t multi_split(const MultiArgs& a, uint32_t s, uint64_t T, uint64_t A) {
+  const bool end = s == a.ntiles;
+  const U128 key = mul64(end ? T - 1 : a.spre[s], end ? 1ull : T);
+  const uint64_t f = end ? 1ull : A;
+  const uint64_t tile = warp_last(0, a.ntiles - 1, [&](uint64_t i) { return le128(mul64(a.pre[i], f), key); });
+  const uint64_t b = tile * SLOT_TILE, e = b + SLOT_TILE < a.n ? b + SLOT_TILE : a.n;
+  return (uint32_t)warp_last(b, e, [&](uint64_t q) { return le128(mul64(a.Q[q - 1], f), key); });
+}
+// splits[s] of every tile and of the end, one warp each.
 static __global__ void __launch_bounds__(BLOCK) k_multi_split(MultiArgs a) {
   if (a.gate && *a.gate == 0u) return;
-  const uint64_t T = a.ctl->keyT, A = a.ctl->keyS, n = a.n;
-  const int lane = threadIdx.x & 31;
+  const uint64_t T = a.ctl->keyT, A = a.ctl->keyS;
   if (T == 0) return;  // empty CDF (flagged)
   const uint32_t s = blockIdx.x * WARPS + (threadIdx.x >> 5);
   if (s > a.ntiles) return;
-  const U128 key = mul64(s < a.ntiles ? a.spre[s] : A, T);
-  if (s == a.ntiles) {  // (every slot lies before S_n)
-    if (lane == 0) a.splits[s] = (uint32_t)(n - 1);
-    return;
-  }
-  const uint64_t tile = warp_last(0, a.ntiles - 1, [&](uint64_t i) { return le128(mul64(a.pre[i], A), key); });
-  const uint64_t b = tile * SLOT_TILE, e = b + SLOT_TILE < n ? b + SLOT_TILE : n;
-  const uint64_t i = warp_last(b, e, [&](uint64_t q) { return le128(mul64(a.Q[q - 1], A), key); });
-  if (lane == 0) a.splits[s] = (uint32_t)i;
+  const uint32_t i = multi_split(a, s, T, A);
+  if ((threadIdx.x & 31) == 0) a.splits[s] = i;
 }
+// Up to this many slot tiles two warps of each tile's CTA search for its splits
+// themselves, beside the other warps' spacings, and k_multi_split is not launched.
+// Cycle in us, launched / own: N = 16,384 37.0 / 34.9, 2^18 40.8 / 39.0, 2^20 61.0 /
+// 56.8, 2^21 92.8 / 91.6, 2^22 151.6 / 153.8, 2^24 521 / 542.
+constexpr uint32_t MULTI_OWN = 1024;
 
 // The exact ancestor of a slot at S, not before particle i.
 static __device__ __noinline__ uint32_t multi_exact(const uint64_t* Q, uint64_t n, uint64_t S, uint64_t T,
@@ -188,6 +195,7 @@ template <bool CUT>
 __global__ void __launch_bounds__(BLOCK, 4) k_multi(MultiArgs a) {
   __shared__ uint64_t s_q[CUT ? 1 : MULTI_CAP + 1];
   __shared__ uint64_t s_warp[WARPS];
+  __shared__ uint32_t s_split[CUT ? 1 : 2];
   if (a.gate && *a.gate == 0u) return;
   const Ctl* const c = a.ctl;
   const uint64_t n = a.n, T = c->keyT;
@@ -203,19 +211,35 @@ __global__ void __launch_bounds__(BLOCK, 4) k_multi(MultiArgs a) {
   const int z = c->multi_z;
   uint32_t i0 = 0, i1 = 0;
   bool staged = false;
-  if constexpr (!CUT) {
-    i0 = a.splits[blockIdx.x];
-    i1 = a.splits[blockIdx.x + 1];
+  auto stage = [&]() {
     staged = i1 - i0 <= MULTI_CAP;
     if (staged)
       for (uint32_t i = threadIdx.x; i < i1 - i0; i += BLOCK) s_q[i] = a.Q[i0 + i];
     if (threadIdx.x == 0) s_q[staged ? i1 - i0 : 0] = ~0ull;
+  };
+  if constexpr (!CUT) {
+    if (a.splits) {
+      i0 = a.splits[blockIdx.x];
+      i1 = a.splits[blockIdx.x + 1];
+      stage();
+    } else if (warp < 2) {
+      const uint32_t v = multi_split(a, blockIdx.x + warp, T, A);
+      if (lane == 0) s_split[warp] = v;
+    }
   }
   uint64_t run[MULTI_PER];
   spacings8(a, t, j0, run);
   const uint64_t incl = warp_incl_scan(run[MULTI_PER - 1], lane);
   if (lane == 31) s_warp[warp] = incl;
   __syncthreads();
+  if constexpr (!CUT) {
+    if (!a.splits) {
+      i0 = s_split[0];
+      i1 = s_split[1];
+      stage();
+      __syncthreads();
+    }
+  }
   uint64_t off = (lane & 7) < warp ? s_warp[lane & 7] : 0;
 #pragma unroll
   for (int o = 4; o > 0; o >>= 1) off += __shfl_xor_sync(0xffffffffu, off, o);
@@ -225,9 +249,43 @@ __global__ void __launch_bounds__(BLOCK, 4) k_multi(MultiArgs a) {
     if (nextq - P < 5ull) an = multi_exact(a.Q, n, S0 + run[e], T, A, an);
     out[e] = an < n ? an : (uint32_t)(n - 1);
   };
-  if (CUT || staged) {
+  if constexpr (CUT) {
+    // four slots' table entries, then their CDF values, then their climbs step by
+    // step together, so that the loads of four are in flight at once (one slot
+    // after the other a cycle of 8193 particles was 10 us longer)
+    const uint64_t brho = c->bucket_rho;
+#pragma unroll
+    for (int h = 0; h < MULTI_PER; h += 4) {
+      uint64_t P[4], nextq[4];
+      uint32_t i[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        // bucket floor(n S / A): X is low by less than 4 units of 2^-32, and a
+        // bucket one too low only starts the climb earlier
+        const uint64_t S = (S0 + run[h + e]) << z;
+        P[e] = slot_x(S, rho);
+        const uint32_t b = (uint32_t)(slot_x(S, brho) >> 32);
+        i[e] = a.I[b < n ? b : n - 1];
+      }
+#pragma unroll
+      for (int e = 0; e < 4; ++e) nextq[e] = a.Q[i[e]];
+      bool more = true;
+      while (more) {
+        more = false;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          if (nextq[e] <= P[e] && i[e] + 1 < n) {
+            nextq[e] = a.Q[++i[e]];
+            more = true;
+          }
+        }
+      }
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (j0 + h + e < n) keep(h + e, P[e], nextq[e], i[e]);
+    }
+  } else if (staged) {
     uint32_t i = 0;
-    const uint64_t brho = CUT ? c->bucket_rho : 0;
     const uint32_t cnt = i1 - i0;
     auto bisect = [&](uint64_t P) {
       uint32_t hi = cnt;
@@ -239,29 +297,19 @@ __global__ void __launch_bounds__(BLOCK, 4) k_multi(MultiArgs a) {
     };
 #pragma unroll
     for (int e = 0; e < MULTI_PER; ++e) {
-      const uint64_t S = (S0 + run[e]) << z, P = slot_x(S, rho);
+      const uint64_t P = slot_x((S0 + run[e]) << z, rho);
       if (j0 + e < n) {
-        if constexpr (CUT) {
-          // bucket floor(n S / A): X is low by less than 4 units of 2^-32, and a
-          // bucket one too low only starts the climb earlier
-          const uint32_t b = (uint32_t)(slot_x(S, brho) >> 32);
-          i = a.I[b < n ? b : n - 1];
-          uint64_t nextq = a.Q[i];
-          while (nextq <= P && i + 1 < n) nextq = a.Q[++i];
-          keep(e, P, nextq, i);
+        if (e == 0) {
+          bisect(P);
         } else {
-          if (e == 0) {
-            bisect(P);
-          } else {
-            uint32_t steps = 0;
-            while (steps < 16u && s_q[i] <= P) {
-              ++i;
-              ++steps;
-            }
-            if (steps == 16u) bisect(P);
+          uint32_t steps = 0;
+          while (steps < 16u && s_q[i] <= P) {
+            ++i;
+            ++steps;
           }
-          keep(e, P, s_q[i], i0 + i);
+          if (steps == 16u) bisect(P);
         }
+        keep(e, P, s_q[i], i0 + i);
       }
     }
   } else {
