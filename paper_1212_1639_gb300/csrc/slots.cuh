@@ -180,8 +180,11 @@ static __device__ __noinline__ uint64_t div_2by1(uint64_t hi, uint64_t lo, uint6
 // R = (Y >> 32) + 1 unless Y is within 4 of a whole number.  Stratified: with
 // c = X >> 32, slot c is below n Q when r_c / T < frac(n Q / T); r_c / T is the
 // leading 32 bits u of slot c's uniform to within a unit, so R = c + (frac > u)
-// unless they are within 5.  The doubtful cases (one in 2^29) take the exact
-// divisions below.  A high product per particle where a walk would carry a
+// unless they are within 5.  The doubtful cases take the exact divisions of
+// slot_below_exact: one in 2^29, and Q = 0 and Q = T, which the stratified map and
+// the cut-point table meet in every call and which are told apart there (by
+// divisions, with the thread's other values, they made a cycle of 8193 particles
+// 2 to 4 us longer).  A high product per particle where a walk would carry a
 // 64-bit remainder from one particle to the next and compare it with T, 2 T
 // and 3 T.
 // Stratified: the 32-bit uniforms of the slots a tile can reach come from a
@@ -204,13 +207,6 @@ __device__ __forceinline__ uint64_t slot_x(uint64_t q, uint64_t rho) {
   const uint32_t rh = (uint32_t)(rho >> 32), rl = (uint32_t)rho;
   return (uint64_t)qh * rh + __umulhi(qh, rl) + __umulhi(ql, rh);
 }
-template <int POS>
-static __device__ __noinline__ uint32_t slot_below_exact(uint64_t q, const Ctl* c, uint64_t n,
-                                                         uint64_t seed, uint32_t filter, uint32_t t) {
-  const SysDiv dv = make_sysdiv(c->keyT);
-  if (POS == SLOTS_SYS) return (uint32_t)sys_first_slot(q, n, c->keyR, dv);
-  return (uint32_t)strat_first(q, n, c->keyT, dv, seed, filter, t);
-}
 // R of Q 2^z; *close falls below 8 when R is doubtful
 template <int POS>
 __device__ __forceinline__ uint32_t slot_below(uint64_t q, const SlotMap& m, uint32_t* close) {
@@ -222,10 +218,35 @@ __device__ __forceinline__ uint32_t slot_below(uint64_t q, const SlotMap& m, uin
   } else {
     const uint32_t c = (uint32_t)(X >> 32), f = (uint32_t)X;
     const uint32_t i = c - m.u0;
-    const uint32_t u = i < m.nu ? m.u[i] : strat_u32(c, m.seed, m.filter, m.t);
+    // (a value as close to a whole number as Q = T is doubtful whatever u is)
+    const uint32_t u = i < m.nu ? m.u[i] : f + 8u < 8u ? 0u : strat_u32(c, m.seed, m.filter, m.t);
     *close = min(*close, min(f + 8u, f - u + 5u));
     return c + (f > u ? 1u : 0u);
   }
+}
+
+// R of one of a thread's values when one or more of them are doubtful: the ends and
+// the others without a division.
+template <int POS>
+static __device__ __noinline__ uint32_t slot_below_exact(uint64_t q, const Ctl* c, uint64_t n,
+                                                         uint64_t seed, uint32_t filter, uint32_t t) {
+  const uint64_t T = c->keyT;
+  if (q == 0) return 0;
+  if (q == T) return (uint32_t)n;
+  SlotMap m;
+  m.rho = c->slot_rho;
+  m.r32 = c->slot_r32;
+  m.u = nullptr;
+  m.u0 = m.nu = 0;
+  m.seed = seed;
+  m.filter = filter;
+  m.t = t;
+  uint32_t close = ~0u;
+  const uint32_t v = slot_below<POS>(q << c->slot_z, m, &close);
+  if (close >= 8u) return v;
+  const SysDiv dv = make_sysdiv(T);
+  if (POS == SLOTS_SYS) return (uint32_t)sys_first_slot(q, n, c->keyR, dv);
+  return (uint32_t)strat_first(q, n, T, dv, seed, filter, t);
 }
 
 // The last CTA of k_sums (out of line: its registers are not the others').
