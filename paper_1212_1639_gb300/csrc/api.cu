@@ -343,7 +343,10 @@ void launch_cdf(pf_filter* f, cudaStream_t s, KTimer* tm) {
   a.src_vec = a.anc_vec = 1;
   const unsigned sg = sums_grid(f->n);
   const int pos = slot_pos(f->scheme);
-  if (pos != SLOTS_NONE) a.heavy = (char*)f->pre + pre_bytes(f->n);
+  // (no list where a tile's own CTA stores all the windows it can have)
+  constexpr int SRC = sizeof(R) == 8 ? SRC_E64 : SRC_LOG;
+  if (pos != SLOTS_NONE && (HeavyRule<SRC>::OWN == 0 || f->n > (HeavyRule<SRC>::OWN + 1) * SLOT_WIN))
+    a.heavy = (char*)f->pre + pre_bytes(f->n);
   if constexpr (sizeof(R) == 8) {
     a.src = f->Q;
     a.l = (const double*)f->ell;

@@ -97,6 +97,26 @@ __device__ __forceinline__ void st4(uint64_t* p, uint64_t a, uint64_t b, uint64_
   asm volatile("st.global.v4.b64 [%0], {%1,%2,%3,%4};" ::"l"(p), "l"(a), "l"(b), "l"(c), "l"(d) : "memory");
 }
 
+// The further windows of a tile of weight `sum` that other CTAs store (k_sums
+// lists it), 0: its own CTA stores all its windows, up to OWN past the first.
+// The estimate of its slots is within 32 of them, so a last window may turn out
+// empty.  A window by the tile's own CTA takes 0.9 us, the tile built once more by
+// another 2.5, in binary64, where that takes the exponentials again, 5.
+template <int SRC>
+struct HeavyRule {
+  static constexpr uint32_t OWN = SRC == SRC_E64 ? 6 : 0;
+  float per_slot;
+  uint64_t most;  // a tile of at most this is not listed
+  __device__ __forceinline__ HeavyRule(uint64_t T, uint64_t n) {
+    const float Tf = __ull2float_rn(T), nf = (float)n;
+    per_slot = nf / Tf;
+    most = f2u64_rz(Tf * ((float)((OWN + 1) * SLOT_WIN - 16) / nf));
+  }
+  __device__ __forceinline__ uint32_t operator()(uint64_t sum) const {
+    return sum > most ? (uint32_t)((__ull2float_rn(sum) * per_slot + 40.0f) * (1.0f / SLOT_WIN)) : 0u;
+  }
+};
+
 template <int SRC> struct SrcT { typedef float R; };
 template <> struct SrcT<SRC_E64> { typedef double R; };
 
@@ -324,14 +344,12 @@ static __device__ __noinline__ void sums_last(const SlotArgs& a, uint64_t* s_tot
     if (w < warp) run += s_tot[w];
     T += s_tot[w];
   }
-  // (a group's entries past the last tile are padding).  heavy: a tile of about
-  // a window's slots or more, sum > (window - 16) T / n in binary32
+  // (a group's entries past the last tile are padding)
   bool heavy = false;
-  const float Tf = __ull2float_rn(T), nf = (float)a.n;
-  const uint64_t most = f2u64_rz(Tf * ((float)(SLOT_WIN - 16) / nf));
+  const HeavyRule<SRC> rule(T, a.n);
   auto put4 = [&](uint32_t i, const uint64_t* v) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) heavy |= v[q] > most;
+    for (int q = 0; q < 4; ++q) heavy |= v[q] > rule.most;
     const uint64_t r1 = run + v[0], r2 = r1 + v[1], r3 = r2 + v[2];
     if (i < t1) st4(a.pre + i, run, r1, r2, r3);
     run = r3 + v[3];
@@ -409,23 +427,17 @@ static __device__ __noinline__ void sums_last(const SlotArgs& a, uint64_t* s_tot
     if (threadIdx.x == 0) c->heavy_chunks = 0;
     return;
   }
-  // The heavy list: tiles of about a window's slots or more, in tile order, with
-  // the number of their first chunk.  A chunk is one further window; the
-  // estimate of a tile's slots is within 32 of them, so a last window may turn
-  // out empty.
-  const float per_slot = nf / Tf;
-  auto chunks = [&](uint64_t sum) -> uint32_t {
-    return sum > most ? (uint32_t)((__ull2float_rn(sum) * per_slot + 40.0f) * (1.0f / SLOT_WIN)) : 0u;
-  };
+  // The heavy list: the tiles whose further windows other CTAs store, in tile
+  // order, with the number of their first chunk (a chunk is one such window).
   // each of this thread's heavy tiles, in order (the first sums from registers:
   // a trip to L2 per tile took 3 us here)
   auto each = [&](auto f) {
     if (!heavy) return;
 #pragma unroll
     for (uint32_t i = 0; i < KEEP; ++i)
-      if (const uint32_t k = chunks(kept[i])) f(t0 + i, k);
+      if (const uint32_t k = rule(kept[i])) f(t0 + i, k);
     for (uint32_t i = t0 + KEEP; i < t1; ++i)
-      if (const uint32_t k = chunks((i + 1 < a.ntiles ? a.pre[i + 1] : T) - a.pre[i])) f(i, k);
+      if (const uint32_t k = rule((i + 1 < a.ntiles ? a.pre[i + 1] : T) - a.pre[i])) f(i, k);
   };
   uint64_t cnt = 0;  // entries, then chunks
   each([&](uint32_t, uint32_t k) { cnt += (1ull << 32) + k; });
@@ -638,12 +650,12 @@ static __device__ __noinline__ double heavy_exp64(const SlotArgs& a, uint64_t i)
 // path per heavy particle (k_slots at N = 2^24 on weights of log-spread 1:
 // 112 -> 64 us).
 //
-// A tile of more slots than its window leaves the others to the CTAs of the
-// heavy list (k_sums): CTA b < heavy_chunks, after its own tile, rebuilds the
-// heavy tile of chunk b and stores that window.  With all the mass on one particle
-// of 2^23 the kernel takes 43 us (binary64 55), by one CTA window after window
-// 2.5 ms.  Binary64 overwrites its source with Q, so there the heavy tile is
-// rebuilt from l.
+// A tile of more slots than its window (binary64: than seven) holds leaves the
+// others to the CTAs of the heavy list (k_sums): CTA b < heavy_chunks, after its
+// own tile, rebuilds the heavy tile of chunk b and stores that window.  With all
+// the mass on one particle of 2^23 the kernel takes 43 us (binary64 55), by one
+// CTA window after window 2.5 ms.  Binary64 overwrites its source with Q, so there
+// the heavy tile is rebuilt from l.
 template <int SRC, int POS>
 __global__ void __launch_bounds__(BLOCK, 4) k_slots(SlotArgs a) {
   typedef typename SrcT<SRC>::R R;
@@ -759,14 +771,23 @@ __global__ void __launch_bounds__(BLOCK, 4) k_slots(SlotArgs a) {
 #pragma unroll
     for (int e = 1; e < SLOT_PER; ++e) most = max(most, Rs[e] - Rs[e - 1]);
     // the window's base: slots in aligned groups of four
-    const uint32_t wb = (S0 & ~3u) + wsel * SLOT_WIN;
-    if (!__any_sync(0xffffffffu, most > 5u || j < wb || Rs[SLOT_PER - 1] - wb > SLOT_WIN))
-      win_mark(s_win, wb, j, Rs, mk0);
-    else
-      win_mark_clipped<SLOT_WIN>(s_win, s_run, &s_nruns, wb, j, Rs, mk0);
-    __syncthreads();
-    win_runs<BLOCK>(s_win, s_run, &s_nruns);
-    win_store<BLOCK>(s_win, a.anc, wb, max(S0, wb), min(s_end, wb + SLOT_WIN), (uint32_t)tbase, a.anc_vec);
+    uint32_t wb = (S0 & ~3u) + wsel * SLOT_WIN;
+    while (true) {
+      if (!__any_sync(0xffffffffu, most > 5u || j < wb || Rs[SLOT_PER - 1] - wb > SLOT_WIN))
+        win_mark(s_win, wb, j, Rs, mk0);
+      else
+        win_mark_clipped<SLOT_WIN>(s_win, s_run, &s_nruns, wb, j, Rs, mk0);
+      __syncthreads();
+      win_runs<BLOCK>(s_win, s_run, &s_nruns);
+      win_store<BLOCK>(s_win, a.anc, wb, max(S0, wb), min(s_end, wb + SLOT_WIN), (uint32_t)tbase, a.anc_vec);
+      wb += SLOT_WIN;
+      if (HeavyRule<SRC>::OWN == 0 || pass == 1 || s_end <= wb) break;
+      const uint64_t next = tile + 1 < a.ntiles ? a.pre[tile + 1] : c->keyT;
+      if (HeavyRule<SRC>(c->keyT, n)(next - pre)) break;
+      __syncthreads();  // the window has been read
+      clear();
+      __syncthreads();
+    }
     if (pass == 1 || blockIdx.x >= c->heavy_chunks) return;
     // the heavy tile of chunk blockIdx.x: the last entry whose first chunk is
     // not above it
