@@ -343,9 +343,10 @@ void launch_cdf(pf_filter* f, cudaStream_t s, KTimer* tm) {
   a.src_vec = a.anc_vec = 1;
   const unsigned sg = sums_grid(f->n);
   const int pos = slot_pos(f->scheme);
-  // (no list where a tile's own CTA stores all the windows it can have)
+  // (no list where no tile can have more windows than its own CTA stores: 64
+  // slots below HeavyRule's line, which is drawn on an estimate)
   constexpr int SRC = sizeof(R) == 8 ? SRC_E64 : SRC_LOG;
-  if (pos != SLOTS_NONE && (HeavyRule<SRC>::OWN == 0 || f->n > (HeavyRule<SRC>::OWN + 1) * SLOT_WIN))
+  if (pos != SLOTS_NONE && (HeavyRule<SRC>::OWN == 0 || f->n > (HeavyRule<SRC>::OWN + 1) * SLOT_WIN - 64))
     a.heavy = (char*)f->pre + pre_bytes(f->n);
   if constexpr (sizeof(R) == 8) {
     a.src = f->Q;

@@ -32,6 +32,23 @@ def test_filter_with_heavy_tiles(pf, orc, prec, scheme, ess):
     g.close()
 
 
+@pytest.mark.parametrize("scheme", ["systematic", "stratified"])
+@pytest.mark.parametrize("n", [4097, 8193, 12_289, 28_607, 28_608, 28_609, 28_656, 28_657, 28_672, 28_673, 32_769])
+def test_binary64_windows_of_one_tile(pf, orc, n, scheme):
+    """All slots in one tile: its own CTA stores seven windows, other CTAs the rest."""
+    g = pf.Filter(n, seed=n, scheme=scheme, precision="fp64", **KW)
+    o = orc.Filter(orc.make_config(n, seed=n, scheme=pf.SCHEMES[scheme], precision=1, **KW))
+    tiles = []
+    for y in (60.0, -60.0, 60.0):
+        g.step(y)
+        o.step(y)
+        a = g.ancestors().cpu().numpy().view(np.uint32)
+        assert np.array_equal(a, o.ancestors()), y
+        tiles.append(len(np.unique(a // 2048)))
+    assert min(tiles) == 1
+    g.close()
+
+
 @pytest.mark.parametrize("prec", ["fp32", "fp64"])
 @pytest.mark.parametrize("shape", [None, (512, 152, 1, 0), (256, 152, 8, 16384), (512, 152, 8, 16384)])
 def test_batch_with_heavy_particles(pf, prec, shape):
