@@ -429,14 +429,8 @@ static __device__ __noinline__ void sums_last(const SlotArgs& a, uint64_t* s_tot
   }
   // The heavy list: the tiles whose further windows other CTAs store, in tile
   // order, with the number of their first chunk (a chunk is one such window).
-  // each of this thread's heavy tiles, in order (the first sums from registers:
-  // a trip to L2 per tile took 3 us here)
   auto each = [&](auto f) {
-    if (!heavy) return;
-#pragma unroll
-    for (uint32_t i = 0; i < KEEP; ++i)
-      if (const uint32_t k = rule(kept[i])) f(t0 + i, k);
-    for (uint32_t i = t0 + KEEP; i < t1; ++i)
+    for (uint32_t i = t0; i < t1; ++i)
       if (const uint32_t k = rule((i + 1 < a.ntiles ? a.pre[i + 1] : T) - a.pre[i])) f(i, k);
   };
   uint64_t cnt = 0;  // entries, then chunks
