@@ -38,6 +38,15 @@ pf_status pf_diag_cdf_wait(const float* w_dev, uint64_t n, uint32_t withhold_til
 pf_status pf_diag_block(pf_alloc_fn alloc, pf_free_fn free, void* ctx, size_t bytes, void** raw,
                         void** start);
 
+/* The correctly rounded arithmetic that the kernels use in place of the
+ * compiler's division and square root, element by element on device arrays of
+ * n values (8-byte aligned).  op 0..8: binary32, n even, the values taken in
+ * pairs: 0 1/a, 1 a/b, 2 sqrt a, 3 sqrt a one value at a time, 4 a/b of the
+ * predictive weights (any operands), 5 and 6 a/b of the inverse-gamma draws for
+ * shapes below and from 2^60, 7 1/(a+b) and 8 sqrt((a b) (1/(a+b))) of the
+ * propagation.  op 16, 17: binary64 a/b and sqrt a.  Synchronises `stream`. */
+pf_status pf_diag_arith(int op, const void* a, const void* b, void* out, uint64_t n, void* stream);
+
 #ifdef __cplusplus
 }
 #endif

@@ -14,8 +14,8 @@ CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 LIB = os.path.join(HERE, "libpf.so")
 SOURCES = ["api.cu", "batch_f32.cu", "batch_f64.cu"]
-DEPS = ["api.cu", "batch_f32.cu", "batch_f64.cu", "kernels.cuh", "device.cuh", "slots.cuh", "multi.cuh", "small.cuh", "batch.cuh",
-        "batch_launch.h", "batch_kernels.cuh", "batch_api.cuh", "server_api.cuh"]
+DEPS = ["api.cu", "batch_f32.cu", "batch_f64.cu", "kernels.cuh", "device.cuh", "slots.cuh", "multi.cuh", "small.cuh", "diag.cuh",
+        "batch.cuh", "batch_launch.h", "batch_kernels.cuh", "batch_api.cuh", "server_api.cuh"]
 ARCH = "-gencode=arch=compute_103a,code=sm_103a"
 
 
@@ -30,7 +30,8 @@ def _stale():
     if not os.path.exists(LIB):
         return True
     t = os.path.getmtime(LIB)
-    files = [os.path.join(CSRC, d) for d in DEPS] + [os.path.join(INCLUDE, "pf.h"), __file__]
+    files = [os.path.join(CSRC, d) for d in DEPS] + [__file__]
+    files += [os.path.join(INCLUDE, h) for h in ("pf.h", "pf_diag.h")]
     return any(os.path.getmtime(f) > t for f in files)
 
 

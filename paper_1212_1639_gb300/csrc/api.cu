@@ -18,6 +18,7 @@
 #include "../../include/pf_diag.h"
 #include "kernels.cuh"
 #include "small.cuh"
+#include "diag.cuh"
 
 using namespace pfk;
 
@@ -1601,6 +1602,22 @@ pf_status pf_diag_block(pf_alloc_fn alloc, pf_free_fn free, void* ctx, size_t by
                         void** start) {
   if (!alloc || !free || !raw || !start) return set_err(PF_ERR_INVALID, "NULL pointer");
   return device_block(alloc, free, ctx, nullptr, bytes, raw, start);
+}
+
+pf_status pf_diag_arith(int op, const void* a, const void* b, void* out, uint64_t n, void* stream) {
+  if (!a || !b || !out) return set_err(PF_ERR_INVALID, "NULL pointer");
+  const bool f32 = op >= 0 && op < OP_F32_COUNT;
+  if (!f32 && op != OP_DIV64 && op != OP_SQRT64) return set_err(PF_ERR_INVALID, "bad operation");
+  if (n < 1 || n > (1ull << 30) || (f32 && n % 2 != 0)) return set_err(PF_ERR_INVALID, "bad count");
+  if (((uintptr_t)a | (uintptr_t)b | (uintptr_t)out) & 7) return set_err(PF_ERR_INVALID, "not 8-byte aligned");
+  cudaStream_t s = (cudaStream_t)stream;
+  if (f32)
+    k_arith32<<<(unsigned)cdiv(n / 2, BLOCK), BLOCK, 0, s>>>(op, (const float2*)a, (const float2*)b, (float2*)out, n / 2);
+  else
+    k_arith64<<<(unsigned)cdiv(n, BLOCK), BLOCK, 0, s>>>(op, (const double*)a, (const double*)b, (double*)out, n);
+  CK(cudaGetLastError());
+  CK(cudaStreamSynchronize(s));
+  return PF_OK;
 }
 
 pf_status pf_cutpoint_search(const uint64_t* Q_dev, uint64_t n, uint32_t* I_dev, void* stream) {

@@ -297,6 +297,10 @@ __device__ __forceinline__ R log_pred(R x, R s2, R t2, R y) {
   return (R)-0.5 * sum;
 }
 
+// a / b of a pair: paired where both lanes' operands are safe for it
+__device__ __forceinline__ float2 quot2(float2 a, float2 b) {
+  return pair_safe(b, a) ? div_rn2(a, b) : make_float2(a.x / b.x, a.y / b.y);
+}
 // log_pred on two particles with paired operations; per lane the same IEEE
 // operations in the same order, so the same bits.
 __device__ __forceinline__ float2 log_pred2(float2 x, float2 s2, float2 t2, float yn) {
@@ -304,7 +308,7 @@ __device__ __forceinline__ float2 log_pred2(float2 x, float2 s2, float2 t2, floa
   const float2 dx = sub2(splat2(yn), x);
   const float2 q = mul2(dx, dx);
   const float2 lg = det_log2(s);
-  const float2 r = pair_safe(s, q) ? div_rn2(q, s) : make_float2(q.x / s.x, q.y / s.y);
+  const float2 r = quot2(q, s);
   const float2 sum = add2(lg, r);
   return mul2(splat2(-0.5f), sum);
 }

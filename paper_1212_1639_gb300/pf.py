@@ -137,6 +137,7 @@ _SIGS = {
     "pf_resample_noalloc": [_V, C.c_uint64, C.c_uint64, C.c_uint32, C.c_uint32, C.c_int32, _V,
                             _V],
     "pf_cdf": [_V, C.c_uint64, _V, _V],
+    "pf_diag_arith": [C.c_int32, _V, _V, _V, C.c_uint64, _V],
     "pf_diag_block": [ALLOC_FN, FREE_FN, _V, C.c_size_t, C.POINTER(_V), C.POINTER(_V)],
     "pf_diag_cdf_wait": [_V, C.c_uint64, C.c_uint32, C.c_uint32, _V, _V],
     "pf_cutpoint_search": [_V, C.c_uint64, _V, _V],
@@ -723,6 +724,18 @@ def diag_cdf_wait(w, withhold_tile, spin_limit, stream=None):
         st = _lib.pf_diag_cdf_wait(_ptr(w), w.numel(), int(withhold_tile), int(spin_limit), _ptr(Q),
                                    _stream_ptr(stream))
     return st, Q
+
+
+def diag_arith(op, a, b, stream=None):
+    """pf_diag_arith on two CUDA tensors of one type and size."""
+    torch = _torch()
+    assert a.is_cuda and b.is_cuda and a.dtype == b.dtype and a.numel() == b.numel()
+    assert a.is_contiguous() and b.is_contiguous()
+    assert a.dtype == (torch.float64 if op >= 16 else torch.float32)
+    out = torch.empty_like(a)
+    _check(_lib.pf_diag_arith(int(op), _ptr(a), _ptr(b), _ptr(out), a.numel(), _stream_ptr(stream)),
+           "pf_diag_arith")
+    return out
 
 
 def cutpoint_search(Q, stream=None):
