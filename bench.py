@@ -175,7 +175,7 @@ def pow2_label(n):
 
 def kernels_hash():
     h = hashlib.sha256()
-    for f in ("kernels.cuh", "slots.cuh", "device.cuh"):
+    for f in ("kernels.cuh", "slots.cuh", "multi.cuh", "small.cuh", "device.cuh"):
         h.update(open(os.path.join(ROOT, "paper_1212_1639_gb300", "csrc", f), "rb").read())
     return h.hexdigest()[:16]
 

@@ -61,13 +61,13 @@ typedef enum {
  *                         paper's parallelized cut-point search and cut-point
  *                         method (Section 3.2); identical output.
  *  SYSTEMATIC_CUTPOINT    same positions as SYSTEMATIC, cut-point search.
- *                         In the cut-point search thread i writes the whole
- *                         run of table entries that point at particle i, as
- *                         the paper's algorithm does; under degenerate
- *                         weights (one particle holding nearly all the mass,
- *                         the worst case Section 3.2 discusses) one thread
- *                         writes up to n entries serially, so both
- *                         *_CUTPOINT schemes take O(n) time there.  The
+ *                         The table is built by whole warps or blocks, so
+ *                         a particle that holds nearly all the mass costs no
+ *                         serial run of entries (the worst case Section 3.2
+ *                         discusses).  The cut-point method climbs as the
+ *                         paper's does, entry by entry: where many particles
+ *                         of little weight share a bucket, a slot of that
+ *                         bucket climbs over all of them, up to O(n).  The
  *                         other schemes have no such case.
  *  STRATIFIED             positions = (j + u_j) T / n, one uniform u_j in
  *                         each stratum (Section 3.1, "Stratified

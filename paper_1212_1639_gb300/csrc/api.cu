@@ -92,7 +92,7 @@ struct pf_filter {
   cudaStream_t stream = nullptr;
   bool own_stream = false;
   // multinomial schemes: the exponential spacings need nothing from the
-  // cycle's weights or CDF, so they are scanned on a second stream, forked
+  // cycle's weights or CDF, so they are summed on a second stream, forked
   // from and joined back into the filter's stream (a parallel branch of the
   // captured graph)
   cudaStream_t side = nullptr;
@@ -374,10 +374,6 @@ void launch_cdf(pf_filter* f, cudaStream_t s, KTimer* tm) {
   mark(tm, pos == SLOTS_NONE ? "cdf" : a.cut ? "cutpoint_search" : "cdf_resample", s);
 }
 
-// One cycle (Steps 1-4), enqueued on f->stream; reads t and y on the device.
-// With form CF_HEAD / CF_MID the propagation also computes the next cycle's
-// weights against y_{t+2} (*ynx_src when set, else ynx_val); with CF_MID /
-// CF_TAIL the weights kernel is left out, its work done by the previous cycle.
 // The binary32 propagation, slots handed out by ticket in the learning forms
 // where each warp has many 64-slot units (PROP_DYN).
 template <bool LEARN, bool FUSE, bool ESS>
@@ -390,6 +386,10 @@ void launch_prop2(unsigned grid, cudaStream_t s, const FilterArgs<float>& a) {
   }
   k_propagate2<LEARN, FUSE, ESS, false><<<grid, BLOCK, 0, s>>>(a);
 }
+// One cycle (Steps 1-4), enqueued on f->stream; reads t and y on the device.
+// With form CF_HEAD / CF_MID the propagation also computes the next cycle's
+// weights against y_{t+2} (*ynx_src when set, else ynx_val); with CF_MID /
+// CF_TAIL the weights kernel is left out, its work done by the previous cycle.
 template <class R>
 pf_status enqueue_cycle(pf_filter* f, KTimer* tm = nullptr, const double* y_src = nullptr,
                         double y_val = 0.0, int form = CF_PLAIN, const double* ynx_src = nullptr,
@@ -1313,7 +1313,7 @@ struct Scratch {
   uint64_t* pre;          // CDF tile prefixes, then the heavy list
   uint64_t* spre;
   uint32_t* splits;
-  uint64_t* stat[2];      // pf_cdf: tile status of the scan
+  uint64_t* stat;         // pf_cdf: tile status of the scan
   Ctl* ctl;
 };
 
@@ -1333,8 +1333,7 @@ size_t scratch_layout(uint64_t n, int scheme, bool cdf, char* base, Scratch* s) 
     return p;
   };
   s->ctl = (Ctl*)take(true, sizeof(Ctl));
-  s->stat[0] = (uint64_t*)take(cdf, ntiles * 8);
-  s->stat[1] = (uint64_t*)take(cdf, ntiles * 8);
+  s->stat = (uint64_t*)take(cdf, ntiles * 8);
   s->pre = (uint64_t*)take(!cdf, pre_heavy_bytes(n));
   s->spre = (uint64_t*)take(!cdf && is_multinomial(scheme), pre_bytes(n));
   s->splits = (uint32_t*)take(!cdf && is_multinomial(scheme), ((size_t)slot_tiles(n) + 1) * 4);
@@ -1345,7 +1344,7 @@ size_t scratch_layout(uint64_t n, int scheme, bool cdf, char* base, Scratch* s) 
 
 // The leading bytes that must start at zero.
 size_t scratch_zero_bytes(uint64_t n, bool cdf) {
-  return align256(sizeof(Ctl)) + (cdf ? 2 * align256(cdiv(n, TILE) * 8) : 0);
+  return align256(sizeof(Ctl)) + (cdf ? align256(cdiv(n, TILE) * 8) : 0);
 }
 
 // Weights -> ancestors, or the CDF, on stream s with the
@@ -1409,11 +1408,8 @@ pf_status run_resample(const float* w, uint64_t n, uint64_t seed, uint32_t filte
   ScanArgs sa;
   sa.src = w;
   sa.Q = Q_out;
-  sa.stat[0] = sc.stat[0];
-  sa.stat[1] = sc.stat[1];
+  sa.stat = sc.stat;
   sa.ctl = sc.ctl;
-  sa.t_dev = nullptr;
-  sa.t_arg = 0;
   sa.n = n;
   sa.k = cdf_shift(n);
   sa.vec_ok = ((uintptr_t)w & 15) == 0;

@@ -5,11 +5,12 @@
 // first) and runs the complete cycle of a filter with block barriers only:
 //   1. predictive weights l_i and their maximum (Algorithm "Particle
 //      Learning", Step 1),
-//   2. the exact fixed-point CDF (Section 3) by a chunked block scan with a
-//      carry between chunks,
-//   3. resampling (Section 3.1): systematic by a per-thread walk over equally
-//      spaced slot keys, multinomial by exponential spacings (a second
-//      chunked block scan) and the same walk over the sorted position keys,
+//   2. the exact fixed-point CDF (Section 3) and
+//   3. resampling (Section 3.1): systematic by the sums of the filter's (in a
+//      cluster, of each CTA's) weights, then tile by tile the CDF from its prefix
+//      and the slots by the slot map, as k_slots does; multinomial by a chunked
+//      block scan with a carry between chunks, exponential spacings (a second
+//      such scan) and a per-thread walk over the sorted position keys,
 //   4. propagation of x, the sufficient statistics and theta (Steps 2-4),
 //      with the block's queue of gamma draws that missed the squeeze,
 // then folds the filter's log marginal likelihood increment and advances its

@@ -97,9 +97,6 @@ __device__ __forceinline__ uint64_t ld_status(const uint64_t* p) {
   asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
   return v;
 }
-__device__ __forceinline__ uint32_t ld_volatile_u32(const uint32_t* p) {
-  return *(volatile const uint32_t*)p;
-}
 
 template <class T>
 __device__ __forceinline__ T shfl_up(T v, int d) {
@@ -682,11 +679,8 @@ __device__ __forceinline__ uint64_t quant_weight(float w, int s) {
 struct ScanArgs {
   const float* src;         // weights
   uint64_t* Q;
-  uint64_t* stat[2];        // tile status by cycle parity; the other parity's
-                            // entries are cleared for the next cycle
+  uint64_t* stat;           // tile status, zero before the launch
   Ctl* ctl;
-  const uint32_t* t_dev;    // cycle index in device memory, or NULL
-  uint32_t t_arg;
   uint64_t n;
   int k;
   int vec_ok;               // src is 16-byte aligned
@@ -709,9 +703,6 @@ static __global__ void __launch_bounds__(BLOCK, 4) k_scan(ScanArgs a) {
   __syncthreads();
   const uint32_t tile = s_tile;
   const uint64_t base = (uint64_t)tile * TILE + (uint64_t)threadIdx.x * SCAN_PER;
-  const uint32_t par = (a.t_dev ? *a.t_dev : a.t_arg) & 1u;
-  uint64_t* const stat = par ? a.stat[1] : a.stat[0];
-  uint64_t* const stat_next = par ? a.stat[0] : a.stat[1];
   // quantisation is relative to the power of two of the largest weight
   int e2;
   (void)frexpf(__uint_as_float((uint32_t)a.ctl->maxenc), &e2);
@@ -759,11 +750,8 @@ static __global__ void __launch_bounds__(BLOCK, 4) k_scan(ScanArgs a) {
   if (warp == 0) {
     // tile total = last thread's staged inclusive value
     const uint64_t total = s_stage[(BLOCK - 1) * (SCAN_PER + 1) + SCAN_PER - 1];
-    const uint64_t excl = lookback(stat, tile, total, &a.ctl->err, a.spin_limit, a.withhold);
-    if (lane == 0) {
-      s_excl = excl;
-      stat_next[tile] = 0;
-    }
+    const uint64_t excl = lookback(a.stat, tile, total, &a.ctl->err, a.spin_limit, a.withhold);
+    if (lane == 0) s_excl = excl;
   }
   __syncthreads();
   const uint64_t off = s_excl;
@@ -1201,9 +1189,10 @@ __device__ __forceinline__ Gathered<R> gather_rec(const StateV<R>& src, uint32_t
   return g;
 }
 
-// Persistent grid: a thread handles the slots spread_slot() + k * stride.  The ancestor index is loaded two slots ahead and the ancestor's
-// record one slot ahead, so the dependent index -> gather latency overlaps the
-// arithmetic of the current slot.
+// Persistent grid: a thread handles the slots spread_slot() + k * stride.  The
+// ancestor index is loaded two slots ahead and the ancestor's record one slot
+// ahead, so the dependent index -> gather latency overlaps the arithmetic of the
+// current slot.
 //
 // With FUSE the kernel also computes the next cycle's predictive weights
 // l_j = log p(y_{t+2} | x'_j, sigma^2'_j, tau^2'_j) and their maximum, which
@@ -1359,8 +1348,8 @@ __global__ void __launch_bounds__(BLOCK, 3) k_propagate(FilterArgs<R> a) {
 // ---------------------------------------------------------------------------
 // k_propagate for binary32 state, two slots per thread per pass: the pair
 // 2i, 2i + 1, which shares its second draw (theta_draws2), shares each paired
-// FADD2 / FMUL2 / FFMA2, while divisions, square roots, comparisons and the
-// fixed-point statistics run per lane.  Per slot the operations are those of
+// FMUL2 / FFMA2, its quotients and roots among them (state_scale2, ig2), while
+// additions, comparisons and the fixed-point statistics run per lane.  Per slot the operations are those of
 // the scalar propagation, in the same order, so the results are the same bits.
 // ---------------------------------------------------------------------------
 constexpr uint32_t WQ2_CAP = 160;  // 31 queued + 4 pushes of 32 per pass
