@@ -267,13 +267,42 @@ static __device__ __noinline__ void mark_out(uint16_t* win, uint32_t (*runs)[3],
   win_mark_clipped<WIN>(win, runs, nruns, wb, j, Rs, mk0);
 }
 
+// The slots from wb on of the particle that owns slot wb (in the thread of slots
+// [j, r7), first particle `base`), stored straight by the CTA when they are many.
+// Returns the base of the next window.  (Clusters: with the windows' loop in the
+// kernel and this much out of line they spill 40 bytes instead of 224, 80 filters
+// of 512 to 131,072 particles 164 -> 145 us per cycle; one filter of 131,072 on a
+// cluster of eight, all its mass on one particle, 147 us with every window built
+// and read, 107 so, 129 by one thread's walk over the CDF before.)
+template <int NT>
+static __device__ __noinline__ uint32_t store_owner(uint64_t* own, uint32_t* anc, uint32_t wb, uint32_t base, uint32_t j,
+                                                    uint32_t r0, uint32_t r1, uint32_t r2, uint32_t r3, uint32_t r4,
+                                                    uint32_t r5, uint32_t r6, uint32_t r7) {
+  if (j <= wb && wb < r7) {
+    const uint32_t Rs[SLOT_PER] = {r0, r1, r2, r3, r4, r5, r6, r7};
+    uint32_t o = base, end = r0;
+#pragma unroll
+    for (int e = 1; e < SLOT_PER; ++e)
+      if (Rs[e - 1] <= wb) {
+        o = base + e;
+        end = Rs[e];
+      }
+    *own = (uint64_t)end << 32 | o;
+  }
+  __syncthreads();
+  const uint32_t o = (uint32_t)*own, end = (uint32_t)(*own >> 32), full = end & ~3u;
+  if (end - wb <= (uint32_t)(NT * SLOT_PER / 2)) return wb;
+  for (uint32_t x = wb + 4u * threadIdx.x; x < full; x += 4u * NT)
+    *reinterpret_cast<uint4*>(anc + x) = make_uint4(o, o, o, o);
+  if (threadIdx.x < end - full) anc[full + threadIdx.x] = o;
+  return full;  // (slots [full, end) are stored again, alike)
+}
+
 // The slots from wb on of a tile with more than its first window holds (S0: its
 // first slot), window after window, from the CDF values that its CTA has stored;
-// the slots of a particle that owns many of them go out straight.  Out of line:
-// few tiles come here, and its registers are not the others'.  Cycle of one
-// filter of 131,072 particles on a cluster of eight, all its mass on one
-// particle: 147 us with every window of 4096 slots built and read, 119 so (one
-// thread's walk over the CDF, before: 129).
+// the slots of a particle that owns many of them go out straight.  Filters of one
+// CTA: all of it out of line, which leaves their tiles' loop its registers (4096
+// filters 1262 -> 1168 us per cycle).
 template <class R, int NT>
 static __device__ __noinline__ void batch_windows(BatchSmem<R, NT>& sm, const uint64_t* Q, uint32_t* anc, uint64_t tb,
                                                   uint64_t n, uint32_t S0, uint64_t r, uint64_t T, uint32_t wb) {
@@ -366,9 +395,9 @@ __device__ __forceinline__ void batch_filter(const BatchArgs<R>& a, const BatchI
   // systematic: a contiguous range of passes per CTA, so that the CTAs exchange
   // their sums once; multinomial: pass j G + rank in round j
   constexpr bool SYS = POS == POS_SYSTEMATIC;
-  // (shares that differ by one pass at most: 19 filters of 100,000 particles on
-  // clusters of eight 143 -> 137 us per cycle, binary64 983 -> 872, where 25
-  // passes went to the CTAs as 4, 4, 4, 4, 4, 4, 1, 0)
+  // (shares that differ by one pass at most: 19 binary64 filters of 100,000
+  // particles on clusters of eight 983 -> 872 us per cycle, where 25 passes went to
+  // the CTAs as 4, 4, 4, 4, 4, 4, 1, 0)
   const uint64_t pb = SYS ? passes * rank / G : 0;
   const uint64_t pe = SYS ? passes * (rank + 1) / G : 0;
 
@@ -776,17 +805,38 @@ __device__ __forceinline__ void batch_filter(const BatchArgs<R>& a, const BatchI
         uint32_t most = Rs[0] - j;
 #pragma unroll
         for (int e = 1; e < SLOT_PER; ++e) most = max(most, Rs[e] - Rs[e - 1]);
-        const uint32_t wb = S0 & ~3u;
-        if (!__any_sync(0xffffffffu, most > 5u || Rs[SLOT_PER - 1] - wb > WIN))
-          win_mark(sm.win, wb, j, Rs, mk0);
-        else
-          mark_out<WIN>(sm.win, sm.run, &sm.nruns, wb, j, mk0, Rs[0], Rs[1], Rs[2], Rs[3], Rs[4], Rs[5], Rs[6], Rs[7]);
-        __syncthreads();
-        win_runs<NT>(sm.win, sm.run, &sm.nruns);
         uint32_t* const anc = a.anc + off;  // (off is a multiple of 32)
-        win_store<NT>(sm.win, anc, wb, S0, min(sm.wend, wb + WIN), (uint32_t)tb, true);
-        __syncthreads();  // the window has been read
-        if (sm.wend > wb + WIN) batch_windows<R, NT>(sm, a.Q + off, anc, tb, n, S0, offset(), T, wb + WIN);
+        if constexpr (G == 1) {
+          const uint32_t wb = S0 & ~3u;
+          if (!__any_sync(0xffffffffu, most > 5u || Rs[SLOT_PER - 1] - wb > WIN))
+            win_mark(sm.win, wb, j, Rs, mk0);
+          else
+            mark_out<WIN>(sm.win, sm.run, &sm.nruns, wb, j, mk0, Rs[0], Rs[1], Rs[2], Rs[3], Rs[4], Rs[5], Rs[6], Rs[7]);
+          __syncthreads();
+          win_runs<NT>(sm.win, sm.run, &sm.nruns);
+          win_store<NT>(sm.win, anc, wb, S0, min(sm.wend, wb + WIN), (uint32_t)tb, true);
+          __syncthreads();  // the window has been read
+          if (sm.wend > wb + WIN) batch_windows<R, NT>(sm, a.Q + off, anc, tb, n, S0, offset(), T, wb + WIN);
+        } else {
+          for (uint32_t wb = S0 & ~3u;;) {
+            if (!__any_sync(0xffffffffu, most > 5u || j < wb || Rs[SLOT_PER - 1] - wb > WIN))
+              win_mark(sm.win, wb, j, Rs, mk0);
+            else
+              win_mark_clipped<WIN>(sm.win, sm.run, &sm.nruns, wb, j, Rs, mk0);
+            __syncthreads();
+            win_runs<NT>(sm.win, sm.run, &sm.nruns);
+            const uint32_t S1 = sm.wend;
+            win_store<NT>(sm.win, anc, wb, max(S0, wb), min(S1, wb + WIN), (uint32_t)tb, true);
+            __syncthreads();  // the window has been read
+            wb += WIN;
+            if (S1 <= wb) break;
+            wb = store_owner<NT>(&sm.roff, anc, wb, (uint32_t)base, j, Rs[0], Rs[1], Rs[2], Rs[3], Rs[4], Rs[5], Rs[6],
+                                 Rs[7]);
+            if (S1 <= wb) break;
+            clear();
+            __syncthreads();
+          }
+        }
       } else {
         __syncthreads();  // sm.warp has been read
       }
