@@ -288,14 +288,13 @@ pf_status launch_resample(int scheme, const MultiArgs& ma, const uint32_t* I, cu
     k_multi<true><<<ma.ntiles, BLOCK, 0, s>>>(ma);
     mark(tm, "cutpoint_method", s);
   } else {
-    MultiArgs mb = ma;
     if (ma.ntiles <= MULTI_OWN) {
-      mb.splits = nullptr;
+      k_multi<false, true><<<ma.ntiles, BLOCK, 0, s>>>(ma);
     } else {
       k_multi_split<<<(unsigned)cdiv(ma.ntiles + 1, WARPS), BLOCK, 0, s>>>(ma);
       mark(tm, "split", s);
+      k_multi<false><<<ma.ntiles, BLOCK, 0, s>>>(ma);
     }
-    k_multi<false><<<ma.ntiles, BLOCK, 0, s>>>(mb);
     mark(tm, "merge", s);
   }
   CK(cudaGetLastError());

@@ -191,11 +191,12 @@ static __device__ __noinline__ uint32_t multi_exact(const uint64_t* Q, uint64_t 
 // 4, so an ancestor whose next CDF value is within that of P takes the exact
 // comparison.  CUT: the paper's Section 3.2 method instead -- start at the
 // cut-point table's entry of the slot's bucket and climb.
-template <bool CUT>
+// OWN: the CTA's first two warps search for its splits (MULTI_OWN).
+template <bool CUT, bool OWN = false>
 __global__ void __launch_bounds__(BLOCK, 4) k_multi(MultiArgs a) {
   __shared__ uint64_t s_q[CUT ? 1 : MULTI_CAP + 1];
   __shared__ uint64_t s_warp[WARPS];
-  __shared__ uint32_t s_split[CUT ? 1 : 2];
+  __shared__ uint32_t s_split[OWN ? 2 : 1];
   if (a.gate && *a.gate == 0u) return;
   const Ctl* const c = a.ctl;
   const uint64_t n = a.n, T = c->keyT;
@@ -218,7 +219,7 @@ __global__ void __launch_bounds__(BLOCK, 4) k_multi(MultiArgs a) {
     if (threadIdx.x == 0) s_q[staged ? i1 - i0 : 0] = ~0ull;
   };
   if constexpr (!CUT) {
-    if (a.splits) {
+    if constexpr (!OWN) {
       i0 = a.splits[blockIdx.x];
       i1 = a.splits[blockIdx.x + 1];
       stage();
@@ -232,13 +233,11 @@ __global__ void __launch_bounds__(BLOCK, 4) k_multi(MultiArgs a) {
   const uint64_t incl = warp_incl_scan(run[MULTI_PER - 1], lane);
   if (lane == 31) s_warp[warp] = incl;
   __syncthreads();
-  if constexpr (!CUT) {
-    if (!a.splits) {
-      i0 = s_split[0];
-      i1 = s_split[1];
-      stage();
-      __syncthreads();
-    }
+  if constexpr (OWN) {
+    i0 = s_split[0];
+    i1 = s_split[1];
+    stage();
+    __syncthreads();
   }
   uint64_t off = (lane & 7) < warp ? s_warp[lane & 7] : 0;
 #pragma unroll
